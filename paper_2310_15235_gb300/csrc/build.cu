@@ -351,7 +351,8 @@ __global__ void k_gather_elements(const double* __restrict__ pos, const float* _
                                   double size, float h_default, int* __restrict__ inv,
                                   double* __restrict__ pos64, float4* __restrict__ pos32,
                                   float* __restrict__ Lelem, float* __restrict__ km,
-                                  float* __restrict__ hn, float* __restrict__ ms) {
+                                  float* __restrict__ hn, float* __restrict__ ms,
+                                  int* __restrict__ luminous) {
   int64_t s = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (s >= N) return;
   int i = perm[s];
@@ -374,6 +375,8 @@ __global__ void k_gather_elements(const double* __restrict__ pos, const float* _
   float hh = h ? h[i] : h_default;
   hn[s] = float(double(hh) / size);
   ms[s] = mass[i];
+  const unsigned lit = __ballot_sync(__activemask(), lt > 0.0);
+  if (lt > 0.0 && (lit & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(luminous, __popc(lit));
 }
 
 // ---------------------------------------------------------------------------
@@ -459,7 +462,7 @@ __global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, doubl
                                   uint32_t* __restrict__ flags64, float* __restrict__ Lnode,
                                   float4* __restrict__ csrc, double* __restrict__ c64,
                                   double* __restrict__ B64, float* __restrict__ alpha_leaf,
-                                  NodeW* __restrict__ nodes) {
+                                  uint32_t* __restrict__ lmask, NodeW* __restrict__ nodes) {
   int64_t q = lb + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (q >= le) return;
   const int d = depth[q];
@@ -467,7 +470,7 @@ __global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, doubl
   node_box_norm(prefix[q], d, lo, ext);
   const int c = child[q];
   double cs[4] = {0, 0, 0, 0};
-  uint32_t has = 0;
+  uint32_t has = 0, lit = 0;
   if (c < 0) {
     const int f = first[q], n = count[q];
     double Lb[4] = {0, 0, 0, 0}, kmb[4] = {0, 0, 0, 0};
@@ -483,6 +486,7 @@ __global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, doubl
       }
       for (int a = 0; a < 3; ++a) cs[a] = __dadd_rn(cs[a], __dmul_rn(lt, pos64[3 * int64_t(e) + a]));
       cs[3] = __dadd_rn(cs[3], lt);
+      if (lt > 0.0 && e - f < 32) lit |= 1u << (e - f);
     }
     const double V = ext[0] * ext[1] * ext[2];  // exact powers of two
     for (int b = 0; b < nbp; ++b) {
@@ -502,6 +506,7 @@ __global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, doubl
   for (int a = 0; a < 3; ++a) cc[a] = cs[3] > 0.0 ? cs[a] / cs[3] : lo[a] + 0.5 * ext[a];
   if (cs[3] > 0.0) has |= kMetaHasL;
   flags64[q] = has;
+  lmask[q] = lit;
   // B: farthest box corner from the centre of luminosity (Sec. 2.5.2)
   double B2 = 0.0;
   for (int corner = 0; corner < 8; ++corner) {
@@ -595,6 +600,7 @@ static void free_tree(Tree* t, cudaStream_t st) {
   dfree(t->c64, st);
   dfree(t->B64, st);
   dfree(t->alpha_leaf, st);
+  dfree(t->lmask, st);
   dfree(t->dtau, st);
   dfree(t->nodes_refined, st);
   for (Table& tb : t->tables) {
@@ -602,6 +608,7 @@ static void free_tree(Tree* t, cudaStream_t st) {
     dfree(tb.dirs, st);
     dfree(tb.dirs64, st);
     dfree(tb.geo, st);
+    dfree(tb.beam_inv, st);
     dfree(tb.csm_tau, st);
     dfree(tb.csm_d, st);
     dfree(tb.csm_anti, st);
@@ -696,6 +703,10 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
     for (float m : hm) ngas += m > 0.0f;
     h_default = float(std::cbrt(t->size * t->size * t->size / double(std::max<int64_t>(ngas, 1))));
   }
+  DeviceTemp<int> dtotal_t(st);  // a scan's total, the number of luminous elements
+  int*& dtotal = dtotal_t.p;
+  T2_CHECK(dalloc(&dtotal, 2, st));
+  T2_CUDA(cudaMemsetAsync(dtotal, 0, 2 * sizeof(int), st));
   T2_CHECK(dalloc(&t->inv, N, st));
   T2_CHECK(dalloc(&t->pos64, 3 * N, st));
   T2_CHECK(dalloc(&t->pos32, N, st));
@@ -706,22 +717,21 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
   if (N > 0)
     k_gather_elements<<<blocks_for(N, 256), 256, 0, st>>>(
         pos, mass, kappa, lum, h, t->perm, N, nb, nbp, t->lo[0], t->lo[1], t->lo[2], t->size,
-        h_default, t->inv, t->pos64, t->pos32, t->Lelem, t->km, t->hn, t->mass); note_launch();
+        h_default, t->inv, t->pos64, t->pos32, t->Lelem, t->km, t->hn, t->mass, dtotal + 1);
+  note_launch();
 
   // 4. bisection, one depth at a time
   int64_t cap = 0;
   T2_CHECK(grow(t, std::max<int64_t>(1024, 4 * (N / std::max(t->bucket, 1)) + 64), cap, st));
   k_init_root<<<1, 1, 0, st>>>(N, t->prefix, t->depth, t->first, t->count, t->child, t->parent); note_launch();
-  DeviceTemp<int> flag_t(st), fscan_t(st), mid_t(st), dtotal_t(st);
+  DeviceTemp<int> flag_t(st), fscan_t(st), mid_t(st);
   int*& flag = flag_t.p;
   int*& fscan = fscan_t.p;
   int*& mid = mid_t.p;
-  int*& dtotal = dtotal_t.p;
   int64_t flag_cap = 1024;
   T2_CHECK(dalloc(&flag, flag_cap, st));
   T2_CHECK(dalloc(&fscan, flag_cap, st));
   T2_CHECK(dalloc(&mid, flag_cap, st));
-  T2_CHECK(dalloc(&dtotal, 1, st));
   t->level_begin.assign(1, 0);
   int64_t lb = 0, le = 1;
   int level = 0;
@@ -768,8 +778,8 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
   T2_CHECK(dalloc(&t->int_index, n, st));
   k_leaf_flags<<<blocks_for(n, 256), 256, 0, st>>>(t->child, n, t->int_index); note_launch();
   T2_CHECK(scan_exclusive_i32(t->int_index, n, dtotal, st));
-  int nint = 0;
-  T2_CUDA(cudaMemcpyAsync(&nint, dtotal, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int totals[2] = {0, 0};  // internal nodes, luminous elements
+  T2_CUDA(cudaMemcpyAsync(totals, dtotal, sizeof(totals), cudaMemcpyDeviceToHost, st));
   k_finish_int_index<<<blocks_for(n, 256), 256, 0, st>>>(t->child, n, t->int_index); note_launch();
   dfree(dtotal, st);
 
@@ -780,6 +790,7 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
   T2_CHECK(dalloc(&t->c64, 3 * n, st));
   T2_CHECK(dalloc(&t->B64, n, st));
   T2_CHECK(dalloc(&t->alpha_leaf, n * nbp, st));
+  T2_CHECK(dalloc(&t->lmask, n, st));
   DeviceTemp<double> L64_t(st), cs64_t(st);
   DeviceTemp<uint32_t> fl_t(st);
   double*& L64 = L64_t.p;
@@ -794,14 +805,15 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
     k_aggregate_level<<<blocks_for(b - a, 128), 128, 0, st>>>(
         a, b, nb, nbp, inv_size2, t->prefix, t->depth, t->first, t->count, t->child,
         t->int_index, t->pos64, t->Lelem, t->perm, kappa, mass, L64, cs64, fl, t->Lnode, t->csrc, t->c64,
-        t->B64, t->alpha_leaf, t->nodes); note_launch();
+        t->B64, t->alpha_leaf, t->lmask, t->nodes); note_launch();
   }
   dfree(L64, st);
   dfree(cs64, st);
   dfree(fl, st);
   T2_CUDA(cudaGetLastError());
   T2_CUDA(cudaStreamSynchronize(st));
-  t->n_internal = nint;
+  t->n_internal = totals[0];
+  t->n_luminous = totals[1];
   return TREVR2_OK;
 }
 

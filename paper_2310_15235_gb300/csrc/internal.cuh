@@ -70,6 +70,13 @@ struct Table {
   float4* dirs = nullptr;      // [npix] beam directions (xyz), w = pair index (int bits)
   double* dirs64 = nullptr;    // [npix][3]
   TransGeo* geo = nullptr;     // [3][P]
+  // beams by direction for the cell-by-cell absorption (nside <= kCellNside),
+  // built on first use: for every cell shape and square of a cube map of
+  // directions, all beams in the order of the size from which on a cell there
+  // can be crossed by them, and how many there are for each class of sizes
+  float4* beam_inv = nullptr;     // [npix, by beam_slot] 1 / direction, w = pair (owns all three)
+  uint8_t* beam_list = nullptr;   // [3][6 nf^2][npix rounded up to 16], nf = beam_map_side(nside)
+  uint8_t* beam_count = nullptr;  // [3][6 nf^2][kConeClasses + 1]
   // complex source model (Sec. 2.7), built on first use with TREVR2_CSM
   float* csm_tau = nullptr;    // [n][npix][nbp] optical depth of each luminous cell's ray
   float* csm_d = nullptr;      // [n][npix] its length (normalised)
@@ -87,6 +94,7 @@ struct Tree {
   int64_t n_nodes = 0;
   int64_t n_internal = 0;
   int max_depth = 0;
+  int64_t n_luminous = 0;  // elements with some luminosity
   bool has_h = false;
   cudaStream_t last_stream = nullptr;
 
@@ -115,6 +123,7 @@ struct Tree {
   double* c64 = nullptr;      // [n][3] normalised centre of luminosity
   double* B64 = nullptr;      // [n] normalised B
   float* alpha_leaf = nullptr;// [n][nbp] normalised bucket absorption (0 internal)
+  uint32_t* lmask = nullptr;  // [n] leaves: which of their first 32 elements are luminous
   // refinement tau_refine (Sec. 2.5.2): node records with B raised where the
   // optical depth varies by more than tau_refine inside the cell
   float* dtau = nullptr;          // [n] optical-depth variation of each cell
@@ -202,6 +211,24 @@ int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, in
 // cached): Eq. transmissionavg, or with `linear` the volume-weighted linear
 // average of the halves (Sec. 2.6's comparison scheme).
 int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear = false);
+
+// The finest beams whose absorption is summed cell by cell (their indices fit
+// one byte: 192 beams at nside 4); finer ones are walked beam by beam.
+constexpr int kCellNside = 4;
+constexpr int kConeClasses = 32;
+// 1 / n of a beam with a zero component: large enough to put any face not
+// exactly at the origin beyond the root cube, small enough to stay finite.
+constexpr float kFlatInv = 1e30f;
+// Where the cell-by-cell walk keeps beam k in its tables (its own inverse): a
+// look-up's beams are neighbours, k +- 1 in their ring or about 16 apart in the
+// next at nside 4, and these fall into different 16-byte banks.
+__host__ __device__ inline int beam_slot(int k) { return k ^ ((k >> 4) & 3); }
+// Squares per cube face and axis: a square's half-diagonal is 0.18 / nside
+// rad, a fifth of the spacing of the beams.
+__host__ __device__ inline int beam_map_side(int nside) { return 8 * nside; }
+
+// The beam look-up tables of one table's nside (built and cached).
+int ensure_beam_map(Table* tb, cudaStream_t st);
 
 inline int nbp_of(int nb) { return nb <= 1 ? 1 : (nb == 2 ? 2 : 4); }
 

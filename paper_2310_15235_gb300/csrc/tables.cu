@@ -74,6 +74,103 @@ __global__ void k_trans_geo(int P, const double* __restrict__ dirs64, TransGeo* 
   geo[idx] = g;
 }
 
+// The unit vector through point (a, b) of face f of the cube [-1, 1]^3:
+// f / 2 is the face's axis, odd f its negative side, (a, b) the other two
+// axes in increasing order.
+__device__ __forceinline__ void cube_vec(int f, float a, float b, float v[3]) {
+  const int m = f >> 1;
+  const float r = 1.0f / sqrtf(1.0f + a * a + b * b), s = (f & 1) ? -r : r;
+  v[0] = m == 0 ? s : a * r;
+  v[1] = m == 1 ? s : (m == 0 ? a * r : b * r);
+  v[2] = m == 2 ? s : b * r;
+}
+
+// One cell shape (depth mod 3) and one square of the direction map per warp.
+// A cell whose centre lies in the square, with half-diagonal over distance at
+// most rho, is held by the box about the square's own direction with the
+// shape's half-extents at rho, each widened by the square's range on that axis
+// (1e-4 covers the FP32 arithmetic here and in the walk): the beams that cross
+// that box are the cell's candidates.  They only grow with rho, so a beam's
+// place is the first class (rho up to sin of the cone half-angle acos(1 -
+// (c / kConeClasses)^2)) that has it, and a class's candidates are the first
+// ones of the list.
+__global__ void k_beam_map(int npix, int stride, int nf, const float4* __restrict__ dirs,
+                           uint8_t* __restrict__ list, uint8_t* __restrict__ count,
+                           float4* __restrict__ beam_inv) {
+  if (blockIdx.x == 0 && threadIdx.x < npix) {
+    const float4 n = dirs[threadIdx.x];
+    beam_inv[beam_slot(threadIdx.x)] =
+        make_float4(n.x != 0.0f ? 1.0f / n.x : kFlatInv, n.y != 0.0f ? 1.0f / n.y : kFlatInv,
+                    n.z != 0.0f ? 1.0f / n.z : kFlatInv, n.w);
+  }
+  const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (id >= 18 * nf * nf) return;
+  const int shape = id / (6 * nf * nf), sq = id % (6 * nf * nf);
+  const int f = sq / (nf * nf), i = (sq / nf) % nf, j = sq % nf;
+  const float w = 2.0f / nf;
+  float c[3], half[3], wide[3];
+  cube_vec(f, -1.0f + (i + 0.5f) * w, -1.0f + (j + 0.5f) * w, c);
+  const float norm = rsqrtf((shape >= 1 ? 0.25f : 1.0f) + (shape >= 2 ? 0.25f : 1.0f) + 1.0f);
+  half[0] = shape >= 1 ? 0.5f * norm : norm;
+  half[1] = shape >= 2 ? 0.5f * norm : norm;
+  half[2] = norm;
+  for (int a = 0; a < 3; ++a) wide[a] = 1e-4f;
+  for (int q = 0; q < 4; ++q) {  // no square straddles an axis: the corners are extreme
+    float v[3];
+    cube_vec(f, -1.0f + (i + (q & 1)) * w, -1.0f + (j + (q >> 1)) * w, v);
+    for (int a = 0; a < 3; ++a) wide[a] = fmaxf(wide[a], fabsf(v[a] - c[a]) + 1e-4f);
+  }
+  constexpr int kGroups = (12 * kCellNside * kCellNside + 31) / 32;
+  int first[kGroups];
+#pragma unroll
+  for (int g = 0; g < kGroups; ++g) {
+    const int k = 32 * g + lane;
+    first[g] = kConeClasses + 2;  // no beam
+    if (k >= npix) continue;
+    const float4 n4 = dirs[k];
+    const float n[3] = {n4.x, n4.y, n4.z};
+    // crossing times of the widened box: (c -+ (rho half + wide)) / n
+    float mid[3], grow[3], base[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float inv = n[a] != 0.0f ? 1.0f / n[a] : kFlatInv;
+      mid[a] = c[a] * inv;
+      grow[a] = half[a] * fabsf(inv);
+      base[a] = wide[a] * fabsf(inv);
+    }
+    int lo = 1, hi = kConeClasses + 1;  // hi: only as one of all beams
+    while (lo < hi) {
+      const int m = (lo + hi) >> 1;
+      const float u = float(m) / float(kConeClasses), cr = 1.0f - u * u;
+      const float rho = sqrtf(fmaxf(0.0f, 1.0f - cr * cr));
+      float t0 = 0.0f, t1 = INFINITY;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float e = fmaf(rho, grow[a], base[a]);
+        t0 = fmaxf(t0, mid[a] - e);
+        t1 = fminf(t1, mid[a] + e);
+      }
+      if (t0 <= t1) hi = m; else lo = m + 1;
+    }
+    first[g] = lo;
+  }
+  uint8_t* out = list + size_t(id) * stride;
+  uint8_t* cnt = count + size_t(id) * (kConeClasses + 1);
+  if (lane == 0) cnt[0] = 0;
+  int base = 0;
+  for (int cls = 1; cls <= kConeClasses + 1; ++cls) {
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) {
+      const unsigned m = __ballot_sync(0xffffffffu, first[g] == cls);
+      if (first[g] == cls)
+        out[base + __popc(m & ((1u << lane) - 1u))] = uint8_t(beam_slot(32 * g + lane));
+      base += __popc(m);
+    }
+    if (lane == 0 && cls <= kConeClasses) cnt[cls] = uint8_t(base);
+  }
+  for (int k = npix + lane; k < stride; k += 32) out[k] = 0;
+}
+
 __device__ __forceinline__ float combine_alpha(float a1, float a2, float w1, float w12, float d) {
   const float x1 = d * a1, x2 = d * a2, x12 = 0.5f * (x1 + x2);
   float m = INFINITY;
@@ -132,6 +229,27 @@ __global__ void k_alpha_level(int64_t lb, int64_t le, int P, int nb, bool linear
       al = linear ? 0.5f * (a1[b] + a2[b]) : combine_alpha(a1[b], a2[b], g.w1, g.w12, d);
     tab[(int64_t(iq) * P + p) * NBP + b] = al;
   }
+}
+
+int ensure_beam_map(Table* tb, cudaStream_t st) {
+  if (tb->beam_list) return TREVR2_OK;
+  const int npix = 12 * tb->nside * tb->nside, stride = (npix + 15) & ~15;
+  const int nf = beam_map_side(tb->nside);
+  const size_t squares = size_t(18) * nf * nf, inv_bytes = size_t(npix) * sizeof(float4);
+  DeviceTemp<uint8_t> map(st);  // inverses, lists, counts
+  T2_CHECK(device_alloc(reinterpret_cast<void**>(&map.p),
+                        inv_bytes + squares * (stride + kConeClasses + 1), st, "beam map"));
+  uint8_t* list = map.p + inv_bytes;
+  uint8_t* count = list + squares * stride;
+  k_beam_map<<<unsigned((squares + 7) / 8), 256, 0, st>>>(npix, stride, nf, tb->dirs, list, count,
+                                                          reinterpret_cast<float4*>(map.p));
+  note_launch();
+  T2_CUDA(cudaGetLastError());
+  tb->beam_inv = reinterpret_cast<float4*>(map.p);
+  tb->beam_list = list;
+  tb->beam_count = count;
+  map.p = nullptr;
+  return TREVR2_OK;
 }
 
 int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear) {

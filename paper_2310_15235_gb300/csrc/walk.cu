@@ -27,11 +27,13 @@
 // capacity of one warp's buffers are handled in further passes.
 #include <cfloat>
 #include <cmath>
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <string>
 #include <vector>
 
+#include "cells.cuh"
 #include "walk.cuh"
 
 namespace trevr2 {
@@ -47,26 +49,8 @@ __device__ __forceinline__ void add_csm(const WalkArgs& a, int ref, int k, BandV
   for (int b = 0; b < NBP; ++b) tk.v[b] += c.v[b];
 }
 
-// Box extents for phase A's stack pops, the same values as node_ext: the
-// longest side 2^-floor(depth / 3) by depth in shared memory (256 bytes, so
-// that the walk kernels keep their blocks per SM), the others halved on the
-// axes already split at this depth.  x, y, z, and w = the split axis's extent
-// (z's).  Every kernel that runs phase A fills the table before its first
-// receiver.
-__shared__ float g_ext_e[64];
-
-__device__ __forceinline__ void init_ext_tab() {
-  if (threadIdx.x < 64) g_ext_e[threadIdx.x] = __int_as_float((127 - int(threadIdx.x) / 3) << 23);
-  __syncthreads();
-}
-
-__device__ __forceinline__ float4 ext_of(uint32_t meta) {
-  const float e = g_ext_e[meta & kMetaDepthMask];
-  const uint32_t r = (meta >> kMetaAxisShift) & 3u;
-  return make_float4(r > 0u ? 0.5f * e : e, r > 1u ? 0.5f * e : e, e, e);
-}
-
-// Phase A: lanes take beams from the order above through a per-warp counter.
+// Phase A beam by beam (beams finer than kCellNside, and directed beams, whose
+// directions no table holds): lanes take beams from the order above through a per-warp counter.
 // Each beam first descends the receiver's ancestors (chain[0..], root to the
 // receiver's leaf, in shared memory): they hold the receiver, so they open,
 // and each one's chord is its parent's near-half interval; only their
@@ -225,38 +209,142 @@ __device__ __forceinline__ void eval_sources(const WalkArgs& a, int lane, const 
   }
 }
 
+// A warp's part of a walk block's shared memory and of the walk buffers.
+struct WarpMem {
+  int* stk;          // traversal stacks / increments, boxes and crossings
+  int* lstk;         // this lane's stack (beam by beam)
+  int* off;          // [npix] ends of the beams' buckets, then scratch
+  int* order;        // [npix] beams by distance (beam by beam)
+  int* next_beam;
+  NodeW* chain;      // the receiver's ancestors (beam by beam)
+  float* far;        // [npix] the beams' farthest sources (cell by cell)
+  const float4* binv;  // [npix] the block's copy of 1 / direction (cell by cell)
+  SrcEntry* U;
+  int* Up;
+  SrcEntry* V;
+  float* T;
+  float* own;        // [M][4] depth inside the cell that holds a source (cell by cell)
+  int* cells;
+};
+
+template <bool kCells>
+__device__ __forceinline__ WarpMem warp_mem(const WalkArgs& a, int* smem, int64_t gw,
+                                            SrcEntry* srcU, int* pixU, SrcEntry* srcV, float* srcT,
+                                            int* cells) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  WarpMem w;
+  w.binv = reinterpret_cast<const float4*>(smem);
+  int* wsm = smem + (kCells ? 4 * a.npix : 0) + wib * a.warp_ints;
+  w.stk = wsm;
+  w.lstk = wsm + lane * 2 * (a.max_depth + 2);
+  w.off = wsm + a.region_ints;
+  w.order = w.off + a.npix;
+  w.far = reinterpret_cast<float*>(w.off + a.npix);
+  w.next_beam = w.off + 2 * a.npix + 32;  // after the beam order and its counts
+  w.chain = reinterpret_cast<NodeW*>(w.off + 2 * a.npix + 36);
+  w.U = srcU + gw * a.M;
+  w.Up = pixU + gw * a.M;
+  w.V = srcV + gw * a.M;
+  w.T = srcT + gw * a.M * 4;
+  w.cells = cells + gw * (a.cell_cap + 4 * a.M);
+  w.own = reinterpret_cast<float*>(w.cells + a.cell_cap);
+  return w;
+}
+
+// Fills a walk block's shared tables.
+template <bool kCells>
+__device__ __forceinline__ void init_block(const WalkArgs& a, int* smem) {
+  if constexpr (kCells) {
+    float4* binv = reinterpret_cast<float4*>(smem);
+    for (int k = threadIdx.x; k < a.npix; k += blockDim.x) binv[k] = a.beam_inv[k];
+  }
+  init_ext_tab();
+}
+
+// tau of every source of one origin (n staged sources V binned by beam) into
+// w.T, from all its cells or (cell by cell) from the window of `listed` cells
+// that starts at clo: set for the first window, added for the later ones.
+template <int NBP, bool kBucket, bool kPP, bool kCSM, bool kCells>
+__device__ __forceinline__ void absorb(const WalkArgs& a, float3 x, int si, int lane, const WarpMem& w,
+                                       int n, int listed, int clo, int leaf, float rpp) {
+  if constexpr (kCells) {
+    absorb_cells<NBP, kPP>(a, x, lane, w.stk, w.binv, w.off, w.far, w.V, w.T, w.own, n, w.cells,
+                           min(listed - clo, a.cell_cap), clo == 0, rpp);
+    if (clo + a.cell_cap >= listed) {
+      sum_increments<NBP>(lane, a.npix, w.off, w.T, w.own);
+      if constexpr (kCSM)
+        for (int k = lane; k < a.npix; k += 32)
+          for (int e = k ? w.off[k - 1] : 0; e < w.off[k]; ++e) {
+            BandVec<NBP> t = load_bands<NBP>(w.T + int64_t(e) * NBP);
+            add_csm<NBP>(a, w.V[e].ref, k, t);
+            store_bands<NBP>(w.T + int64_t(e) * NBP, t);
+          }
+    }
+  } else {
+    const int nbeams = order_beams(a, lane, w.V, w.off, w.order, w.order + a.npix);
+    if (lane == 0) *w.next_beam = 32;
+    __syncwarp();
+    phase_absorb<NBP, kBucket, kPP, kCSM>(a, x, si, lane, w.lstk, w.V, w.T, w.off, w.order, nbeams,
+                                          w.next_beam, w.chain, leaf, rpp);
+  }
+  __syncwarp();
+}
+
+// The sources of one origin in passes of M, each pass's absorbing cells in
+// windows of cell_cap (one pass and one window unless a cut holds more):
+// stages a pass's sources, sums their tau over the windows, and hands the
+// pass to eval(n).
+template <int NBP, bool kBucket, bool kPP, bool kCSM, bool kCells, class Eval>
+__device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si, int lane,
+                                            const WarpMem& w, int leaf, float rpp, Eval eval) {
+  int n = 0;
+  for (int lo = 0, clo = 0;;) {
+    int total, listed = 0;
+    if constexpr (kCells) {
+      // a later window only lists cells: no source has an index that high
+      const int2 c = phase_cut<kBucket, kPP>(a, x, si, lane, w.stk, a.src_stack_cap, w.U,
+                                             clo ? INT32_MAX : lo, w.cells, clo, rpp);
+      total = c.x;
+      listed = c.y;
+    } else {
+      total = phase_sources<kBucket, kPP>(a, x, si, lane, w.stk, a.src_stack_cap, w.U, w.Up, lo, rpp);
+    }
+    if (clo == 0) {
+      const int staged = min(total - lo, a.M);
+      make_sources<kBucket, kCSM>(a, x, si, lane, w.U, w.Up, staged);
+      n = staged > 0 ? bin_sources(a, lane, w.U, w.Up, staged, w.V, w.off) : 0;
+    }
+    if (n > 0) {
+      absorb<NBP, kBucket, kPP, kCSM, kCells>(a, x, si, lane, w, n, listed, clo, leaf, rpp);
+      if (kCells && clo + a.cell_cap < listed) {
+        clo += a.cell_cap;
+        continue;
+      }
+      eval(n);
+      __syncwarp();
+    }
+    clo = 0;
+    lo += a.M;
+    if (lo >= total) break;
+  }
+}
+
 // J of one receiver (caller index io of the tree described by a) into
 // Jrow[0, nbsel); the warp's shared stacks and buffers are passed in.
-template <int NBP>
+template <int NBP, bool kCells>
 __device__ __forceinline__ void walk_receiver_si(const WalkArgs& a, int si, float* Jrow, int lane,
-                                                 int* stk, int* off, int* next_beam, int* lstk,
-                                                 SrcEntry* U, int* Up, SrcEntry* V, float* T) {
+                                                 const WarpMem& w) {
   const float4 xr = a.pos32[si];
   // the receiver in FP32, on the FP64 side of every box face
   const float3 x = grazing_coords(a, si, make_float3(xr.x, xr.y, xr.z));
   // the receiver's ancestors, root first
-  NodeW* chain = reinterpret_cast<NodeW*>(off + 2 * a.npix + 36);
-  const int leaf = build_chain(a.nodes, x, lane, chain);
+  const int leaf = kCells ? 0 : build_chain(a.nodes, x, lane, w.chain);
   float Js[NBP], Jc[NBP];
 #pragma unroll
   for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
-  for (int lo = 0;; lo += a.M) {
-    const int total = phase_sources(a, x, si, lane, stk, a.src_stack_cap, U, Up, lo);
-    const int staged = min(total - lo, a.M);
-    make_sources(a, x, si, lane, U, Up, staged);
-    const int n = staged > 0 ? bin_sources(a, lane, U, Up, staged, V, off) : 0;
-    if (n > 0) {
-      int* order = off + a.npix;
-      const int nbeams = order_beams(a, lane, V, off, order, order + a.npix);
-      if (lane == 0) *next_beam = 32;
-      __syncwarp();
-      phase_absorb<NBP>(a, x, si, lane, lstk, V, T, off, order, nbeams, next_beam, chain, leaf);
-      __syncwarp();
-      eval_sources<NBP>(a, lane, V, T, n, Js, Jc);
-      __syncwarp();
-    }
-    if (lo + a.M >= total) break;
-  }
+  walk_origin<NBP, false, false, false, kCells>(a, x, si, lane, w, leaf, 0.0f, [&](int n) {
+    eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
+  });
   // FP64 reduction of the lane partial sums
   double Jd[NBP];
 #pragma unroll
@@ -285,42 +373,33 @@ __device__ __forceinline__ void walk_receiver_si(const WalkArgs& a, int si, floa
 
 // The same for the receiver with caller index io (NaN row and a status bit
 // for an index outside [0, N)).
-template <int NBP>
+template <int NBP, bool kCells>
 __device__ __forceinline__ void walk_receiver(const WalkArgs& a, int64_t io, float* Jrow, int lane,
-                                              int* stk, int* off, int* next_beam, int* lstk,
-                                              SrcEntry* U, int* Up, SrcEntry* V, float* T) {
+                                              const WarpMem& w) {
   if (io < 0 || io >= a.N) {
     if (lane == 0) atomicOr(a.status, kStatusBadActive);
     if (lane < a.nbsel) Jrow[lane] = __int_as_float(0x7fc00000);
     return;
   }
-  walk_receiver_si<NBP>(a, a.inv[io], Jrow, lane, stk, off, next_beam, lstk, U, Up, V, T);
+  walk_receiver_si<NBP, kCells>(a, a.inv[io], Jrow, lane, w);
 }
 
 // One warp per receiver, receivers from a global counter.
-template <int NBP, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, kWalkWarpsPerSM / WARPS) k_walk(WalkArgs a) {
-  init_ext_tab();
-  extern __shared__ int smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t gw = int64_t(blockIdx.x) * WARPS + wib;
-  int* wsm = smem + wib * (a.stack_ints + 2 * a.npix + 36 + 8 * (a.max_depth + 1));
-  int* stk = wsm;
-  int* off = wsm + a.stack_ints;
-  int* next_beam = off + 2 * a.npix + 32;  // after the beam order and its counts
-  int* lstk = stk + lane * 2 * (a.max_depth + 2);
-  SrcEntry* U = a.srcU + gw * a.M;
-  int* Up = a.pixU + gw * a.M;
-  SrcEntry* V = a.srcV + gw * a.M;
-  float* T = a.srcT + gw * a.M * 4;
+template <int NBP, int WARPS, bool kCells>
+__global__ void __launch_bounds__(WARPS * 32, (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
+    k_walk(WalkArgs a) {
+  extern __shared__ __align__(16) int smem[];
+  init_block<kCells>(a, smem);
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = int64_t(blockIdx.x) * WARPS + (threadIdx.x >> 5);
+  const WarpMem w = warp_mem<kCells>(a, smem, gw, a.srcU, a.pixU, a.srcV, a.srcT, a.cells);
   for (;;) {
     unsigned long long slot = 0;
     if (lane == 0) slot = atomicAdd(a.counter, 1ull);
     slot = __shfl_sync(0xffffffffu, slot, 0);
     if (slot >= (unsigned long long)a.A) break;
     const int64_t r = a.order ? int64_t(a.order[slot]) : int64_t(slot);
-    walk_receiver<NBP>(a, a.active[r], a.J + r * a.nbsel, lane, stk, off, next_beam,
-                       lstk, U, Up, V, T);
+    walk_receiver<NBP, kCells>(a, a.active[r], a.J + r * a.nbsel, lane, w);
   }
 }
 
@@ -834,10 +913,9 @@ __device__ __forceinline__ void eval_bucket_pp(const WalkArgs& a, bool soft, int
 // J of the receivers in slots [p0, p1), all in leaf q, into their rows
 // (kPP: with the p-p absorption of Sec. 2.4; kCSM: with the complex source
 // model of Sec. 2.7).
-template <int NBP, bool kPP, bool kCSM>
+template <int NBP, bool kPP, bool kCSM, bool kCells>
 __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0, int64_t p1,
-                            int q, int64_t gw, int lane, int* stk, int* off, int* next_beam,
-                            int* lstk, SrcEntry* U, int* Up, SrcEntry* V, float* T) {
+                            int q, int64_t gw, int lane, const WarpMem& w) {
   if (q < 0) {  // receivers outside [0, N): NaN rows and a status bit
     for (int64_t p = p0 + lane; p < p1; p += 32)
       for (int c = 0; c < a.nbsel; ++c) a.J[int64_t(a.order[p]) * a.nbsel + c] = __int_as_float(0x7fc00000);
@@ -868,8 +946,7 @@ __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0,
       }
     }
   }
-  NodeW* chain = reinterpret_cast<NodeW*>(off + 2 * a.npix + 36);
-  const int leaf = build_chain(a.nodes, o, lane, chain);  // == q
+  const int leaf = kCells ? q : build_chain(a.nodes, o, lane, w.chain);  // == q
   const bool soft = (bk.rflags & TREVR2_SOFT) != 0;
   // Sec. 2.4: the bucket's p-p radius and particles
   int npp = 0;
@@ -878,7 +955,7 @@ __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0,
     const double r0 = 0.5 * sqrt(double(e.x) * e.x + double(e.y) * e.y + double(e.z) * e.z);
     double r64 = 0.0;
     __syncwarp();
-    npp = collect_pp<NBP>(a, bk, a.origin64 + kOriginWords * gw, r0, lane, stk, gw, r64);
+    npp = collect_pp<NBP>(a, bk, a.origin64 + kOriginWords * gw, r0, lane, w.stk, gw, r64);
     if (lane == 0) a.origin64[kOriginWords * gw + 3] = r64;
     rpp = float(r64);
     __syncwarp();
@@ -902,32 +979,16 @@ __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0,
     double acc[NBP];
 #pragma unroll
     for (int b = 0; b < NBP; ++b) acc[b] = 0.0;
-    for (int lo = 0;; lo += a.M) {
-      const int total = phase_sources<true, kPP>(a, o, si_o, lane, stk, a.src_stack_cap, U, Up, lo,
-                                                 rpp);
-      const int staged = min(total - lo, a.M);
-      make_sources<true, kCSM>(a, o, si_o, lane, U, Up, staged);
-      const int n = staged > 0 ? bin_sources(a, lane, U, Up, staged, V, off) : 0;
-      if (n > 0) {
-        int* order = off + a.npix;
-        const int nbeams = order_beams(a, lane, V, off, order, order + a.npix);
-        if (lane == 0) *next_beam = 32;
-        __syncwarp();
-        phase_absorb<NBP, true, kPP, kCSM>(a, o, si_o, lane, lstk, V, T, off, order, nbeams,
-                                           next_beam, chain, leaf, rpp);
-        __syncwarp();
-        if constexpr (kPP) {
-          // Up, the staged records' beams, is free once they are binned
-          sort_sources_by_cell(a, lane, V, n, o, off, 2 * a.npix + 32, Up);
-          eval_bucket_pp<NBP>(a, soft, lane, V, T, Up, n, nrec, xr, hr, si, acc, npp, ppxh, ppkc,
-                              ppsi, ppw, ppu, ppmask);
-        } else {
-          eval_bucket<NBP>(a, soft, lane, V, T, n, nrec, xr, hr, si, acc);
-        }
-        __syncwarp();
+    walk_origin<NBP, true, kPP, kCSM, kCells>(a, o, si_o, lane, w, leaf, rpp, [&](int n) {
+      if constexpr (kPP) {
+        // Up, the staged records' beams, is free once they are binned
+        sort_sources_by_cell(a, lane, w.V, n, o, w.off, 2 * a.npix + 32, w.Up);
+        eval_bucket_pp<NBP>(a, soft, lane, w.V, w.T, w.Up, n, nrec, xr, hr, si, acc, npp, ppxh,
+                            ppkc, ppsi, ppw, ppu, ppmask);
+      } else {
+        eval_bucket<NBP>(a, soft, lane, w.V, w.T, n, nrec, xr, hr, si, acc);
       }
-      if (lo + a.M >= total) break;
-    }
+    });
     if (lane < nrec) {
       float* Jrow = a.J + int64_t(a.order[c0 + lane]) * a.nbsel;
       for (int c = 0; c < a.nbsel; ++c) {
@@ -954,22 +1015,14 @@ __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0,
 // registers a thread) measured faster than 7 (72, spilling) and than 4 or 6.
 constexpr int kPPBlocksPerSM = 5;
 
-template <int NBP, int WARPS, bool kPP, bool kCSM>
-__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : kWalkWarpsPerSM / WARPS)
+template <int NBP, int WARPS, bool kPP, bool kCSM, bool kCells>
+__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
     k_walk_bucket(WalkArgs a, const __grid_constant__ BucketArgs bk) {
-  init_ext_tab();
-  extern __shared__ int smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t gw = int64_t(blockIdx.x) * WARPS + wib;
-  int* wsm = smem + wib * (a.stack_ints + 2 * a.npix + 36 + 8 * (a.max_depth + 1));
-  int* stk = wsm;
-  int* off = wsm + a.stack_ints;
-  int* next_beam = off + 2 * a.npix + 32;
-  int* lstk = stk + lane * 2 * (a.max_depth + 2);
-  SrcEntry* U = a.srcU + gw * a.M;
-  int* Up = a.pixU + gw * a.M;
-  SrcEntry* V = a.srcV + gw * a.M;
-  float* T = a.srcT + gw * a.M * 4;
+  extern __shared__ __align__(16) int smem[];
+  init_block<kCells>(a, smem);
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = int64_t(blockIdx.x) * WARPS + (threadIdx.x >> 5);
+  const WarpMem w = warp_mem<kCells>(a, smem, gw, a.srcU, a.pixU, a.srcV, a.srcT, a.cells);
   for (;;) {
     unsigned long long slot = 0;
     if (lane == 0) slot = atomicAdd(a.counter, 1ull);
@@ -990,8 +1043,7 @@ __global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : kWalkWarpsP
       p1 += __ffs(~same) - 1;
       break;
     }
-    walk_bucket<NBP, kPP, kCSM>(a, bk, p0, p1, q, gw, lane, stk, off, next_beam, lstk, U, Up, V,
-                                T);
+    walk_bucket<NBP, kPP, kCSM, kCells>(a, bk, p0, p1, q, gw, lane, w);
   }
 }
 
@@ -1027,9 +1079,8 @@ struct BatchArgs {
   int* pixU;
   SrcEntry* srcV;
   float* srcT;
+  int* cells;
   int M;
-  int stack_ints;
-  int npix;
   int max_depth;
   unsigned long long* counter;
   // per-bucket plans (TREVR2_BUCKET): for each distinct key, its sorted
@@ -1055,6 +1106,7 @@ struct BatchSlice {
   int* pixU;
   SrcEntry* srcV;
   float* srcT;
+  int* cells;
   unsigned long long* counter;
 };
 
@@ -1132,22 +1184,14 @@ __global__ void k_batch_tree_range(const __grid_constant__ BatchArgs B) {
 // One launch per tree (its walk arguments are this launch's own parameter,
 // so the walk reads them as directly as k_walk does): one warp per distinct
 // key of the tree, keys from a global counter.
-template <int NBP, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, kWalkWarpsPerSM / WARPS)
+template <int NBP, int WARPS, bool kCells>
+__global__ void __launch_bounds__(WARPS * 32, (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
     k_walk_batched(WalkArgs a, const __grid_constant__ BatchSlice S) {
-  init_ext_tab();
-  extern __shared__ int smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t gw = int64_t(blockIdx.x) * WARPS + wib;
-  int* wsm = smem + wib * (a.stack_ints + 2 * a.npix + 36 + 8 * (a.max_depth + 1));
-  int* stk = wsm;
-  int* off = wsm + a.stack_ints;
-  int* next_beam = off + 2 * a.npix + 32;  // after the beam order and its counts
-  int* lstk = stk + lane * 2 * (a.max_depth + 2);
-  SrcEntry* U = S.srcU + gw * a.M;
-  int* Up = S.pixU + gw * a.M;
-  SrcEntry* V = S.srcV + gw * a.M;
-  float* T = S.srcT + gw * a.M * 4;
+  extern __shared__ __align__(16) int smem[];
+  init_block<kCells>(a, smem);
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = int64_t(blockIdx.x) * WARPS + (threadIdx.x >> 5);
+  const WarpMem w = warp_mem<kCells>(a, smem, gw, S.srcU, S.pixU, S.srcV, S.srcT, S.cells);
   const int64_t u0 = S.tree_range[S.t], u1 = S.tree_range[S.t + 1];
   const uint64_t mask = (uint64_t(1) << S.key_shift) - 1;
   for (;;) {
@@ -1156,8 +1200,7 @@ __global__ void __launch_bounds__(WARPS * 32, kWalkWarpsPerSM / WARPS)
     slot = __shfl_sync(0xffffffffu, slot, 0);
     const int64_t u = u0 + int64_t(slot);
     if (u >= u1) break;
-    walk_receiver_si<NBP>(a, int(S.ukeys[u] & mask), S.Ju + u * S.nbsel, lane, stk, off,
-                          next_beam, lstk, U, Up, V, T);
+    walk_receiver_si<NBP, kCells>(a, int(S.ukeys[u] & mask), S.Ju + u * S.nbsel, lane, w);
   }
 }
 
@@ -1189,23 +1232,15 @@ __global__ void k_batch_leaf(const __grid_constant__ BatchArgs B,
 // walk over many subsets and snapshots), one launch per tree as for
 // k_walk_batched; slots from a global counter, a bucket walked by the warp
 // that takes its first slot.
-template <int NBP, int WARPS, bool kPP, bool kCSM>
-__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : kWalkWarpsPerSM / WARPS)
+template <int NBP, int WARPS, bool kPP, bool kCSM, bool kCells>
+__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
     k_walk_bucket_batched(WalkArgs a, const __grid_constant__ BucketArgs bk,
                           const __grid_constant__ BatchSlice S) {
-  init_ext_tab();
-  extern __shared__ int smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t gw = int64_t(blockIdx.x) * WARPS + wib;
-  int* wsm = smem + wib * (a.stack_ints + 2 * a.npix + 36 + 8 * (a.max_depth + 1));
-  int* stk = wsm;
-  int* off = wsm + a.stack_ints;
-  int* next_beam = off + 2 * a.npix + 32;
-  int* lstk = stk + lane * 2 * (a.max_depth + 2);
-  SrcEntry* U = S.srcU + gw * a.M;
-  int* Up = S.pixU + gw * a.M;
-  SrcEntry* V = S.srcV + gw * a.M;
-  float* T = S.srcT + gw * a.M * 4;
+  extern __shared__ __align__(16) int smem[];
+  init_block<kCells>(a, smem);
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = int64_t(blockIdx.x) * WARPS + (threadIdx.x >> 5);
+  const WarpMem w = warp_mem<kCells>(a, smem, gw, S.srcU, S.pixU, S.srcV, S.srcT, S.cells);
   const int64_t u0 = S.tree_range[S.t], u1 = S.tree_range[S.t + 1];
   for (;;) {
     unsigned long long slot = 0;
@@ -1226,8 +1261,7 @@ __global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : kWalkWarpsP
       p1 += __ffs(~same) - 1;
       break;
     }
-    walk_bucket<NBP, kPP, kCSM>(a, bk, p0, p1, int(uint32_t(bkey)), gw, lane, stk, off,
-                                next_beam, lstk, U, Up, V, T);
+    walk_bucket<NBP, kPP, kCSM, kCells>(a, bk, p0, p1, int(uint32_t(bkey)), gw, lane, w);
   }
 }
 
@@ -1253,7 +1287,12 @@ void fill_walk_args(const Tree* t, const Table* tb, int nside, float theta, cons
   a->inv = t->inv;
   a->hn = t->hn;
   a->km = t->km;
+  a->lmask = t->lmask;
   a->dirs = tb->dirs;
+  a->beam_list = tb->beam_list;
+  a->beam_count = tb->beam_count;
+  a->beam_inv = tb->beam_inv;
+  a->beam_side = beam_map_side(nside);
   a->N = t->N;
   a->nside = nside;
   a->npix = 12 * nside * nside;
@@ -1278,21 +1317,67 @@ void fill_walk_args(const Tree* t, const Table* tb, int nside, float theta, cons
   a->counter = t->counter;
 }
 
-template <int NBP>
+constexpr int kCellCap = 2048;     // cells of a cut listed at once
+constexpr int kCellSources = 512;  // sources whose distances a warp holds at once
+
+size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
+  a->stack_ints = 64 * (a->max_depth + 2);
+  if (!cells) {
+    a->region_ints = a->stack_ints;
+    a->warp_ints = a->region_ints + 2 * a->npix + 36 + 8 * (a->max_depth + 1);
+  } else {
+    // the search for p-p particles needs the larger stack, phase_cut half of it
+    if (!pp) a->stack_ints = 32 * (a->max_depth + 2);
+    a->bin_cap = kCellSources;
+    a->region_ints = std::max(a->stack_ints, kCellStage + kCellHits + a->bin_cap);
+    a->warp_ints = a->region_ints + 2 * a->npix + 36;
+  }
+  a->src_stack_cap = a->stack_ints;
+  if (const int cap = debug_source_stack_cap()) a->src_stack_cap = std::min(cap, a->stack_ints);
+  return (size_t(warps) * a->warp_ints + (cells ? 4 * size_t(a->npix) : 0)) * sizeof(int);
+}
+
+// Whether a walk of this tree sums its absorption cell by cell.  It does where
+// that measured faster on fields of 48^3 and 110^3 elements, 3 bands (ms, cell
+// by cell / beam by beam):
+//  - theta: a cut holds about theta^-3 cells but a beam crosses theta^-1 of
+//    them.  110^3, nside 1: theta 0.42 98.8 / 93.2, 0.5 66.8 / 72.2; nside 2:
+//    96.7 / 95.6, 68.5 / 77.7; nside 4: 0.35 220 / 198, 0.42 145 / 160, 0.5 104 / 134;
+//  - sources: beams without any are not walked.  48^3, theta 0.5, nside 4: 30
+//    sources 2.90 / 2.41, 60 3.24 / 3.26, 120 3.63 / 4.16; nside 2: 3 sources
+//    1.88 / 1.79, 12 2.00 / 2.08; nside 1: 1 source 1.63 / 1.43, 3 1.66 / 1.75;
+//  - refinement opens cells that no beam with sources comes near: beam by beam.
+static bool use_cells(const Tree* t, const Table* tb, float theta) {
+  return tb->nside <= kCellNside && !t->refine_on && theta >= (tb->nside < 4 ? 0.45f : 0.4f) &&
+         3 * t->n_luminous >= 12 * tb->nside * tb->nside;
+}
+
+// The beam look-up tables for a walk cell by cell.
+static int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st) {
+  T2_CHECK(ensure_beam_map(tb, st));
+  a->beam_list = tb->beam_list;
+  a->beam_count = tb->beam_count;
+  a->beam_inv = tb->beam_inv;
+  return TREVR2_OK;
+}
+
+template <int NBP, bool kCells>
 static const void* walk_kernel_nbp(int warps, bool batched) {
   if (batched)
-    return warps == 4 ? reinterpret_cast<const void*>(&k_walk_batched<NBP, 4>)
-                      : reinterpret_cast<const void*>(&k_walk_batched<NBP, 8>);
-  return warps == 4 ? reinterpret_cast<const void*>(&k_walk<NBP, 4>)
-                    : reinterpret_cast<const void*>(&k_walk<NBP, 8>);
+    return warps == 4 ? reinterpret_cast<const void*>(&k_walk_batched<NBP, 4, kCells>)
+                      : reinterpret_cast<const void*>(&k_walk_batched<NBP, 8, kCells>);
+  return reinterpret_cast<const void*>(&k_walk<NBP, kWalkWarps, kCells>);
 }
 
-static const void* walk_kernel(int nbp, int warps, bool batched) {
-  return nbp == 1 ? walk_kernel_nbp<1>(warps, batched)
-       : nbp == 2 ? walk_kernel_nbp<2>(warps, batched)
-                  : walk_kernel_nbp<4>(warps, batched);
+static const void* walk_kernel(int nbp, int warps, bool batched, bool cells) {
+  if (cells)
+    return nbp == 1 ? walk_kernel_nbp<1, true>(warps, batched)
+         : nbp == 2 ? walk_kernel_nbp<2, true>(warps, batched)
+                    : walk_kernel_nbp<4, true>(warps, batched);
+  return nbp == 1 ? walk_kernel_nbp<1, false>(warps, batched)
+       : nbp == 2 ? walk_kernel_nbp<2, false>(warps, batched)
+                  : walk_kernel_nbp<4, false>(warps, batched);
 }
-
 
 // Shared memory attribute and resident blocks per SM of a walk kernel.
 int config_walk_kernel(const void* fn, int warps, size_t smem, int* per_sm, int* sms) {
@@ -1312,18 +1397,21 @@ int config_walk_kernel(const void* fn, int warps, size_t smem, int* per_sm, int*
   return TREVR2_OK;
 }
 
-// Walk buffers: per warp, M source records in and out and their beams; the
+// Walk buffers: per warp, M source records in and out and their beams, and
+// (cell by cell) the list of cell_cap absorbing cells and the M sources' own depths; the
 // optical depths of the binned records reuse the space of the unbinned ones.
-static size_t walk_buffer_bytes(size_t warps, int M) {
-  return warps * size_t(M) * (2 * sizeof(SrcEntry) + sizeof(int));
+static size_t walk_buffer_bytes(size_t warps, int M, int cell_cap) {
+  const size_t cells = cell_cap > 0 ? size_t(cell_cap) * sizeof(int) + size_t(M) * sizeof(float4) : 0;
+  return warps * (size_t(M) * (2 * sizeof(SrcEntry) + sizeof(int)) + cells);
 }
 
 static void place_walk_buffers(char* base, size_t warps, int M, SrcEntry** U, SrcEntry** V,
-                               float** T, int** Up) {
+                               float** T, int** Up, int** cells) {
   *U = reinterpret_cast<SrcEntry*>(base);
   *V = reinterpret_cast<SrcEntry*>(base + warps * M * sizeof(SrcEntry));
   *T = reinterpret_cast<float*>(*U);  // the staged records are dead once binned
   *Up = reinterpret_cast<int*>(base + 2 * warps * M * sizeof(SrcEntry));
+  *cells = *Up + warps * M;
 }
 
 // A grown-on-demand device buffer: at least `need` bytes in *buf.  A failed
@@ -1368,17 +1456,21 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
     T2_CHECK(radix_sort_u64_i32(keys, slots, A, st, bits));
     a.order = slots;
   }
-  const void* fn = walk_kernel(t->nbp, kWalkWarps, false);
-  const size_t smem = walk_smem(kWalkWarps, a.stack_ints, a.npix, a.max_depth);
+  const bool cells = use_cells(t, tb, theta);
+  if (cells) T2_CHECK(use_beam_map(tb, &a, st));
+  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells);
+  const size_t smem = walk_layout(&a, kWalkWarps, cells, false);
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kWalkWarps, smem, &per_sm, &sms));
   int64_t blocks = int64_t(sms) * per_sm;
   blocks = std::min<int64_t>(blocks, (A + kWalkWarps - 1) / kWalkWarps);
   blocks = std::max<int64_t>(blocks, 1);
   const size_t warps = size_t(blocks) * kWalkWarps;
-  const size_t need = walk_buffer_bytes(warps, a.M);
+  a.cell_cap = cells ? kCellCap : 0;
+  const size_t need = walk_buffer_bytes(warps, a.M, a.cell_cap);
   T2_CHECK(grow_buffer(&t->scratch, &t->scratch_bytes, need, st, "walk buffers"));
-  place_walk_buffers(static_cast<char*>(t->scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU);
+  place_walk_buffers(static_cast<char*>(t->scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU,
+                     &a.cells);
   T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
   void* args[] = {&a};
   T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(kWalkWarps * 32), args, smem, st));
@@ -1525,32 +1617,46 @@ static int ensure_csm(Tree* t, Table* tb, cudaStream_t st) {
   return TREVR2_OK;
 }
 
-template <int NBP>
+template <int NBP, bool kCells>
 static const void* bucket_kernel_nbp(bool pp, bool csm) {
   if (csm)
-    return pp ? reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, true, true>)
-              : reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, false, true>);
-  return pp ? reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, true, false>)
-            : reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, false, false>);
+    return pp ? reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, true, true, kCells>)
+              : reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, false, true, kCells>);
+  return pp ? reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, true, false, kCells>)
+            : reinterpret_cast<const void*>(&k_walk_bucket<NBP, kWalkWarps, false, false, kCells>);
+}
+
+static const void* bucket_kernel(int nbp, bool pp, bool csm, bool cells) {
+  if (cells)
+    return nbp == 1 ? bucket_kernel_nbp<1, true>(pp, csm)
+         : nbp == 2 ? bucket_kernel_nbp<2, true>(pp, csm)
+                    : bucket_kernel_nbp<4, true>(pp, csm);
+  return nbp == 1 ? bucket_kernel_nbp<1, false>(pp, csm)
+       : nbp == 2 ? bucket_kernel_nbp<2, false>(pp, csm)
+                  : bucket_kernel_nbp<4, false>(pp, csm);
 }
 
 // p-p particles one warp holds for a bucket (TREVR2_PP); a bucket whose
 // sphere holds more is reported (EUNSUPPORTED).
 constexpr int kPPCapacity = 4096;
 
-template <int NBP>
+template <int NBP, bool kCells>
 static const void* bucket_batched_kernel_nbp(bool pp, bool csm) {
   if (csm)
-    return pp ? reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, true, true>)
-              : reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, false, true>);
-  return pp ? reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, true, false>)
-            : reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, false, false>);
+    return pp ? reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, true, true, kCells>)
+              : reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, false, true, kCells>);
+  return pp ? reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, true, false, kCells>)
+            : reinterpret_cast<const void*>(&k_walk_bucket_batched<NBP, kWalkWarps, false, false, kCells>);
 }
 
-static const void* bucket_batched_kernel(int nbp, bool pp, bool csm) {
-  return nbp == 1 ? bucket_batched_kernel_nbp<1>(pp, csm)
-       : nbp == 2 ? bucket_batched_kernel_nbp<2>(pp, csm)
-                  : bucket_batched_kernel_nbp<4>(pp, csm);
+static const void* bucket_batched_kernel(int nbp, bool pp, bool csm, bool cells) {
+  if (cells)
+    return nbp == 1 ? bucket_batched_kernel_nbp<1, true>(pp, csm)
+         : nbp == 2 ? bucket_batched_kernel_nbp<2, true>(pp, csm)
+                    : bucket_batched_kernel_nbp<4, true>(pp, csm);
+  return nbp == 1 ? bucket_batched_kernel_nbp<1, false>(pp, csm)
+       : nbp == 2 ? bucket_batched_kernel_nbp<2, false>(pp, csm)
+                  : bucket_batched_kernel_nbp<4, false>(pp, csm);
 }
 
 // TREVR2_BUCKET: receivers in Morton order, the leaf of each, one warp per
@@ -1599,23 +1705,25 @@ static int launch_walk_bucket(Tree* t, Table* tb, const int64_t* active, int64_t
   bk.directed = target != nullptr;
   for (int c = 0; c < 3; ++c) bk.target[c] = target ? (target[c] - t->lo[c]) / t->size : 0.0;
   const bool csm = (flags & TREVR2_CSM) != 0;
-  const void* fn = t->nbp == 1 ? bucket_kernel_nbp<1>(bk.pp, csm)
-                 : t->nbp == 2 ? bucket_kernel_nbp<2>(bk.pp, csm)
-                               : bucket_kernel_nbp<4>(bk.pp, csm);
-  const size_t smem = walk_smem(kWalkWarps, a.stack_ints, a.npix, a.max_depth);
+  const bool cells = use_cells(t, tb, theta) && !target;
+  if (cells) T2_CHECK(use_beam_map(tb, &a, st));
+  const void* fn = bucket_kernel(t->nbp, bk.pp, csm, cells);
+  const size_t smem = walk_layout(&a, kWalkWarps, cells, bk.pp != 0);
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kWalkWarps, smem, &per_sm, &sms));
   int64_t blocks = int64_t(sms) * per_sm;
   blocks = std::min<int64_t>(blocks, (A + kWalkWarps - 1) / kWalkWarps);
   blocks = std::max<int64_t>(blocks, 1);
   const size_t warps = size_t(blocks) * kWalkWarps;
-  const size_t wb = (walk_buffer_bytes(warps, a.M) + 255) & ~size_t(255);
+  a.cell_cap = cells ? kCellCap : 0;
+  const size_t wb = (walk_buffer_bytes(warps, a.M, a.cell_cap) + 255) & ~size_t(255);
   const size_t ob = (warps * kOriginWords * sizeof(double) + 255) & ~size_t(255);
   const size_t pb = warps * size_t(bk.pp_cap) *
                     (4 * sizeof(float4) + sizeof(int) + kCubeCells / 32 * sizeof(uint32_t));
   const size_t need = wb + ob + pb;
   T2_CHECK(grow_buffer(&t->scratch, &t->scratch_bytes, need, st, "walk buffers"));
-  place_walk_buffers(static_cast<char*>(t->scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU);
+  place_walk_buffers(static_cast<char*>(t->scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU,
+                     &a.cells);
   a.origin64 = reinterpret_cast<double*>(static_cast<char*>(t->scratch) + wb);
   if (bk.pp) {
     char* pp = static_cast<char*>(t->scratch) + wb + ob;
@@ -1771,15 +1879,17 @@ struct Batch {
   int key_bits = 64;
   int warps = kWalkWarps;  // chosen launch shape
   int M = kSrcCapacity;    // chosen source staging depth
-  const void* fn = nullptr;  // kernel, shared memory and grid of that shape
-  size_t smem = 0;
-  int64_t blocks = 0;
+  // kernel, shared memory and grid of that shape: beam by beam, cell by cell
+  const void* fn[2] = {nullptr, nullptr};
+  size_t smem[2] = {0, 0};
+  int64_t blocks[2] = {0, 0};
   bool ready = false;        // the shape covers every row (false after a failed autotune)
   cudaStream_t last_stream = nullptr;
   // per-bucket plans (TREVR2_BUCKET, with TREVR2_PP / TREVR2_CSM)
   bool bucket = false;
   bool pp = false;
   bool csm = false;
+  bool cells[kMaxBatchTrees] = {};  // per tree: absorption cell by cell
   BucketBatchArgs bb;
   BatchArgs args;
 };
@@ -1788,17 +1898,27 @@ struct Batch {
 // grid and walk buffers (grown if needed).  Nothing changes unless it
 // succeeds: a larger buffer is allocated before the old one is released.
 static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t st) {
-  const void* fn = b->bucket ? bucket_batched_kernel(b->nbp, b->pp, b->csm)
-                             : walk_kernel(b->nbp, warps, true);
-  const size_t smem = walk_smem(warps, b->args.stack_ints, b->args.npix, b->args.max_depth);
-  int per_sm = 0, sms = 0;
-  T2_CHECK(config_walk_kernel(fn, warps, smem, &per_sm, &sms));
-  int64_t g = int64_t(sms) * per_sm;
-  g = std::min<int64_t>(g, (limit + warps - 1) / warps);
-  const int64_t blocks = std::max<int64_t>(g, 1);
-  const size_t nw = size_t(blocks) * warps;
+  // kernel, shared memory and grid of the trees walked beam by beam [0] and
+  // cell by cell [1]: one layout each, the deepest tree's
+  const void* fn[2] = {nullptr, nullptr};
+  size_t smem[2] = {0, 0};
+  int64_t blocks[2] = {0, 0};
+  for (size_t i = 0; i < b->trees.size(); ++i) {
+    const int c = b->cells[i] ? 1 : 0;
+    smem[c] = walk_layout(&b->args.tree[i], warps, c != 0, b->pp);
+    b->args.tree[i].cell_cap = c ? kCellCap : 0;
+    if (fn[c]) continue;
+    fn[c] = b->bucket ? bucket_batched_kernel(b->nbp, b->pp, b->csm, c != 0)
+                      : walk_kernel(b->nbp, warps, true, c != 0);
+    int per_sm = 0, sms = 0;
+    T2_CHECK(config_walk_kernel(fn[c], warps, smem[c], &per_sm, &sms));
+    const int64_t g = std::min<int64_t>(int64_t(sms) * per_sm, (limit + warps - 1) / warps);
+    blocks[c] = std::max<int64_t>(g, 1);
+  }
+  const int cell_cap = blocks[1] ? kCellCap : 0;
+  const size_t nw = size_t(std::max(blocks[0], blocks[1])) * warps;
   // per-bucket plans: the warps' FP64 origin slots and p-p particle arrays
-  const size_t wb = (walk_buffer_bytes(nw, M) + 255) & ~size_t(255);
+  const size_t wb = (walk_buffer_bytes(nw, M, cell_cap) + 255) & ~size_t(255);
   const size_t ob = b->bucket ? (nw * kOriginWords * sizeof(double) + 255) & ~size_t(255) : 0;
   const size_t pp_cap = b->pp ? kPPCapacity : 0;
   const size_t pb = nw * pp_cap *
@@ -1812,7 +1932,7 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
     b->scratch_bytes = need;
   }
   place_walk_buffers(static_cast<char*>(b->scratch), nw, M, &b->args.srcU, &b->args.srcV,
-                     &b->args.srcT, &b->args.pixU);
+                     &b->args.srcT, &b->args.pixU, &b->args.cells);
   b->args.M = M;
   for (size_t i = 0; i < b->trees.size(); ++i) b->args.tree[i].M = M;
   if (b->bucket) {
@@ -1833,9 +1953,11 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
                          : nullptr;
     }
   }
-  b->fn = fn;
-  b->smem = smem;
-  b->blocks = blocks;
+  for (int c = 0; c < 2; ++c) {
+    b->fn[c] = fn[c];
+    b->smem[c] = smem[c];
+    b->blocks[c] = blocks[c];
+  }
   b->warps = warps;
   b->M = M;
   b->args.total = limit;
@@ -1875,18 +1997,20 @@ static int batch_enqueue(Batch* b, const int64_t* active, float* J, cudaStream_t
   sl.pixU = b->args.pixU;
   sl.srcV = b->args.srcV;
   sl.srcT = b->args.srcT;
+  sl.cells = b->args.cells;
   sl.counter = b->counter;
   for (int t = 0; t < b->args.ntrees; ++t) {
     sl.t = t;
+    const int c = b->cells[t] ? 1 : 0;
     T2_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(unsigned long long), st));
     if (b->bucket) {
       void* argv[] = {&b->args.tree[t], &b->bb.tree[t], &sl};
-      T2_CUDA(cudaLaunchKernel(b->fn, dim3(unsigned(b->blocks)), dim3(b->warps * 32), argv,
-                               b->smem, st));
+      T2_CUDA(cudaLaunchKernel(b->fn[c], dim3(unsigned(b->blocks[c])), dim3(b->warps * 32), argv,
+                               b->smem[c], st));
     } else {
       void* argv[] = {&b->args.tree[t], &sl};
-      T2_CUDA(cudaLaunchKernel(b->fn, dim3(unsigned(b->blocks)), dim3(b->warps * 32), argv,
-                               b->smem, st));
+      T2_CUDA(cudaLaunchKernel(b->fn[c], dim3(unsigned(b->blocks[c])), dim3(b->warps * 32), argv,
+                               b->smem[c], st));
     }
     note_launch();
   }
@@ -1996,6 +2120,9 @@ extern "C" int trevr2_batch_create(trevr2_tree* const* trees, int ntrees, const 
     Table* tb = nullptr;
     int rc = ensure_table(t, nside, st, &tb, (flags & TREVR2_LINEAR) != 0);
     if (rc) return fail(rc);
+    b->cells[i] = use_cells(t, tb, theta);
+    if (b->cells[i]) rc = ensure_beam_map(tb, st);
+    if (rc) return fail(rc);
     if (!b->bucket) {
       fill_walk_args(t, tb, nside, theta, bsel, nb, flags & ~TREVR2_ASYNC, kSrcCapacity,
                      &b->args.tree[i]);
@@ -2023,16 +2150,8 @@ extern "C" int trevr2_batch_create(trevr2_tree* const* trees, int ntrees, const 
     b->bb.first[i] = t->first;
   }
   // one shared-memory layout for all trees: the deepest one's
-  for (int i = 0; i < ntrees; ++i) {
-    b->args.tree[i].max_depth = max_depth;
-    b->args.tree[i].stack_ints = 64 * (max_depth + 2);
-    b->args.tree[i].src_stack_cap = b->args.tree[i].stack_ints;
-    if (const int cap = debug_source_stack_cap())
-      b->args.tree[i].src_stack_cap = std::min(cap, b->args.tree[i].stack_ints);
-  }
+  for (int i = 0; i < ntrees; ++i) b->args.tree[i].max_depth = max_depth;
   b->args.max_depth = max_depth;
-  b->args.stack_ints = 64 * (max_depth + 2);
-  b->args.npix = 12 * nside * nside;
   b->args.nbsel = nb;
   b->args.nsub = nsub;
   b->args.ntrees = ntrees;
@@ -2229,7 +2348,7 @@ extern "C" int trevr2_kernel_binary_version(int* version) {
     return TREVR2_EINVAL;
   }
   cudaFuncAttributes attr;
-  T2_CUDA(cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(&k_walk<4, kWalkWarps>)));
+  T2_CUDA(cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(&k_walk<4, kWalkWarps, true>)));
   *version = attr.binaryVersion;
   return TREVR2_OK;
 }
@@ -2299,13 +2418,16 @@ static int launch_walk_noalloc(Tree* t, Table* tb, const int64_t* active, int64_
   a.active = active;
   a.A = A;
   a.J = J;
-  const void* fn = walk_kernel(t->nbp, kWalkWarps, false);
-  const size_t smem = walk_smem(kWalkWarps, a.stack_ints, a.npix, a.max_depth);
+  // beam by beam: walking cell by cell needs larger buffers, which would leave
+  // room for fewer warps in the fixed array
+  const bool cells = false;
+  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells);
+  const size_t smem = walk_layout(&a, kWalkWarps, cells, false);
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kWalkWarps, smem, &per_sm, &sms));
   // The grid is capped by what the fixed array holds; the kernel loops over
   // receivers and passes over sources, so any A and any source count fit.
-  const size_t per_block = walk_buffer_bytes(kWalkWarps, a.M);
+  const size_t per_block = walk_buffer_bytes(kWalkWarps, a.M, 0);
   const int64_t max_blocks = int64_t(kNoAllocScratchBytes / per_block);
   if (max_blocks < 1) {
     set_error("trevr2_J_noalloc: one block needs %zu bytes of walk buffers, the fixed array "
@@ -2317,7 +2439,8 @@ static int launch_walk_noalloc(Tree* t, Table* tb, const int64_t* active, int64_
   blocks = std::min<int64_t>(blocks, max_blocks);
   blocks = std::max<int64_t>(blocks, 1);
   const size_t warps = size_t(blocks) * kWalkWarps;
-  place_walk_buffers(static_cast<char*>(scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU);
+  place_walk_buffers(static_cast<char*>(scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU,
+                     &a.cells);
   T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
   void* args[] = {&a};
   T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(kWalkWarps * 32), args, smem, st));

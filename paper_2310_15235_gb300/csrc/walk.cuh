@@ -17,6 +17,8 @@ constexpr int kWalkWarps = 4;                 // warps per block
 // warps (72 registers a thread) measured faster than 6 at 80 registers and
 // than 8 at 64 registers, which spills.
 constexpr int kWalkWarpsPerSM = 28;
+// Resident warps per SM of the kernels that sum the absorption cell by cell.
+constexpr int kCellWarpsPerSM = 28;
 constexpr int kSrcCapacity = 1024;            // sources held per warp and pass
 constexpr float kFourPi = 12.566370614359172f;
 
@@ -34,6 +36,7 @@ struct WalkArgs {
   const int* inv;
   const float* hn;
   const float* km;
+  const uint32_t* lmask;
   const float4* dirs;
   const int64_t* active;
   const int* order;  // walk order of the receivers (NULL: as given)
@@ -57,6 +60,8 @@ struct WalkArgs {
                     // directed beam (unit vector, pixel or -1)
   int M;
   int stack_ints;   // per warp
+  int region_ints;  // per warp: the stacks, or what phase A keeps in their place
+  int warp_ints;    // shared memory of a warp
   int src_stack_cap;  // entries of the source cut's stack used (<= stack_ints)
   int max_depth;
   uint32_t* status;
@@ -65,6 +70,14 @@ struct WalkArgs {
   const float* csm_tau;  // [n][npix][nbp]
   const float* csm_d;    // [n][npix]
   const int* csm_anti;   // [npix]
+  // absorption cell by cell (beams up to kCellNside; cells.cuh)
+  const uint8_t* beam_list;
+  const uint8_t* beam_count;
+  const float4* beam_inv;
+  int beam_side;    // squares per face and axis of the direction map
+  int* cells;       // [warps][cell_cap] absorbing cells of the cut
+  int cell_cap;
+  int bin_cap;      // sources whose distances a warp holds
 };
 
 __device__ __forceinline__ float3 node_ext(uint32_t meta) {
@@ -450,18 +463,19 @@ static __device__ int phase_sources(const WalkArgs& a, float3 x, int si, int lan
       }
     }
     // push opened halves
-    const int incl = warp_incl_scan(npush, lane);
-    const int tot = __shfl_sync(0xffffffffu, incl, 31);
-    if (npush) {
-      const int pos = sp + incl - npush;
-      if (pos + 2 <= cap) {
-        stk[pos] = child + 1;
-        stk[pos + 1] = child;
-      } else {
-        atomicOr(a.status, kStatusStackOverflow);
+    {
+      const unsigned m = __ballot_sync(0xffffffffu, npush > 0);
+      const int room = (cap - sp) >> 1, at = __popc(m & lt);
+      if (npush) {
+        if (at < room) {
+          stk[sp + 2 * at] = child + 1;
+          stk[sp + 2 * at + 1] = child;
+        } else {
+          atomicOr(a.status, kStatusStackOverflow);
+        }
       }
+      sp += 2 * min(__popc(m), room);
     }
-    sp = min(sp + tot, cap);
     // accepted luminous cells
     {
       const unsigned m = __ballot_sync(0xffffffffu, emit_node);
@@ -524,7 +538,7 @@ static __device__ int bin_sources(const WalkArgs& a, int lane, SrcEntry* U, cons
   for (int k = lane; k < npix; k += 32) off[k] = 0;
   __syncwarp();
   for (int e = lane; e < n; e += 32)
-    if (Up[e] >= 0) atomicAdd(&off[Up[e]], 1);
+    if (const int k = Up[e]; k >= 0) atomicAdd(&off[k], 1);
   __syncwarp();
   // exclusive scan of the bucket sizes
   const int per = (npix + 31) / 32;
@@ -540,8 +554,9 @@ static __device__ int bin_sources(const WalkArgs& a, int lane, SrcEntry* U, cons
   }
   __syncwarp();
   for (int e = lane; e < n; e += 32) {
-    if (Up[e] < 0) continue;
-    const int slot = atomicAdd(&off[Up[e]], 1);
+    const int k = Up[e];
+    if (k < 0) continue;
+    const int slot = atomicAdd(&off[k], 1);
     V[slot] = U[e];
   }
   __syncwarp();
@@ -643,11 +658,10 @@ int config_walk_kernel(const void* fn, int warps, size_t smem, int* per_sm, int*
 // Synchronises `st` and returns (and clears) the tree's device status.
 int read_status(Tree* t, cudaStream_t st);
 
-// Per-warp shared memory of a walk block: the traversal stacks, the beam
-// bucket offsets, the beam order and its 32 bucket counts, the next-beam
-// counter (padded to 16 bytes), the receiver's ancestor records.
-inline size_t walk_smem(int warps, int stack_ints, int npix, int max_depth) {
-  return size_t(warps) * (stack_ints + 2 * npix + 36 + 8 * (max_depth + 1)) * sizeof(int);
-}
+// Sets the per-warp shared memory layout of a forward walk and returns a
+// block's bytes.  Beam by beam: the traversal stacks, the beam bucket offsets,
+// the beam order and its 32 bucket counts, the next-beam counter (padded to 16
+// bytes), the receiver's ancestor records.  Cell by cell: see cells.cuh.
+size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp);
 
 }  // namespace trevr2
