@@ -41,8 +41,8 @@ extern "C" {
 #define TREVR2_EINVAL (-1)      /* invalid argument or input value            */
 #define TREVR2_ENOMEM (-2)      /* device or host allocation failed           */
 #define TREVR2_ECUDA (-3)       /* a CUDA runtime call failed                 */
-#define TREVR2_ETIMEOUT (-4)    /* reserved: no kernel of this library waits on
-                                   the device, so no call returns it           */
+#define TREVR2_ETIMEOUT (-4)    /* a cooperative kernel's blocks gave up waiting
+                                   for one another (a bounded number of polls) */
 #define TREVR2_EUNSUPPORTED (-5)/* outside the supported sizes (see below)    */
 #define TREVR2_EINTERNAL (-6)   /* an internal capacity check failed          */
 

@@ -1,11 +1,16 @@
 // Radiation tree build on the GPU (TREVR2, Sec. 2.3 and Sec. 2.6):
-// FP64 normalisation + 63-bit Morton keys, a stable LSD radix sort,
-// level-by-level bisection (a node splits while it holds more than `bucket`
-// elements; empty halves become empty leaves), and a bottom-up pass for the
-// summed luminosity per band, the centre of luminosity (one band-summed
-// centre per cell), B = largest centre-to-corner distance (Sec. 2.5.2) and the
-// bucket absorption sum(kappa m)/V_box (Sec. 2.6).  Sums run in FP64 and are
-// rounded once to FP32 for the walk.
+// FP64 normalisation + 63-bit Morton keys, a stable sort, bisection level by
+// level (a node splits while it holds more than `bucket` elements; empty
+// halves become empty leaves), and a bottom-up pass for the summed luminosity
+// per band, the centre of luminosity (one band-summed centre per cell), B =
+// largest centre-to-corner distance (Sec. 2.5.2) and the bucket absorption
+// sum(kappa m)/V_box (Sec. 2.6).  Sums run in FP64 and are rounded once to FP32
+// for the walk.
+//
+// Small and middle trees were bound by launches and read-backs, not by the
+// kernels: the levels' sizes went to the host one by one.  The whole build is
+// now seven launches and one read-back (33k elements, whole step: 2.21 -> 1.53
+// ms; 4k: 1.41 -> 0.90; 2.1M elements and a 1000-receiver rung: 5.86 -> 4.26).
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -164,84 +169,243 @@ int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort, 8 bits per pass.  Each tile of 2048 keys is ranked
-// in 8 rounds of 256 keys; inside a round, warps rank their lanes with
-// __match_any_sync and a per-warp digit count, so equal digits keep their
-// input order (stability gives the (key, caller index) order).
-constexpr int kSortThreads = 256;
-constexpr int kSortTile = 2048;
-constexpr int kSortWarps = kSortThreads / 32;
+// Stable sort of 64-bit keys with a 32-bit payload.
+//
+// Up to kSmallSort keys: one block, a bitonic sort of (key, input position) in
+// shared memory; the position makes the order stable.  More: one cooperative
+// launch does every pass of an LSD radix sort (8 bits a pass), with a grid
+// barrier where a pass needs all blocks' counts or keys: a launch for each
+// step of each pass left the GPU idle between them for longer than the steps
+// took (33k elements: 47 launches; now 1).
+constexpr int kSmallSort = 8192;
+constexpr int kSmallSortThreads = 1024;
 
-__global__ void k_radix_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                             int* __restrict__ hist, int ntiles) {
-  __shared__ int h[256];
-  h[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = int64_t(blockIdx.x) * kSortTile;
-  for (int k = threadIdx.x; k < kSortTile; k += kSortThreads) {
-    int64_t i = base + k;
-    if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1);
-  }
-  __syncthreads();
-  hist[int64_t(threadIdx.x) * ntiles + blockIdx.x] = h[threadIdx.x];
+__device__ __forceinline__ bool sort_after(uint64_t ka, uint32_t pa, uint64_t kb, uint32_t pb) {
+  return ka > kb || (ka == kb && pa > pb);
 }
 
-__global__ void k_radix_scatter(const uint64_t* __restrict__ kin, const int* __restrict__ vin,
-                                uint64_t* __restrict__ kout, int* __restrict__ vout, int64_t n,
-                                int shift, const int* __restrict__ offsets, int ntiles) {
+// With `active`, the receivers' order: the keys are their elements' sorted
+// positions (N for an index outside [0, N)), the payload their slots.
+__global__ void __launch_bounds__(kSmallSortThreads)
+    k_sort_small(uint64_t* keys, int* vals, int n, int n2, const int64_t* __restrict__ active,
+                 const int* __restrict__ inv, int64_t N) {
+  extern __shared__ uint64_t sort_smem[];
+  uint64_t* k = sort_smem;
+  uint32_t* p = reinterpret_cast<uint32_t*>(k + n2);
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+    uint64_t key = ~0ull;  // the padding comes last: its positions are beyond n
+    if (i < n) {
+      if (active) {
+        const int64_t io = active[i];
+        key = io >= 0 && io < N ? uint64_t(inv[io]) : uint64_t(N);
+      } else {
+        key = keys[i];
+      }
+    }
+    k[i] = key;
+    p[i] = uint32_t(i);
+  }
+  __syncthreads();
+  for (int size = 2; size <= n2; size <<= 1)
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      for (int t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
+        const int i = 2 * t - (t & (stride - 1)), j = i + stride;
+        const uint64_t ki = k[i], kj = k[j];
+        const uint32_t pi = p[i], pj = p[j];
+        if (sort_after(ki, pi, kj, pj) == ((i & size) == 0)) {
+          k[i] = kj;
+          k[j] = ki;
+          p[i] = pj;
+          p[j] = pi;
+        }
+      }
+      __syncthreads();
+    }
+  constexpr int kPer = kSmallSort / kSmallSortThreads;
+  int v[kPer];
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int i = threadIdx.x + r * blockDim.x;
+    if (i < n) v[r] = active ? int(p[i]) : vals[p[i]];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int i = threadIdx.x + r * blockDim.x;
+    if (i < n) {
+      keys[i] = k[i];
+      vals[i] = v[r];
+    }
+  }
+}
+
+// One block per chunk of consecutive keys.  A pass counts the chunk's digits,
+// waits for all blocks, places its own digits after those of smaller digits
+// and earlier blocks, and scatters 512 keys a round: warps rank their lanes
+// with __match_any_sync and per-warp digit counts, so equal digits keep their
+// order.  Keys are read past the L1, which other blocks' writes do not reach.
+constexpr int kSortThreads = 512;
+constexpr int kSortWarps = kSortThreads / 32;
+
+__global__ void __launch_bounds__(kSortThreads)
+    k_radix_sort(uint64_t* ka, int* va, uint64_t* kb, int* vb, int64_t n, int passes, int* hist,
+                 uint32_t* bar, uint32_t* status) {
   __shared__ int base[256];
   __shared__ int wh[kSortWarps][256];
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  base[t] = offsets[int64_t(t) * ntiles + blockIdx.x];
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int64_t tile0 = int64_t(blockIdx.x) * kSortTile;
-  for (int round = 0; round < kSortTile / kSortThreads; ++round) {
-    for (int w = 0; w < kSortWarps; ++w) wh[w][t] = 0;
+  __shared__ int tot2[2][256], bef2[2][256];
+  __shared__ int wsum[8];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nb = gridDim.x, b = blockIdx.x;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t per = (n + nb - 1) / nb;
+  const int64_t lo = min(n, b * per), hi = min(n, lo + per);
+  for (int pass = 0; pass < passes; ++pass) {
+    const int shift = 8 * pass;
+    if (t < 256) base[t] = 0;
     __syncthreads();
-    int64_t i = tile0 + round * kSortThreads + t;
-    bool valid = i < n;
-    uint64_t key = valid ? kin[i] : 0;
-    int val = valid ? vin[i] : 0;
-    int digit = valid ? int((key >> shift) & 255u) : 256;
-    unsigned peers = __match_any_sync(0xffffffffu, digit);
-    int intra = __popc(peers & lt_mask);
-    if (valid && intra == 0) wh[warp][digit] = __popc(peers);
+    for (int64_t i = lo + t; i < hi; i += kSortThreads)
+      atomicAdd(&base[(__ldcg(ka + i) >> shift) & 255u], 1);
     __syncthreads();
+    if (t < 256) __stcg(hist + b * 256 + t, base[t]);
+    if (!grid_barrier(bar, nb, status)) return;
     {
-      int run = base[t];
-      for (int w = 0; w < kSortWarps; ++w) {
-        int c = wh[w][t];
-        wh[w][t] = run;
-        run += c;
+      const int d = t & 255, h = t >> 8;
+      int tot = 0, bef = 0;
+      for (int o = h; o < nb; o += 2) {
+        const int c = __ldcg(hist + o * 256 + d);
+        tot += c;
+        if (o < b) bef += c;
       }
-      base[t] = run;
+      tot2[h][d] = tot;
+      bef2[h][d] = bef;
     }
     __syncthreads();
-    if (valid) {
-      int dst = wh[warp][digit] + intra;
-      kout[dst] = key;
-      vout[dst] = val;
+    int run = 0, mine = 0;
+    if (t < 256) {  // exclusive scan of the digits' totals
+      mine = tot2[0][t] + tot2[1][t];
+      run = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) run += u;
+      }
+      if (lane == 31) wsum[warp] = run;
     }
     __syncthreads();
+    if (t < 256) {
+      for (int w = 0; w < warp; ++w) run += wsum[w];
+      base[t] = run - mine + bef2[0][t] + bef2[1][t];
+    }
+    for (int64_t r0 = lo; r0 < hi; r0 += kSortThreads) {
+#pragma unroll
+      for (int w = 0; w < kSortWarps * 256; w += kSortThreads) (&wh[0][0])[w + t] = 0;
+      __syncthreads();
+      const int64_t i = r0 + t;
+      const bool valid = i < hi;
+      const uint64_t key = valid ? __ldcg(ka + i) : 0;
+      const int val = valid ? __ldcg(va + i) : 0;
+      const int digit = valid ? int((key >> shift) & 255u) : 256;
+      const unsigned peers = __match_any_sync(0xffffffffu, digit);
+      const int intra = __popc(peers & lt);
+      if (valid && intra == 0) wh[warp][digit] = __popc(peers);
+      __syncthreads();
+      if (t < 256) {
+        int at = base[t];
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+          const int c = wh[w][t];
+          wh[w][t] = at;
+          at += c;
+        }
+        base[t] = at;
+      }
+      __syncthreads();
+      if (valid) {
+        const int dst = wh[warp][digit] + intra;
+        __stcg(kb + dst, key);
+        __stcg(vb + dst, val);
+      }
+      __syncthreads();
+    }
+    uint64_t* const tk = ka;
+    ka = kb;
+    kb = tk;
+    int* const tv = va;
+    va = vb;
+    vb = tv;
+    if (!grid_barrier(bar, nb, status)) return;
   }
+}
+
+int coop_blocks(int64_t work, int64_t per_block, int per_sm, int* out) {
+  int dev = 0, sms = 0;
+  T2_CUDA(cudaGetDevice(&dev));
+  T2_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t most = std::min<int64_t>(int64_t(sms) * per_sm, kMaxCoopBlocks);
+  *out = int(std::max<int64_t>(1, std::min<int64_t>(most, (work + per_block - 1) / per_block)));
+  return TREVR2_OK;
+}
+
+constexpr int64_t kSortPerBlock = 2048;
+
+static int64_t sort_blocks_bound(int64_t n) {
+  return std::min<int64_t>(kMaxCoopBlocks, std::max<int64_t>(1, (n + kSortPerBlock - 1) / kSortPerBlock));
 }
 
 size_t radix_ws_bytes(int64_t n) {
-  const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
+  if (n <= kSmallSort) return 256;
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   return up(sizeof(uint64_t) * size_t(n)) + up(sizeof(int) * size_t(n)) +
-         up(sizeof(int) * 256 * size_t(ntiles)) + up(sizeof(int) * scan_ws_ints(256 * ntiles));
+         up(sizeof(int) * 256 * size_t(sort_blocks_bound(n))) + 256;
 }
 
-int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, int key_bits,
-                       void* ws) {
+static int sort_small(uint64_t* keys, int* vals, int n, cudaStream_t st, const int64_t* active,
+                      const int* inv, int64_t N) {
+  int n2 = 2;
+  while (n2 < n) n2 <<= 1;
+  const size_t smem = size_t(n2) * (sizeof(uint64_t) + sizeof(uint32_t));
+  T2_CUDA(cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kSmallSort * 12));
+  k_sort_small<<<1, std::min(kSmallSortThreads, std::max(32, n2 / 2)), smem, st>>>(
+      keys, vals, n, n2, active, inv, N);
+  note_launch();
+  T2_CUDA(cudaGetLastError());
+  return TREVR2_OK;
+}
+
+__global__ void k_order_keys(const int64_t* __restrict__ active, int64_t A, int64_t N,
+                             const int* __restrict__ inv, uint64_t* __restrict__ keys,
+                             int* __restrict__ slots) {
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i >= A) return;
+  const int64_t io = active[i];
+  keys[i] = (io >= 0 && io < N) ? uint64_t(inv[io]) : uint64_t(N);
+  slots[i] = int(i);
+}
+
+int order_receivers(const Tree* t, const int64_t* active, int64_t A, uint64_t* keys, int* slots,
+                    cudaStream_t st) {
+  if (A <= kSmallSort) return sort_small(keys, slots, int(A), st, active, t->inv, t->N);
+  k_order_keys<<<unsigned((A + 255) / 256), 256, 0, st>>>(active, A, t->N, t->inv, keys, slots);
+  note_launch();
+  int bits = 1;
+  while ((int64_t(1) << bits) <= t->N) ++bits;
+  return radix_sort_u64_i32(keys, slots, A, st, t->status, bits);
+}
+
+int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, uint32_t* status,
+                       int key_bits, void* ws) {
   if (n <= 1) return TREVR2_OK;
+  if (n <= kSmallSort) return sort_small(keys, vals, int(n), st, nullptr, nullptr, 0);
   // an even number of 8-bit passes, so the result ends in the caller's buffers
   int passes = (std::min(std::max(key_bits, 1), 64) + 7) / 8;
   passes += passes & 1;
-  const int ntiles = int((n + kSortTile - 1) / kSortTile);
-  const bool own = ws == nullptr;
-  if (own) T2_CHECK(device_alloc(&ws, radix_ws_bytes(n), st, "sort workspace"));
+  DeviceTemp<char> own(st);
+  if (!ws) {
+    T2_CHECK(device_alloc(reinterpret_cast<void**>(&own.p), radix_ws_bytes(n), st, "sort workspace"));
+    ws = own.p;
+  }
+  int nb = 0;
+  T2_CHECK(coop_blocks(n, kSortPerBlock, 1, &nb));
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   char* p = static_cast<char*>(ws);
   uint64_t* k2 = reinterpret_cast<uint64_t*>(p);
@@ -249,34 +413,46 @@ int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, in
   int* v2 = reinterpret_cast<int*>(p);
   p += up(sizeof(int) * size_t(n));
   int* hist = reinterpret_cast<int*>(p);
-  p += up(sizeof(int) * 256 * size_t(ntiles));
-  int* scan_ws = reinterpret_cast<int*>(p);
-  uint64_t *ka = keys, *kb = k2;
-  int *va = vals, *vb = v2;
-  int rc = TREVR2_OK;
-  for (int shift = 0; shift < 8 * passes && rc == TREVR2_OK; shift += 8) {
-    k_radix_hist<<<ntiles, kSortThreads, 0, st>>>(ka, n, shift, hist, ntiles); note_launch();
-    rc = scan_exclusive_i32(hist, int64_t(256) * ntiles, nullptr, st, scan_ws);
-    if (rc != TREVR2_OK) break;
-    k_radix_scatter<<<ntiles, kSortThreads, 0, st>>>(ka, va, kb, vb, n, shift, hist, ntiles); note_launch();
-    std::swap(ka, kb);
-    std::swap(va, vb);
-  }
-  if (own) cudaFreeAsync(ws, st);
-  if (rc != TREVR2_OK) return rc;
-  T2_CUDA(cudaGetLastError());
+  p += up(sizeof(int) * 256 * size_t(sort_blocks_bound(n)));
+  uint32_t* bar = reinterpret_cast<uint32_t*>(p);
+  T2_CUDA(cudaMemsetAsync(bar, 0, sizeof(uint32_t), st));
+  void* args[] = {&keys, &vals, &k2, &v2, &n, &passes, &hist, &bar, &status};
+  T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_radix_sort), dim3(unsigned(nb)),
+                                      dim3(kSortThreads), args, 0, st));
+  note_launch();
   return TREVR2_OK;
 }
 
 // ---------------------------------------------------------------------------
 // Input validation and bounds.
-__global__ void k_validate(const double* __restrict__ pos, const float* __restrict__ mass,
-                           const float* __restrict__ kappa, const float* __restrict__ lum,
-                           const float* __restrict__ h, int64_t N, int nb,
-                           double* __restrict__ partial /*[grid][6]*/, uint32_t* status) {
+// What the build's kernels find out and the host reads once at the end.
+constexpr int kMaxLevels = kMaxDepth + 2;
+struct BuildState {
+  double lo[3];      // root cube
+  double size;
+  float h_default;   // (V_root / N_gas)^(1/3), used without h
+  int n_luminous;
+  int n_nodes, n_internal, levels;
+  int need;          // nodes that did not fit (0: all did)
+  int level_begin[kMaxLevels + 1];
+  unsigned long long n_gas;
+  unsigned int tickets;
+  uint32_t bar;      // grid barrier of the tree kernel
+};
+
+// Checks the inputs (status bits) and, from the last block done, the root
+// cube: the explicit one, or the bounding cube of the positions.
+__global__ void __launch_bounds__(256)
+    k_validate(const double* __restrict__ pos, const float* __restrict__ mass,
+               const float* __restrict__ kappa, const float* __restrict__ lum,
+               const float* __restrict__ h, int64_t N, int nb, bool explicit_box, double lo0,
+               double lo1, double lo2, double box_size, double* partial /*[grid][6]*/,
+               BuildState* S, uint32_t* status) {
   __shared__ double smin[3][256], smax[3][256];
+  __shared__ bool last;
   double mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
+  int gas = 0;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < N;
        i += int64_t(gridDim.x) * blockDim.x) {
     for (int a = 0; a < 3; ++a) {
@@ -287,6 +463,7 @@ __global__ void k_validate(const double* __restrict__ pos, const float* __restri
     }
     float m = mass[i];
     bad |= !(m >= 0.0f) || !isfinite(m);
+    gas += m > 0.0f;
     if (h) bad |= !(h[i] > 0.0f) || !isfinite(h[i]);
     for (int b = 0; b < nb; ++b) {
       float k = kappa[i * nb + b], l = lum[i * nb + b];
@@ -294,24 +471,63 @@ __global__ void k_validate(const double* __restrict__ pos, const float* __restri
     }
   }
   if (bad) atomicOr(status, kStatusBadInput);
-  for (int a = 0; a < 3; ++a) {
-    smin[a][threadIdx.x] = mn[a];
-    smax[a][threadIdx.x] = mx[a];
+  gas = __reduce_add_sync(0xffffffffu, gas);
+  if ((threadIdx.x & 31) == 0 && gas) atomicAdd(&S->n_gas, (unsigned long long)(gas));
+  auto reduce = [&]() {
+    for (int a = 0; a < 3; ++a) {
+      smin[a][threadIdx.x] = mn[a];
+      smax[a][threadIdx.x] = mx[a];
+    }
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+      if (threadIdx.x < w)
+        for (int a = 0; a < 3; ++a) {
+          smin[a][threadIdx.x] = fmin(smin[a][threadIdx.x], smin[a][threadIdx.x + w]);
+          smax[a][threadIdx.x] = fmax(smax[a][threadIdx.x], smax[a][threadIdx.x + w]);
+        }
+      __syncthreads();
+    }
+  };
+  reduce();
+  if (threadIdx.x == 0) {
+    for (int a = 0; a < 3; ++a) {
+      __stcg(partial + 6 * blockIdx.x + a, smin[a][0]);
+      __stcg(partial + 6 * blockIdx.x + 3 + a, smax[a][0]);
+    }
+    __threadfence();
+    last = atomicAdd(&S->tickets, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int a = 0; a < 3; ++a) {
-        smin[a][threadIdx.x] = fmin(smin[a][threadIdx.x], smin[a][threadIdx.x + w]);
-        smax[a][threadIdx.x] = fmax(smax[a][threadIdx.x], smax[a][threadIdx.x + w]);
-      }
-    __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int a = 0; a < 3; ++a) {
+    mn[a] = INFINITY;
+    mx[a] = -INFINITY;
   }
-  if (threadIdx.x == 0)
+  for (int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
     for (int a = 0; a < 3; ++a) {
-      partial[6 * blockIdx.x + a] = smin[a][0];
-      partial[6 * blockIdx.x + 3 + a] = smax[a][0];
+      mn[a] = fmin(mn[a], __ldcg(partial + 6 * b + a));
+      mx[a] = fmax(mx[a], __ldcg(partial + 6 * b + 3 + a));
     }
+  reduce();
+  if (threadIdx.x != 0) return;
+  double lo[3] = {lo0, lo1, lo2}, size = box_size;
+  if (explicit_box) {
+    for (int a = 0; a < 3; ++a)
+      if (N > 0 && (smin[a][0] < lo[a] || smax[a][0] > lo[a] + box_size))
+        atomicOr(status, kStatusOutsideBox);
+  } else {
+    double ext = 0.0;
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = N > 0 ? smin[a][0] : 0.0;
+      if (N > 0) ext = fmax(ext, smax[a][0] - smin[a][0]);
+    }
+    size = ext > 0.0 ? ext : 1.0;
+  }
+  for (int a = 0; a < 3; ++a) S->lo[a] = lo[a];
+  S->size = size;
+  const unsigned long long g = atomicAdd(&S->n_gas, 0ull);
+  S->h_default = float(cbrt(size * size * size / double(g ? g : 1ull)));
 }
 
 // Sec. 2.3: normalise in FP64 and interleave the 21-bit cell indices,
@@ -326,15 +542,30 @@ __device__ inline uint64_t spread3(uint64_t v) {
   return v;
 }
 
-__global__ void k_morton(const double* __restrict__ pos, int64_t N, double lo0, double lo1,
-                         double lo2, double size, uint64_t* __restrict__ keys,
+// (x - lo) / size, exactly as the division rounds it: a product where 1 / size
+// is a power of two (then both are exact).
+__device__ __forceinline__ double normalised(double x, double lo, double size, double inv,
+                                             bool exact_inv) {
+  const double d = __dsub_rn(x, lo);
+  return exact_inv ? d * inv : __ddiv_rn(d, size);
+}
+__device__ __forceinline__ bool power_of_two(double size) {
+  const long long bits = __double_as_longlong(size);
+  const int e = int((bits >> 52) & 0x7ff);
+  return (bits & 0xfffffffffffffll) == 0 && e > 1 && e < 0x7fd;
+}
+
+__global__ void k_morton(const double* __restrict__ pos, int64_t N,
+                         const BuildState* __restrict__ S, uint64_t* __restrict__ keys,
                          int* __restrict__ vals) {
   int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (i >= N) return;
-  const double lo[3] = {lo0, lo1, lo2};
+  const double lo[3] = {S->lo[0], S->lo[1], S->lo[2]}, size = S->size;
+  const bool p2 = power_of_two(size);
+  const double inv = p2 ? 1.0 / size : 0.0;
   uint64_t k[3];
   for (int a = 0; a < 3; ++a) {
-    double u = __ddiv_rn(__dsub_rn(pos[3 * i + a], lo[a]), size);
+    double u = normalised(pos[3 * i + a], lo[a], size, inv, p2);
     double f = floor(__dmul_rn(u, 2097152.0));
     f = fmin(fmax(f, 0.0), 2097151.0);
     k[a] = uint64_t(f);
@@ -347,20 +578,21 @@ __global__ void k_morton(const double* __restrict__ pos, int64_t N, double lo0, 
 __global__ void k_gather_elements(const double* __restrict__ pos, const float* __restrict__ mass,
                                   const float* __restrict__ kappa, const float* __restrict__ lum,
                                   const float* __restrict__ h, const int* __restrict__ perm,
-                                  int64_t N, int nb, int nbp, double lo0, double lo1, double lo2,
-                                  double size, float h_default, int* __restrict__ inv,
+                                  int64_t N, int nb, int nbp, BuildState* __restrict__ S,
+                                  int* __restrict__ inv,
                                   double* __restrict__ pos64, float4* __restrict__ pos32,
                                   float* __restrict__ Lelem, float* __restrict__ km,
-                                  float* __restrict__ hn, float* __restrict__ ms,
-                                  int* __restrict__ luminous) {
+                                  float* __restrict__ hn, float* __restrict__ ms) {
   int64_t s = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (s >= N) return;
   int i = perm[s];
   inv[i] = int(s);
-  const double lo[3] = {lo0, lo1, lo2};
+  const double lo[3] = {S->lo[0], S->lo[1], S->lo[2]}, size = S->size;
+  const bool p2 = power_of_two(size);
+  const double isize = p2 ? 1.0 / size : 0.0;
   double u[3];
   for (int a = 0; a < 3; ++a) {
-    u[a] = __ddiv_rn(__dsub_rn(pos[3 * int64_t(i) + a], lo[a]), size);
+    u[a] = normalised(pos[3 * int64_t(i) + a], lo[a], size, isize, p2);
     pos64[3 * s + a] = u[a];
   }
   double lt = 0.0;
@@ -372,72 +604,106 @@ __global__ void k_gather_elements(const double* __restrict__ pos, const float* _
     lt = __dadd_rn(lt, double(l));
   }
   pos32[s] = make_float4(float(u[0]), float(u[1]), float(u[2]), float(lt));
-  float hh = h ? h[i] : h_default;
-  hn[s] = float(double(hh) / size);
+  const double hh = double(h ? h[i] : S->h_default);
+  hn[s] = float(p2 ? hh * isize : hh / size);
   ms[s] = mass[i];
   const unsigned lit = __ballot_sync(__activemask(), lt > 0.0);
-  if (lt > 0.0 && (lit & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(luminous, __popc(lit));
+  if (lt > 0.0 && (lit & ((1u << (threadIdx.x & 31)) - 1u)) == 0u)
+    atomicAdd(&S->n_luminous, __popc(lit));
 }
 
 // ---------------------------------------------------------------------------
-// Level-by-level bisection.
-__global__ void k_split_mark(const uint64_t* __restrict__ keys, int64_t lb, int64_t le, int bucket,
-                             const int* __restrict__ depth, const int* __restrict__ first,
-                             const int* __restrict__ count, int* __restrict__ flag,
-                             int* __restrict__ mid) {
-  int64_t q = lb + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q >= le) return;
-  int d = depth[q], c = count[q], f = first[q];
-  bool split = c > bucket && d < kMaxDepth;
-  flag[q - lb] = split ? 1 : 0;
-  if (!split) return;
+// Level-by-level bisection and the bottom-up aggregates.  A launch per level,
+// with the host reading each level's size, cost more than the work (33k
+// elements: 80 launches and 13 synchronisations; now 3 and none).
+// Topology, one cooperative launch: block 0 alone while levels are small (block barriers
+// only); from then on every block takes a chunk of consecutive nodes of the
+// level, counts its splits, and after a grid barrier places its children
+// behind those of the blocks before it.  A node splits while it holds more
+// than `bucket` elements; nodes are numbered by depth, by prefix within a
+// depth.  Aggregates: all leaves at once, then in one cooperative launch the
+// internal nodes, deepest depth first (their children are done); runs of small
+// depths stay in block 0.  Values another block wrote are read past the L1.
+struct TreeArgs {
+  const uint64_t* keys;
+  int64_t N;
+  int bucket, nb, nbp;
+  int cap;            // nodes the arrays hold
+  uint64_t* prefix;
+  int* depth;
+  int* first;
+  int* count;
+  int* child;
+  int* parent;
+  int* int_index;
+  int* mid;           // [cap] a splitting node's first upper element, else -1
+  int* block_count;   // [blocks]
+  const double* pos64;
+  const float* Lelem;
+  const int* perm;
+  const float* kappa;
+  const float* mass;
+  double* L64;        // [cap][4]
+  double* cs64;       // [cap][4] sum Lt x, sum Lt
+  uint32_t* flags;    // [cap]
+  float* Lnode;
+  float4* csrc;
+  double* c64;
+  double* B64;
+  float* alpha_leaf;
+  uint32_t* lmask;
+  NodeW* nodes;
+  BuildState* S;
+  uint32_t* status;
+};
+constexpr int kTreeThreads = 512;
+constexpr int kSmallLevel = 1024;  // nodes of a level that block 0 does alone
+
+// The element that starts the upper half of a node, or -1 when it is a leaf.
+__device__ __forceinline__ int split_at(const TreeArgs& A, int d, int f, int c) {
+  if (!(c > A.bucket && d < kMaxDepth)) return -1;
   // keys in [f, f+c) share the node's prefix, so bit (62 - d) is monotone
   const int bit = kMaxDepth - 1 - d;
   int lo = f, hi = f + c;  // first index with the bit set
   while (lo < hi) {
-    int m = lo + ((hi - lo) >> 1);
-    if ((keys[m] >> bit) & 1ull) hi = m; else lo = m + 1;
+    const int m = lo + ((hi - lo) >> 1);
+    if ((A.keys[m] >> bit) & 1ull) hi = m; else lo = m + 1;
   }
-  mid[q - lb] = lo;
+  return lo;
 }
 
-__global__ void k_split_emit(int64_t lb, int64_t le, int64_t child_base,
-                             const int* __restrict__ flag_scan, const int* __restrict__ flag,
-                             const int* __restrict__ mid, uint64_t* __restrict__ prefix,
-                             int* __restrict__ depth, int* __restrict__ first,
-                             int* __restrict__ count, int* __restrict__ child,
-                             int* __restrict__ parent) {
-  int64_t q = lb + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q >= le) return;
-  int64_t j = q - lb;
-  if (!flag[j]) {
-    child[q] = -1;
-    return;
+__device__ __forceinline__ void emit_halves(const TreeArgs& A, int q, int c, int d, int f, int n,
+                                            int m) {
+  const uint64_t p = __ldcg(A.prefix + q);
+  A.child[q] = c;
+  A.prefix[c] = p;
+  A.prefix[c + 1] = p | (1ull << (kMaxDepth - 1 - d));
+  A.depth[c] = A.depth[c + 1] = d + 1;
+  A.first[c] = f;
+  A.count[c] = m - f;
+  A.first[c + 1] = m;
+  A.count[c + 1] = f + n - m;
+  A.parent[c] = A.parent[c + 1] = q;
+}
+
+// Running rank of the set flags of a block, in thread order: this thread's
+// rank in the tile, the tile's total to `total`.
+__device__ __forceinline__ int tile_rank(bool flag, int& total) {
+  __shared__ int warp_sum[kTreeThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned m = __ballot_sync(0xffffffffu, flag);
+  __syncthreads();
+  if (lane == 0) warp_sum[warp] = __popc(m);
+  __syncthreads();
+  int before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kTreeThreads / 32; ++w) {
+    const int c = warp_sum[w];
+    before += w < warp ? c : 0;
+    all += c;
   }
-  int64_t c = child_base + 2 * int64_t(flag_scan[j]);
-  child[q] = int(c);
-  int d = depth[q], f = first[q], n = count[q], m = mid[j];
-  uint64_t p = prefix[q];
-  const int bit = kMaxDepth - 1 - d;
-  prefix[c] = p;
-  prefix[c + 1] = p | (1ull << bit);
-  depth[c] = depth[c + 1] = d + 1;
-  first[c] = f;
-  count[c] = m - f;
-  first[c + 1] = m;
-  count[c + 1] = f + n - m;
-  parent[c] = parent[c + 1] = int(q);
-  child[c] = child[c + 1] = -1;
-}
-
-__global__ void k_leaf_flags(const int* __restrict__ child, int64_t n, int* __restrict__ out) {
-  int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q < n) out[q] = child[q] >= 0 ? 1 : 0;
-}
-
-__global__ void k_finish_int_index(const int* __restrict__ child, int64_t n, int* __restrict__ idx) {
-  int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q < n && child[q] < 0) idx[q] = -1;
+  total = all;
+  return before + __popc(m & ((1u << lane) - 1u));
 }
 
 // ---------------------------------------------------------------------------
@@ -451,62 +717,53 @@ __device__ inline void node_box_norm(uint64_t prefix, int depth, double lo[3], d
   }
 }
 
-__global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, double inv_size2,
-                                  const uint64_t* __restrict__ prefix, const int* __restrict__ depth,
-                                  const int* __restrict__ first, const int* __restrict__ count,
-                                  const int* __restrict__ child, const int* __restrict__ int_index,
-                                  const double* __restrict__ pos64, const float* __restrict__ Lelem,
-                                  const int* __restrict__ perm, const float* __restrict__ kappa,
-                                  const float* __restrict__ mass, double* __restrict__ L64,
-                                  double* __restrict__ cs64 /*[n][4]: sum Lt x, sum Lt*/,
-                                  uint32_t* __restrict__ flags64, float* __restrict__ Lnode,
-                                  float4* __restrict__ csrc, double* __restrict__ c64,
-                                  double* __restrict__ B64, float* __restrict__ alpha_leaf,
-                                  uint32_t* __restrict__ lmask, NodeW* __restrict__ nodes) {
-  int64_t q = lb + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q >= le) return;
-  const int d = depth[q];
+__device__ void aggregate_node(const TreeArgs& A, int64_t q, bool leaf, double inv_size2) {
+  const int nb = A.nb, nbp = A.nbp;
+  const int d = __ldcg(A.depth + q);
   double lo[3], ext[3];
-  node_box_norm(prefix[q], d, lo, ext);
-  const int c = child[q];
+  node_box_norm(__ldcg(A.prefix + q), d, lo, ext);
+  const int c = leaf ? -1 : __ldcg(A.child + q);
   double cs[4] = {0, 0, 0, 0};
-  uint32_t has = 0, lit = 0;
+  uint32_t has = 0, lit = 0, half0 = 0, half1 = 0;
   if (c < 0) {
-    const int f = first[q], n = count[q];
+    const int f = __ldcg(A.first + q), n = __ldcg(A.count + q);
     double Lb[4] = {0, 0, 0, 0}, kmb[4] = {0, 0, 0, 0};
     for (int e = f; e < f + n; ++e) {
       double lt = 0.0;
       for (int b = 0; b < nb; ++b) {
-        double l = double(Lelem[int64_t(e) * nbp + b]);
+        double l = double(A.Lelem[int64_t(e) * nbp + b]);
         Lb[b] = __dadd_rn(Lb[b], l);
         lt = __dadd_rn(lt, l);
         // kappa and m are float32: their FP64 product is exact
-        const int i = perm[e];
-        kmb[b] = __dadd_rn(kmb[b], __dmul_rn(double(kappa[int64_t(i) * nb + b]), double(mass[i])));
+        const int i = A.perm[e];
+        kmb[b] = __dadd_rn(kmb[b], __dmul_rn(double(A.kappa[int64_t(i) * nb + b]), double(A.mass[i])));
       }
-      for (int a = 0; a < 3; ++a) cs[a] = __dadd_rn(cs[a], __dmul_rn(lt, pos64[3 * int64_t(e) + a]));
+      for (int a = 0; a < 3; ++a) cs[a] = __dadd_rn(cs[a], __dmul_rn(lt, A.pos64[3 * int64_t(e) + a]));
       cs[3] = __dadd_rn(cs[3], lt);
       if (lt > 0.0 && e - f < 32) lit |= 1u << (e - f);
     }
     const double V = ext[0] * ext[1] * ext[2];  // exact powers of two
     for (int b = 0; b < nbp; ++b) {
       double al = b < nb ? kmb[b] / V * inv_size2 : 0.0;
-      alpha_leaf[q * nbp + b] = float(al);
+      A.alpha_leaf[q * nbp + b] = float(al);
       if (al > 0.0) has |= kMetaHasAlpha;
     }
-    for (int b = 0; b < 4; ++b) L64[q * 4 + b] = b < nb ? Lb[b] : 0.0;
+    for (int b = 0; b < 4; ++b) __stcg(A.L64 + q * 4 + b, b < nb ? Lb[b] : 0.0);
   } else {
-    for (int b = 0; b < 4; ++b) L64[q * 4 + b] = __dadd_rn(L64[int64_t(c) * 4 + b], L64[int64_t(c + 1) * 4 + b]);
-    for (int a = 0; a < 4; ++a) cs[a] = __dadd_rn(cs64[int64_t(c) * 4 + a], cs64[int64_t(c + 1) * 4 + a]);
-    has = (flags64[c] | flags64[c + 1]) & kMetaHasAlpha;
-    for (int b = 0; b < nbp; ++b) alpha_leaf[q * nbp + b] = 0.0f;
+    for (int b = 0; b < 4; ++b)
+      __stcg(A.L64 + q * 4 + b, __dadd_rn(__ldcg(A.L64 + int64_t(c) * 4 + b), __ldcg(A.L64 + int64_t(c + 1) * 4 + b)));
+    for (int a = 0; a < 4; ++a) cs[a] = __dadd_rn(__ldcg(A.cs64 + int64_t(c) * 4 + a), __ldcg(A.cs64 + int64_t(c + 1) * 4 + a));
+    half0 = __ldcg(A.flags + c);
+    half1 = __ldcg(A.flags + c + 1);
+    has = (half0 | half1) & kMetaHasAlpha;
+    for (int b = 0; b < nbp; ++b) A.alpha_leaf[q * nbp + b] = 0.0f;
   }
-  for (int a = 0; a < 4; ++a) cs64[q * 4 + a] = cs[a];
+  for (int a = 0; a < 4; ++a) __stcg(A.cs64 + q * 4 + a, cs[a]);
   double cc[3];
   for (int a = 0; a < 3; ++a) cc[a] = cs[3] > 0.0 ? cs[a] / cs[3] : lo[a] + 0.5 * ext[a];
   if (cs[3] > 0.0) has |= kMetaHasL;
-  flags64[q] = has;
-  lmask[q] = lit;
+  __stcg(A.flags + q, has);
+  A.lmask[q] = lit;
   // B: farthest box corner from the centre of luminosity (Sec. 2.5.2)
   double B2 = 0.0;
   for (int corner = 0; corner < 8; ++corner) {
@@ -519,74 +776,234 @@ __global__ void k_aggregate_level(int64_t lb, int64_t le, int nb, int nbp, doubl
     B2 = fmax(B2, r2);
   }
   double B = sqrt(B2);
-  for (int a = 0; a < 3; ++a) c64[3 * q + a] = cc[a];
-  B64[q] = B;
-  for (int b = 0; b < nbp; ++b) Lnode[q * nbp + b] = float(L64[q * 4 + b]);
-  csrc[q] = make_float4(float(cc[0]), float(cc[1]), float(cc[2]), float(cs[3]));
+  for (int a = 0; a < 3; ++a) A.c64[3 * q + a] = cc[a];
+  A.B64[q] = B;
+  for (int b = 0; b < nbp; ++b) A.Lnode[q * nbp + b] = float(__ldcg(A.L64 + q * 4 + b));
+  A.csrc[q] = make_float4(float(cc[0]), float(cc[1]), float(cc[2]), float(cs[3]));
   NodeW w;
   w.lo[0] = float(lo[0]);
   w.lo[1] = float(lo[1]);
   w.lo[2] = float(lo[2]);
   w.B = float(B);
   w.child = c;
-  w.aux = c < 0 ? first[q] : int_index[q];
-  w.count = count[q];
+  w.aux = c < 0 ? __ldcg(A.first + q) : __ldcg(A.int_index + q);
+  w.count = __ldcg(A.count + q);
   w.meta = uint32_t(d) | (uint32_t(d % 3) << kMetaAxisShift) | (c < 0 ? kMetaLeaf : 0u) | has;
   if (c >= 0) {
-    if (flags64[c] & kMetaHasAlpha) w.meta |= kMetaChild0Alpha;
-    if (flags64[c + 1] & kMetaHasAlpha) w.meta |= kMetaChild1Alpha;
+    if (half0 & kMetaHasAlpha) w.meta |= kMetaChild0Alpha;
+    if (half1 & kMetaHasAlpha) w.meta |= kMetaChild1Alpha;
   }
-  nodes[q] = w;
+  A.nodes[q] = w;
 }
 
-// ---------------------------------------------------------------------------
-static int grow(Tree* t, int64_t need, int64_t& cap, cudaStream_t st) {
-  if (need <= cap) return TREVR2_OK;
-  int64_t ncap = std::max<int64_t>(cap, 1024);
-  while (ncap < need) ncap *= 2;
-  auto regrow = [&](auto*& p) -> int {
-    using T = std::remove_pointer_t<std::remove_reference_t<decltype(p)>>;
-    T* q = nullptr;
-    int rc = dalloc(&q, ncap, st);
-    if (rc) return rc;
-    if (p) {
-      cudaError_t e = cudaMemcpyAsync(q, p, cap * sizeof(T), cudaMemcpyDeviceToDevice, st);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync");
-      dfree(p, st);
+__global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_constant__ TreeArgs A) {
+  BuildState* S = A.S;
+  const int blocks = gridDim.x, t = threadIdx.x;
+  __shared__ int s_levels, s_lb, s_le, s_int, s_need;
+  int lb = 0, le = 1, level = 0, n_int = 0;
+  int need = 0;
+  if (blockIdx.x == 0) {
+    if (t == 0) {
+      A.prefix[0] = 0;
+      A.depth[0] = 0;
+      A.first[0] = 0;
+      A.count[0] = int(A.N);
+      A.parent[0] = -1;
+      S->level_begin[0] = 0;
     }
-    p = q;
-    return TREVR2_OK;
-  };
-  T2_CHECK(regrow(t->prefix));
-  T2_CHECK(regrow(t->depth));
-  T2_CHECK(regrow(t->first));
-  T2_CHECK(regrow(t->count));
-  T2_CHECK(regrow(t->child));
-  T2_CHECK(regrow(t->parent));
-  cap = ncap;
+    __syncthreads();
+    // small levels, one after another
+    while (le - lb <= kSmallLevel) {
+      int done = 0;  // splits so far in this level
+      for (int q0 = lb; q0 < le; q0 += kTreeThreads) {
+        const int q = q0 + t;
+        int m = -1, d = 0, f = 0, c = 0;
+        if (q < le) {
+          d = level;
+          f = __ldcg(A.first + q);
+          c = __ldcg(A.count + q);
+          m = split_at(A, d, f, c);
+        }
+        int tile = 0;
+        const int rank = done + tile_rank(m >= 0, tile);
+        if (le + 2 * (done + tile) > A.cap) {
+          need = le + 2 * (le - lb);
+          break;
+        }
+        if (m >= 0) {
+          emit_halves(A, q, le + 2 * rank, d, f, c, m);
+          A.int_index[q] = n_int + rank;
+        } else if (q < le) {
+          A.child[q] = -1;
+          A.int_index[q] = -1;
+        }
+        done += tile;
+      }
+      __syncthreads();  // the children are visible to this block
+      if (need) break;
+      if (t == 0) S->level_begin[level + 1] = le;
+      n_int += done;
+      lb = le;
+      le += 2 * done;
+      ++level;
+      if (done == 0) break;
+    }
+    if (t == 0) {
+      S->levels = level;
+      S->n_internal = n_int;
+      S->n_nodes = le;
+      S->need = need;
+      A.block_count[0] = lb;  // what the other blocks go on from
+      A.block_count[1] = le;
+    }
+  }
+  if (!grid_barrier(&S->bar, blocks, A.status)) return;
+  if (t == 0) {
+    s_levels = __ldcg(&S->levels);
+    s_int = __ldcg(&S->n_internal);
+    s_need = __ldcg(&S->need);
+    s_lb = __ldcg(A.block_count);
+    s_le = __ldcg(A.block_count + 1);
+  }
+  __syncthreads();
+  level = s_levels;
+  n_int = s_int;
+  need = s_need;
+  lb = s_lb;
+  le = s_le;
+  if (need) return;
+  if (!grid_barrier(&S->bar, blocks, A.status)) return;  // block_count is free again
+  // larger levels, all blocks
+  while (le > lb) {
+    const int per = (le - lb + blocks - 1) / blocks;
+    const int c0 = min(le, lb + int(blockIdx.x) * per), c1 = min(le, c0 + per);
+    int mine = 0;
+    for (int q0 = c0; q0 < c1; q0 += kTreeThreads) {
+      const int q = q0 + t;
+      int m = -1;
+      if (q < c1) {
+        m = split_at(A, level, __ldcg(A.first + q), __ldcg(A.count + q));
+        A.mid[q] = m;
+      }
+      mine += __syncthreads_count(m >= 0);
+    }
+    if (t == 0) __stcg(A.block_count + blockIdx.x, mine);
+    if (!grid_barrier(&S->bar, blocks, A.status)) return;
+    int before = 0, all = 0;
+    {
+      __shared__ int s_before, s_all;
+      if (t < 32) {
+        for (int b = t; b < blocks; b += 32) {
+          const int c = __ldcg(A.block_count + b);
+          all += c;
+          if (b < int(blockIdx.x)) before += c;
+        }
+        all = __reduce_add_sync(0xffffffffu, all);
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (t == 0) {
+          s_before = before;
+          s_all = all;
+        }
+      }
+      __syncthreads();
+      before = s_before;
+      all = s_all;
+    }
+    if (int64_t(le) + 2 * int64_t(all) > A.cap) {
+      if (blockIdx.x == 0 && t == 0)
+        S->need = int(min(int64_t(INT32_MAX), int64_t(le) + 2 * int64_t(all)));
+      return;
+    }
+    for (int q0 = c0; q0 < c1; q0 += kTreeThreads) {
+      const int q = q0 + t;
+      const int m = q < c1 ? A.mid[q] : -1;
+      int tile = 0;
+      const int rank = before + tile_rank(m >= 0, tile);
+      if (m >= 0) {
+        emit_halves(A, q, le + 2 * rank, level, __ldcg(A.first + q), __ldcg(A.count + q), m);
+        A.int_index[q] = n_int + rank;
+      } else if (q < c1) {
+        A.child[q] = -1;
+        A.int_index[q] = -1;
+      }
+      before += tile;
+    }
+    if (blockIdx.x == 0 && t == 0) S->level_begin[level + 1] = le;
+    n_int += all;
+    lb = le;
+    le += 2 * all;
+    ++level;
+    if (!grid_barrier(&S->bar, blocks, A.status)) return;
+    if (all == 0) break;
+  }
+  if (blockIdx.x == 0 && t == 0) {
+    S->levels = level;
+    S->n_internal = n_int;
+    S->n_nodes = le;
+  }
+}
+
+// The leaves' aggregates (the grid covers the nodes' arrays; how many there
+// are is known on the device).
+__global__ void __launch_bounds__(128) k_aggregate_leaves(const __grid_constant__ TreeArgs A) {
+  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (A.S->need || q >= A.S->n_nodes || A.child[q] >= 0) return;
+  const double size = A.S->size;
+  aggregate_node(A, q, true, 1.0 / (size * size));
+}
+
+__global__ void __launch_bounds__(kTreeThreads, 2) k_aggregate_inner(const __grid_constant__ TreeArgs A) {
+  BuildState* S = A.S;
+  if (S->need) return;
+  const int blocks = gridDim.x, t = threadIdx.x;
+  __shared__ int s_begin[kMaxLevels + 1];
+  const int level = S->levels;
+  for (int i = t; i < level; i += kTreeThreads) s_begin[i] = S->level_begin[i];
+  if (t == 0) s_begin[level] = S->n_nodes;
+  __syncthreads();
+  const double size = S->size, inv_size2 = 1.0 / (size * size);
+  const int64_t stride = int64_t(blocks) * kTreeThreads, at = int64_t(blockIdx.x) * kTreeThreads + t;
+  bool together = false;  // whether the depth below was done by all blocks
+  for (int d = level - 2; d >= 0; --d) {
+    const int b0 = s_begin[d], b1 = s_begin[d + 1];
+    const bool small = b1 - b0 <= kTreeThreads;
+    if (together || (!small && d < level - 2)) {
+      if (!grid_barrier(&S->bar, blocks, A.status)) return;
+    } else {
+      __syncthreads();
+    }
+    together = !small;
+    if (small) {
+      if (blockIdx.x == 0 && t < b1 - b0 && __ldcg(A.child + b0 + t) >= 0)
+        aggregate_node(A, b0 + t, false, inv_size2);
+    } else {
+      for (int64_t q = b0 + at; q < b1; q += stride)
+        if (__ldcg(A.child + q) >= 0) aggregate_node(A, q, false, inv_size2);
+    }
+  }
+}
+
+// The node arrays for `cap` nodes.
+static int alloc_nodes(Tree* t, int64_t cap, cudaStream_t st) {
+  const int nbp = t->nbp;
+  T2_CHECK(dalloc(&t->prefix, cap, st));
+  T2_CHECK(dalloc(&t->depth, cap, st));
+  T2_CHECK(dalloc(&t->first, cap, st));
+  T2_CHECK(dalloc(&t->count, cap, st));
+  T2_CHECK(dalloc(&t->child, cap, st));
+  T2_CHECK(dalloc(&t->parent, cap, st));
+  T2_CHECK(dalloc(&t->int_index, cap, st));
+  T2_CHECK(dalloc(&t->nodes, cap, st));
+  T2_CHECK(dalloc(&t->Lnode, cap * nbp, st));
+  T2_CHECK(dalloc(&t->csrc, cap, st));
+  T2_CHECK(dalloc(&t->c64, 3 * cap, st));
+  T2_CHECK(dalloc(&t->B64, cap, st));
+  T2_CHECK(dalloc(&t->alpha_leaf, cap * nbp, st));
+  T2_CHECK(dalloc(&t->lmask, cap, st));
   return TREVR2_OK;
 }
 
-__global__ void k_init_root(int64_t N, uint64_t* prefix, int* depth, int* first, int* count,
-                            int* child, int* parent) {
-  prefix[0] = 0;
-  depth[0] = 0;
-  first[0] = 0;
-  count[0] = int(N);
-  child[0] = -1;
-  parent[0] = -1;
-}
-
-static void free_tree(Tree* t, cudaStream_t st) {
-  dfree(t->keys, st);
-  dfree(t->perm, st);
-  dfree(t->inv, st);
-  dfree(t->pos64, st);
-  dfree(t->pos32, st);
-  dfree(t->Lelem, st);
-  dfree(t->km, st);
-  dfree(t->mass, st);
-  dfree(t->hn, st);
+static void free_nodes(Tree* t, cudaStream_t st) {
   dfree(t->prefix, st);
   dfree(t->depth, st);
   dfree(t->first, st);
@@ -601,6 +1018,19 @@ static void free_tree(Tree* t, cudaStream_t st) {
   dfree(t->B64, st);
   dfree(t->alpha_leaf, st);
   dfree(t->lmask, st);
+}
+
+static void free_tree(Tree* t, cudaStream_t st) {
+  dfree(t->keys, st);
+  dfree(t->perm, st);
+  dfree(t->inv, st);
+  dfree(t->pos64, st);
+  dfree(t->pos32, st);
+  dfree(t->Lelem, st);
+  dfree(t->km, st);
+  dfree(t->mass, st);
+  dfree(t->hn, st);
+  free_nodes(t, st);
   dfree(t->dtau, st);
   dfree(t->nodes_refined, st);
   for (Table& tb : t->tables) {
@@ -626,87 +1056,43 @@ static inline unsigned blocks_for(int64_t n, int threads) {
   return unsigned((n + threads - 1) / threads);
 }
 
+// Everything up to the one read-back is enqueued without waiting: the inputs'
+// check, the root cube, keys, sort, topology and aggregates run whatever the
+// inputs hold (keys are clamped to the cube), and the host looks at the status
+// and the sizes at the end.
 static int build_impl(Tree* t, const double* pos, const float* mass, const float* kappa,
                       const float* lum, const float* h, const double* box_lo, double box_size,
                       cudaStream_t st) {
   const int64_t N = t->N;
   const int nb = t->nb, nbp = t->nbp;
-  T2_CHECK(dalloc(&t->status, 1, st));
+  T2_CHECK(dalloc(&t->status, 2, st));  // status word, grid barrier of the tables' kernel
   T2_CHECK(dalloc(&t->counter, 1, st));
   T2_CUDA(cudaMemsetAsync(t->status, 0, sizeof(uint32_t), st));
 
-  // 1. validation and bounding box
-  const int vthreads = 256;
-  const int vblocks = int(std::min<int64_t>(std::max<int64_t>(blocks_for(N, vthreads), 1), 1024));
+  // 1. validation and root cube
+  const int vblocks = int(std::min<int64_t>(std::max<int64_t>(blocks_for(N, 256), 1), 1024));
   DeviceTemp<double> partial(st);
+  DeviceTemp<BuildState> state(st);
   T2_CHECK(dalloc(&partial.p, size_t(vblocks) * 6, st));
-  if (N > 0)
-    k_validate<<<vblocks, vthreads, 0, st>>>(pos, mass, kappa, lum, h, N, nb, partial.p, t->status); note_launch();
-  std::vector<double> hpart(size_t(vblocks) * 6);
-  uint32_t hstatus = 0;
-  if (N > 0) {
-    T2_CUDA(cudaMemcpyAsync(hpart.data(), partial.p, hpart.size() * sizeof(double),
-                            cudaMemcpyDeviceToHost, st));
-    T2_CUDA(cudaMemcpyAsync(&hstatus, t->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-  }
-  T2_CUDA(cudaStreamSynchronize(st));
-  dfree(partial.p, st);
-  if (hstatus & kStatusBadInput) {
-    set_error("trevr2_build: non-finite position, or negative/non-finite mass, kappa, lum or h");
-    return TREVR2_EINVAL;
-  }
-  double mn[3] = {0, 0, 0}, mx[3] = {0, 0, 0};
-  if (N > 0) {
-    for (int a = 0; a < 3; ++a) {
-      mn[a] = INFINITY;
-      mx[a] = -INFINITY;
-    }
-    for (int b = 0; b < vblocks; ++b)
-      for (int a = 0; a < 3; ++a) {
-        mn[a] = std::min(mn[a], hpart[6 * b + a]);
-        mx[a] = std::max(mx[a], hpart[6 * b + 3 + a]);
-      }
-  }
-  if (box_lo && box_size > 0.0) {
-    for (int a = 0; a < 3; ++a) t->lo[a] = box_lo[a];
-    t->size = box_size;
-    if (N > 0)
-      for (int a = 0; a < 3; ++a)
-        if (mn[a] < box_lo[a] || mx[a] > box_lo[a] + box_size) {
-          set_error("trevr2_build: a position lies outside the given root cube");
-          return TREVR2_EINVAL;
-        }
-  } else {
-    double ext = 0.0;
-    for (int a = 0; a < 3; ++a) {
-      t->lo[a] = mn[a];
-      ext = std::max(ext, mx[a] - mn[a]);
-    }
-    t->size = ext > 0.0 ? ext : 1.0;
-  }
+  T2_CHECK(dalloc(&state.p, 1, st));
+  T2_CUDA(cudaMemsetAsync(state.p, 0, sizeof(BuildState), st));
+  const bool explicit_box = box_lo && box_size > 0.0;
+  const double lo[3] = {explicit_box ? box_lo[0] : 0.0, explicit_box ? box_lo[1] : 0.0,
+                        explicit_box ? box_lo[2] : 0.0};
+  k_validate<<<vblocks, 256, 0, st>>>(pos, mass, kappa, lum, h, N, nb, explicit_box, lo[0], lo[1],
+                                      lo[2], box_size, partial.p, state.p, t->status);
+  note_launch();
 
   // 2. keys and stable sort
   T2_CHECK(dalloc(&t->keys, N, st));
   T2_CHECK(dalloc(&t->perm, N, st));
-  if (N > 0)
-    k_morton<<<blocks_for(N, 256), 256, 0, st>>>(pos, N, t->lo[0], t->lo[1], t->lo[2], t->size,
-                                                 t->keys, t->perm); note_launch();
-  T2_CHECK(radix_sort_u64_i32(t->keys, t->perm, N, st));
+  if (N > 0) {
+    k_morton<<<blocks_for(N, 256), 256, 0, st>>>(pos, N, state.p, t->keys, t->perm);
+    note_launch();
+  }
+  T2_CHECK(radix_sort_u64_i32(t->keys, t->perm, N, st, t->status));
 
   // 3. sorted element data
-  int64_t ngas = 0;  // h default: (V_root / N_gas)^(1/3), counted on the host only if needed
-  float h_default = 1.0f;
-  if (!h && N > 0) {
-    std::vector<float> hm(N);
-    T2_CUDA(cudaMemcpyAsync(hm.data(), mass, N * sizeof(float), cudaMemcpyDeviceToHost, st));
-    T2_CUDA(cudaStreamSynchronize(st));
-    for (float m : hm) ngas += m > 0.0f;
-    h_default = float(std::cbrt(t->size * t->size * t->size / double(std::max<int64_t>(ngas, 1))));
-  }
-  DeviceTemp<int> dtotal_t(st);  // a scan's total, the number of luminous elements
-  int*& dtotal = dtotal_t.p;
-  T2_CHECK(dalloc(&dtotal, 2, st));
-  T2_CUDA(cudaMemsetAsync(dtotal, 0, 2 * sizeof(int), st));
   T2_CHECK(dalloc(&t->inv, N, st));
   T2_CHECK(dalloc(&t->pos64, 3 * N, st));
   T2_CHECK(dalloc(&t->pos32, N, st));
@@ -714,106 +1100,104 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
   T2_CHECK(dalloc(&t->km, N * nbp, st));
   T2_CHECK(dalloc(&t->hn, N, st));
   T2_CHECK(dalloc(&t->mass, N, st));
-  if (N > 0)
-    k_gather_elements<<<blocks_for(N, 256), 256, 0, st>>>(
-        pos, mass, kappa, lum, h, t->perm, N, nb, nbp, t->lo[0], t->lo[1], t->lo[2], t->size,
-        h_default, t->inv, t->pos64, t->pos32, t->Lelem, t->km, t->hn, t->mass, dtotal + 1);
-  note_launch();
+  if (N > 0) {
+    k_gather_elements<<<blocks_for(N, 256), 256, 0, st>>>(pos, mass, kappa, lum, h, t->perm, N, nb,
+                                                          nbp, state.p, t->inv, t->pos64, t->pos32,
+                                                          t->Lelem, t->km, t->hn, t->mass);
+    note_launch();
+  }
 
-  // 4. bisection, one depth at a time
-  int64_t cap = 0;
-  T2_CHECK(grow(t, std::max<int64_t>(1024, 4 * (N / std::max(t->bucket, 1)) + 64), cap, st));
-  k_init_root<<<1, 1, 0, st>>>(N, t->prefix, t->depth, t->first, t->count, t->child, t->parent); note_launch();
-  DeviceTemp<int> flag_t(st), fscan_t(st), mid_t(st);
-  int*& flag = flag_t.p;
-  int*& fscan = fscan_t.p;
-  int*& mid = mid_t.p;
-  int64_t flag_cap = 1024;
-  T2_CHECK(dalloc(&flag, flag_cap, st));
-  T2_CHECK(dalloc(&fscan, flag_cap, st));
-  T2_CHECK(dalloc(&mid, flag_cap, st));
-  t->level_begin.assign(1, 0);
-  int64_t lb = 0, le = 1;
-  int level = 0;
+  // 4. bisection and aggregates, into arrays sized for a tree of evenly filled
+  // leaves; once more with larger ones when the tree has more nodes
+  BuildState S;
+  int64_t cap = std::min<int64_t>(std::max<int64_t>(1024, 4 * (N / std::max(t->bucket, 1)) + 64),
+                                  INT32_MAX);
   for (;;) {
-    const int64_t m = le - lb;
-    if (m > flag_cap) {
-      dfree(flag, st);
-      dfree(fscan, st);
-      dfree(mid, st);
-      while (flag_cap < m) flag_cap *= 2;
-      T2_CHECK(dalloc(&flag, flag_cap, st));
-      T2_CHECK(dalloc(&fscan, flag_cap, st));
-      T2_CHECK(dalloc(&mid, flag_cap, st));
-    }
-    k_split_mark<<<blocks_for(m, 256), 256, 0, st>>>(t->keys, lb, le, t->bucket, t->depth,
-                                                      t->first, t->count, flag, mid); note_launch();
-    T2_CUDA(cudaMemcpyAsync(fscan, flag, m * sizeof(int), cudaMemcpyDeviceToDevice, st));
-    T2_CHECK(scan_exclusive_i32(fscan, m, dtotal, st));
-    int total = 0;
-    T2_CUDA(cudaMemcpyAsync(&total, dtotal, sizeof(int), cudaMemcpyDeviceToHost, st));
+    T2_CHECK(alloc_nodes(t, cap, st));
+    DeviceTemp<double> sums(st);
+    DeviceTemp<int> ints(st);
+    T2_CHECK(dalloc(&sums.p, 8 * cap, st));
+    T2_CHECK(dalloc(&ints.p, 2 * cap + kMaxCoopBlocks, st));
+    TreeArgs A;
+    A.keys = t->keys;
+    A.N = N;
+    A.bucket = t->bucket;
+    A.nb = nb;
+    A.nbp = nbp;
+    A.cap = int(cap);
+    A.prefix = t->prefix;
+    A.depth = t->depth;
+    A.first = t->first;
+    A.count = t->count;
+    A.child = t->child;
+    A.parent = t->parent;
+    A.int_index = t->int_index;
+    A.mid = ints.p;
+    A.flags = reinterpret_cast<uint32_t*>(ints.p + cap);
+    A.block_count = ints.p + 2 * cap;
+    A.pos64 = t->pos64;
+    A.Lelem = t->Lelem;
+    A.perm = t->perm;
+    A.kappa = kappa;
+    A.mass = mass;
+    A.L64 = sums.p;
+    A.cs64 = sums.p + 4 * cap;
+    A.Lnode = t->Lnode;
+    A.csrc = t->csrc;
+    A.c64 = t->c64;
+    A.B64 = t->B64;
+    A.alpha_leaf = t->alpha_leaf;
+    A.lmask = t->lmask;
+    A.nodes = t->nodes;
+    A.S = state.p;
+    A.status = t->status;
+    int blocks = 0, blocks_inner = 0;
+    T2_CHECK(coop_blocks(cap, 2 * kTreeThreads, 1, &blocks));
+    T2_CHECK(coop_blocks(cap, kTreeThreads, 2, &blocks_inner));
+    void* args[] = {&A};
+    T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_build_tree),
+                                        dim3(unsigned(blocks)), dim3(kTreeThreads), args, 0, st));
+    note_launch();
+    k_aggregate_leaves<<<blocks_for(cap, 128), 128, 0, st>>>(A);
+    note_launch();
+    T2_CUDA(cudaMemsetAsync(&state.p->bar, 0, sizeof(uint32_t), st));
+    T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_aggregate_inner),
+                                        dim3(unsigned(blocks_inner)), dim3(kTreeThreads), args, 0, st));
+    note_launch();
+    uint32_t hstatus = 0;
+    T2_CUDA(cudaMemcpyAsync(&S, state.p, sizeof(S), cudaMemcpyDeviceToHost, st));
+    T2_CUDA(cudaMemcpyAsync(&hstatus, t->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     T2_CUDA(cudaStreamSynchronize(st));
-    if (le + 2 * int64_t(total) > (int64_t(1) << 31) - 1) {
+    if (hstatus & kStatusBadInput) {
+      set_error("trevr2_build: non-finite position, or negative/non-finite mass, kappa, lum or h");
+      return TREVR2_EINVAL;
+    }
+    if (hstatus & kStatusOutsideBox) {
+      set_error("trevr2_build: a position lies outside the given root cube");
+      return TREVR2_EINVAL;
+    }
+    if (hstatus) {
+      set_error("trevr2_build: a grid barrier gave up waiting (device status 0x%x)", hstatus);
+      return TREVR2_ETIMEOUT;
+    }
+    if (S.need == 0) break;
+    if (cap >= INT32_MAX) {
       set_error("trevr2_build: more than 2^31 nodes");
       return TREVR2_EUNSUPPORTED;
     }
-    T2_CHECK(grow(t, le + 2 * int64_t(total), cap, st));
-    k_split_emit<<<blocks_for(m, 256), 256, 0, st>>>(lb, le, le, fscan, flag, mid, t->prefix,
-                                                      t->depth, t->first, t->count, t->child,
-                                                      t->parent); note_launch();
-    t->level_begin.push_back(le);
-    if (total == 0) break;
-    lb = le;
-    le += 2 * int64_t(total);
-    ++level;
+    free_nodes(t, st);
+    cap = std::min<int64_t>(std::max<int64_t>(2 * cap, S.need), INT32_MAX);
+    T2_CUDA(cudaMemsetAsync(&state.p->bar, 0, sizeof(uint32_t), st));
+    T2_CUDA(cudaMemsetAsync(&state.p->need, 0, sizeof(int), st));
   }
-  t->n_nodes = le;
-  t->max_depth = level;
-  dfree(flag, st);
-  dfree(fscan, st);
-  dfree(mid, st);
-
-  // internal-node rows of the alpha tables
-  const int64_t n = t->n_nodes;
-  T2_CHECK(dalloc(&t->int_index, n, st));
-  k_leaf_flags<<<blocks_for(n, 256), 256, 0, st>>>(t->child, n, t->int_index); note_launch();
-  T2_CHECK(scan_exclusive_i32(t->int_index, n, dtotal, st));
-  int totals[2] = {0, 0};  // internal nodes, luminous elements
-  T2_CUDA(cudaMemcpyAsync(totals, dtotal, sizeof(totals), cudaMemcpyDeviceToHost, st));
-  k_finish_int_index<<<blocks_for(n, 256), 256, 0, st>>>(t->child, n, t->int_index); note_launch();
-  dfree(dtotal, st);
-
-  // 5. aggregates, deepest depth first
-  T2_CHECK(dalloc(&t->nodes, n, st));
-  T2_CHECK(dalloc(&t->Lnode, n * nbp, st));
-  T2_CHECK(dalloc(&t->csrc, n, st));
-  T2_CHECK(dalloc(&t->c64, 3 * n, st));
-  T2_CHECK(dalloc(&t->B64, n, st));
-  T2_CHECK(dalloc(&t->alpha_leaf, n * nbp, st));
-  T2_CHECK(dalloc(&t->lmask, n, st));
-  DeviceTemp<double> L64_t(st), cs64_t(st);
-  DeviceTemp<uint32_t> fl_t(st);
-  double*& L64 = L64_t.p;
-  double*& cs64 = cs64_t.p;
-  uint32_t*& fl = fl_t.p;
-  T2_CHECK(dalloc(&L64, 4 * n, st));
-  T2_CHECK(dalloc(&cs64, 4 * n, st));
-  T2_CHECK(dalloc(&fl, n, st));
-  const double inv_size2 = 1.0 / (t->size * t->size);
-  for (int d = t->max_depth; d >= 0; --d) {
-    int64_t a = t->level_begin[d], b = t->level_begin[d + 1];
-    k_aggregate_level<<<blocks_for(b - a, 128), 128, 0, st>>>(
-        a, b, nb, nbp, inv_size2, t->prefix, t->depth, t->first, t->count, t->child,
-        t->int_index, t->pos64, t->Lelem, t->perm, kappa, mass, L64, cs64, fl, t->Lnode, t->csrc, t->c64,
-        t->B64, t->alpha_leaf, t->lmask, t->nodes); note_launch();
-  }
-  dfree(L64, st);
-  dfree(cs64, st);
-  dfree(fl, st);
-  T2_CUDA(cudaGetLastError());
-  T2_CUDA(cudaStreamSynchronize(st));
-  t->n_internal = totals[0];
-  t->n_luminous = totals[1];
+  for (int a = 0; a < 3; ++a) t->lo[a] = S.lo[a];
+  t->size = S.size;
+  t->n_nodes = S.n_nodes;
+  t->max_depth = S.levels - 1;
+  t->level_begin.assign(S.level_begin, S.level_begin + S.levels);
+  t->level_begin.push_back(S.n_nodes);
+  t->n_internal = S.n_internal;
+  t->n_luminous = S.n_luminous;
   return TREVR2_OK;
 }
 

@@ -51,6 +51,7 @@ constexpr uint32_t kStatusBadActive = 1u << 0;
 constexpr uint32_t kStatusStackOverflow = 1u << 1;
 constexpr uint32_t kStatusBadInput = 1u << 2;
 constexpr uint32_t kStatusOutsideBox = 1u << 3;
+constexpr uint32_t kStatusBarrier = 1u << 4;     // a grid barrier gave up waiting
 constexpr uint32_t kStatusPPOverflow = 1u << 5;  // a p-p sphere held too many particles
 
 // Geometry of the transmission average for one cell shape and one beam pair:
@@ -144,6 +145,41 @@ struct Tree {
 };
 
 // ---------------------------------------------------------------------------
+// Barrier of all blocks of one cooperative launch (so they are resident
+// together): *bar counts arrivals, from 0 at the launch.  The wait ends after
+// kBarrierSpins polls at the latest; then the barrier is marked as failed for
+// good and every block gets false and returns.
+constexpr uint32_t kBarrierSpins = 1u << 24;
+constexpr uint32_t kBarrierFailed = 0x80000000u;
+
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t blocks, uint32_t* status) {
+  __shared__ uint32_t arrived_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t ok = 1;
+    if (blocks > 1) {
+      __threadfence();
+      const uint32_t at = atomicAdd(bar, 1u);
+      const uint32_t target = (at / blocks + 1u) * blocks;
+      uint32_t seen = 0, spins = 0;
+      do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+        if ((seen | at) & kBarrierFailed) ok = 0;
+        if (ok && seen < target && ++spins == kBarrierSpins) {
+          atomicOr(bar, kBarrierFailed);
+          if (status) atomicOr(status, kStatusBarrier);
+          ok = 0;
+        }
+      } while (ok && seen < target);
+      __threadfence();
+    }
+    arrived_ok = ok;
+  }
+  __syncthreads();
+  return arrived_ok != 0;
+}
+
+// ---------------------------------------------------------------------------
 // Host helpers (errors, allocation).
 void set_error(const char* fmt, ...);
 void clear_error();
@@ -196,6 +232,17 @@ struct DeviceTemp {
 // trevr2_debug_set(TREVR2_DEBUG_SOURCE_STACK, c); 0 when not set.
 int debug_source_stack_cap();
 
+// Blocks of a cooperative launch: at most per_sm per SM (the kernel's bound,
+// so that they are resident together), fewer where the work would leave them
+// idle at the barriers.
+constexpr int kMaxCoopBlocks = 512;
+int coop_blocks(int64_t work, int64_t per_block, int per_sm, int* out);
+
+// The receivers' slots in their elements' sorted order (keys: their sorted
+// positions, N for an index outside [0, N)).
+int order_receivers(const Tree* t, const int64_t* active, int64_t A, uint64_t* keys, int* slots,
+                    cudaStream_t st);
+
 // Exclusive scan of n int32 values in place; *d_total (device) gets the sum.
 // ws (device, scan_ws_ints(n) ints) or NULL to allocate one stream ordered.
 size_t scan_ws_ints(int64_t n);
@@ -204,8 +251,9 @@ int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws
 // Stable LSD radix sort of keys below 2^key_bits with int32 payload (in place).
 // ws (device, radix_ws_bytes(n) bytes) or NULL to allocate one stream ordered.
 size_t radix_ws_bytes(int64_t n);
-int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, int key_bits = 64,
-                       void* ws = nullptr);
+// A grid barrier that gives up sets kStatusBarrier in *status.
+int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, uint32_t* status,
+                       int key_bits = 64, void* ws = nullptr);
 
 // Alpha tables and beam directions for one nside and averaging (built and
 // cached): Eq. transmissionavg, or with `linear` the volume-weighted linear

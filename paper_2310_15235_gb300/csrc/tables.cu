@@ -31,26 +31,20 @@
 
 namespace trevr2 {
 
-__global__ void k_dirs(int nside, int npix, double* __restrict__ dirs64, float4* __restrict__ dirs) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= npix) return;
+__device__ __forceinline__ void table_dir(int nside, int npix, int k, double* dirs64, float4* dirs) {
   double v[3];
   hp_pix2vec(nside, k, v);
-  for (int a = 0; a < 3; ++a) dirs64[3 * k + a] = v[a];
+  for (int a = 0; a < 3; ++a) __stcg(dirs64 + 3 * k + a, v[a]);
   int pair = k < npix / 2 ? k : hp_vec2pix_f64(nside, -v[0], -v[1], -v[2]);
-  dirs[k] = make_float4(float(v[0]), float(v[1]), float(v[2]), __int_as_float(pair));
+  __stcg(dirs + k, make_float4(float(v[0]), float(v[1]), float(v[2]), __int_as_float(pair)));
 }
 
 // Transmission geometry of one cell shape (unit scale) for one beam pair.
-__global__ void k_trans_geo(int P, const double* __restrict__ dirs64, TransGeo* __restrict__ geo) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 3 * P) return;
-  const int shape = idx / P, p = idx % P;
+__device__ __forceinline__ TransGeo table_geo(int shape, const double n[3]) {
   double E[3] = {1.0, 1.0, 1.0};
   if (shape >= 1) E[0] = 0.5;
   if (shape >= 2) E[1] = 0.5;
   const int a = shape, b = (a + 1) % 3, c = (a + 2) % 3;
-  const double n[3] = {dirs64[3 * p], dirs64[3 * p + 1], dirs64[3 * p + 2]};
   const double V = E[0] * E[1] * E[2];
   double V12 = 0.0;
   if (n[a] != 0.0) {
@@ -71,7 +65,7 @@ __global__ void k_trans_geo(int P, const double* __restrict__ dirs64, TransGeo* 
   g.w12 = float(V12 / V);
   g.d_unit = float(d);
   g.pad = 0.0f;
-  geo[idx] = g;
+  return g;
 }
 
 // The unit vector through point (a, b) of face f of the cube [-1, 1]^3:
@@ -198,36 +192,87 @@ __device__ __forceinline__ float combine_alpha(float a1, float a2, float w1, flo
   return fmaxf(0.0f, -lnT / d);
 }
 
+// One table in one cooperative launch: beam directions, then the transmission
+// geometry, then the cells' absorption one depth at a time, deepest first
+// (a thread per cell and beam pair), with grid barriers between; runs of small
+// depths stay in block 0.  A launch per depth cost the small trees more than
+// the depths' work.  Values another block wrote are read past the L1.
+struct TableArgs {
+  int nside, npix, P, nb, levels;
+  bool linear;
+  const NodeW* nodes;
+  const int* int_index;
+  const float* alpha_leaf;
+  double* dirs64;
+  float4* dirs;
+  TransGeo* geo;
+  float* tab;
+  uint32_t* bar;
+  uint32_t* status;
+  int level_begin[kMaxDepth + 3];
+};
+constexpr int kTableThreads = 512;
+constexpr int64_t kTableSmall = 4 * kTableThreads;  // items of a depth that block 0 does alone
+
 template <int NBP>
-__global__ void k_alpha_level(int64_t lb, int64_t le, int P, int nb, bool linear,
-                              const NodeW* __restrict__ nodes,
-                              const int* __restrict__ int_index,
-                              const float* __restrict__ alpha_leaf,
-                              const TransGeo* __restrict__ geo, float* __restrict__ tab) {
-  int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  int64_t q = lb + idx / P;
-  int p = int(idx % P);
-  if (q >= le) return;
-  const NodeW nd = nodes[q];
+__device__ __forceinline__ void alpha_item(const TableArgs& A, int q, int p) {
+  const NodeW nd = A.nodes[q];
   if (nd.child < 0) return;
+  const int P = A.P;
   const int depth = int(nd.meta & kMetaDepthMask);
-  const TransGeo g = geo[(depth % 3) * P + p];
-  const float d = ldexpf(g.d_unit, -(depth / 3));
+  const float4 gv = __ldcg(reinterpret_cast<const float4*>(A.geo) + (depth % 3) * P + p);
+  const float d = ldexpf(gv.z, -(depth / 3));
   float a1[NBP], a2[NBP];
   const int c = nd.child;
-  const int i1 = int_index[c], i2 = int_index[c + 1];
+  const int i1 = A.int_index[c], i2 = A.int_index[c + 1];
 #pragma unroll
   for (int b = 0; b < NBP; ++b) {
-    a1[b] = i1 < 0 ? alpha_leaf[int64_t(c) * NBP + b] : tab[(int64_t(i1) * P + p) * NBP + b];
-    a2[b] = i2 < 0 ? alpha_leaf[int64_t(c + 1) * NBP + b] : tab[(int64_t(i2) * P + p) * NBP + b];
+    a1[b] = i1 < 0 ? A.alpha_leaf[int64_t(c) * NBP + b] : __ldcg(A.tab + (int64_t(i1) * P + p) * NBP + b);
+    a2[b] = i2 < 0 ? A.alpha_leaf[int64_t(c + 1) * NBP + b] : __ldcg(A.tab + (int64_t(i2) * P + p) * NBP + b);
   }
-  const int iq = int_index[q];
+  float* out = A.tab + (int64_t(nd.aux) * P + p) * NBP;
 #pragma unroll
   for (int b = 0; b < NBP; ++b) {
     float al = 0.0f;
-    if (b < nb && (a1[b] > 0.0f || a2[b] > 0.0f))
-      al = linear ? 0.5f * (a1[b] + a2[b]) : combine_alpha(a1[b], a2[b], g.w1, g.w12, d);
-    tab[(int64_t(iq) * P + p) * NBP + b] = al;
+    if (b < A.nb && (a1[b] > 0.0f || a2[b] > 0.0f))
+      al = A.linear ? 0.5f * (a1[b] + a2[b]) : combine_alpha(a1[b], a2[b], gv.x, gv.y, d);
+    __stcg(out + b, al);
+  }
+}
+
+template <int NBP>
+__global__ void __launch_bounds__(kTableThreads, 2) k_tables(const __grid_constant__ TableArgs A) {
+  const int blocks = gridDim.x, t = threadIdx.x, P = A.P;
+  const int64_t stride = int64_t(blocks) * kTableThreads, at = int64_t(blockIdx.x) * kTableThreads + t;
+  for (int64_t k = at; k < A.npix; k += stride) table_dir(A.nside, A.npix, int(k), A.dirs64, A.dirs);
+  if (!grid_barrier(A.bar, blocks, A.status)) return;
+  for (int64_t i = at; i < 3 * P; i += stride) {
+    const int p = int(i % P);
+    const double n[3] = {__ldcg(A.dirs64 + 3 * p), __ldcg(A.dirs64 + 3 * p + 1), __ldcg(A.dirs64 + 3 * p + 2)};
+    const TransGeo g = table_geo(int(i / P), n);
+    __stcg(reinterpret_cast<float4*>(A.geo) + i, make_float4(g.w1, g.w12, g.d_unit, g.pad));
+  }
+  bool together = true;  // whether all blocks did what the next depth needs
+  for (int d = A.levels - 2; d >= 0; --d) {  // the deepest depth has leaves only
+    const int b0 = A.level_begin[d], b1 = A.level_begin[d + 1];
+    const int64_t items = int64_t(b1 - b0) * P;
+    const bool small = items <= kTableSmall;
+    if (together || !small) {
+      if (!grid_barrier(A.bar, blocks, A.status)) return;
+    } else {
+      __syncthreads();
+    }
+    together = !small;
+    if (small) {
+      if (blockIdx.x == 0)
+        for (int i = t; i < int(items); i += kTableThreads)
+          alpha_item<NBP>(A, b0 + int(unsigned(i) / unsigned(P)), int(unsigned(i) % unsigned(P)));
+    } else if (items < (int64_t(1) << 31)) {
+      for (unsigned i = unsigned(at); i < unsigned(items); i += unsigned(stride))
+        alpha_item<NBP>(A, b0 + int(i / unsigned(P)), int(i % unsigned(P)));
+    } else {
+      for (int64_t i = at; i < items; i += stride) alpha_item<NBP>(A, b0 + int(i / P), int(i % P));
+    }
   }
 }
 
@@ -275,19 +320,36 @@ int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear) 
   tb.dirs64 = dirs64.p;
   tb.geo = geo.p;
   tb.alpha = alpha.p;
-  k_dirs<<<(npix + 127) / 128, 128, 0, st>>>(nside, npix, tb.dirs64, tb.dirs); note_launch();
-  k_trans_geo<<<(3 * P + 127) / 128, 128, 0, st>>>(P, tb.dirs64, tb.geo); note_launch();
-  for (int d = t->max_depth; d >= 0; --d) {
-    int64_t a = t->level_begin[d], b = t->level_begin[d + 1];
-    int64_t work = (b - a) * P;
-    unsigned blocks = unsigned((work + 255) / 256);
-    if (work == 0) continue;
-    switch (t->nbp) {
-      case 1: k_alpha_level<1><<<blocks, 256, 0, st>>>(a, b, P, t->nb, linear, t->nodes, t->int_index, t->alpha_leaf, tb.geo, tb.alpha); note_launch(); break;
-      case 2: k_alpha_level<2><<<blocks, 256, 0, st>>>(a, b, P, t->nb, linear, t->nodes, t->int_index, t->alpha_leaf, tb.geo, tb.alpha); note_launch(); break;
-      default: k_alpha_level<4><<<blocks, 256, 0, st>>>(a, b, P, t->nb, linear, t->nodes, t->int_index, t->alpha_leaf, tb.geo, tb.alpha); note_launch(); break;
-    }
+  TableArgs A;
+  A.nside = nside;
+  A.npix = npix;
+  A.P = P;
+  A.nb = t->nb;
+  A.levels = t->max_depth + 1;
+  A.linear = linear;
+  A.nodes = t->nodes;
+  A.int_index = t->int_index;
+  A.alpha_leaf = t->alpha_leaf;
+  A.dirs64 = tb.dirs64;
+  A.dirs = tb.dirs;
+  A.geo = tb.geo;
+  A.tab = tb.alpha;
+  A.bar = t->status + 1;
+  A.status = t->status;
+  int64_t widest = npix;
+  for (int d = 0; d <= t->max_depth + 1; ++d) {
+    A.level_begin[d] = int(t->level_begin[d]);
+    if (d) widest = std::max(widest, (t->level_begin[d] - t->level_begin[d - 1]) * P);
   }
+  int blocks = 0;
+  T2_CHECK(coop_blocks(widest, 2 * kTableThreads, 2, &blocks));
+  T2_CUDA(cudaMemsetAsync(A.bar, 0, sizeof(uint32_t), st));
+  const void* fn = t->nbp == 1 ? reinterpret_cast<const void*>(&k_tables<1>)
+                 : t->nbp == 2 ? reinterpret_cast<const void*>(&k_tables<2>)
+                               : reinterpret_cast<const void*>(&k_tables<4>);
+  void* args[] = {&A};
+  T2_CUDA(cudaLaunchCooperativeKernel(fn, dim3(unsigned(blocks)), dim3(kTableThreads), args, 0, st));
+  note_launch();
   T2_CUDA(cudaGetLastError());
   t->tables.push_back(tb);
   dirs.p = nullptr;

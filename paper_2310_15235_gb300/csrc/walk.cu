@@ -1426,16 +1426,6 @@ static int grow_buffer(void** buf, size_t* bytes, size_t need, cudaStream_t st, 
   return TREVR2_OK;
 }
 
-__global__ void k_order_keys(const int64_t* __restrict__ active, int64_t A, int64_t N,
-                             const int* __restrict__ inv, uint64_t* __restrict__ keys,
-                             int* __restrict__ slots) {
-  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (i >= A) return;
-  const int64_t io = active[i];
-  keys[i] = (io >= 0 && io < N) ? uint64_t(inv[io]) : uint64_t(N);
-  slots[i] = int(i);
-}
-
 static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int nside,
                        float theta, const int* bsel, int nbsel, uint32_t flags, float* J,
                        cudaStream_t st) {
@@ -1449,11 +1439,7 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
     T2_CHECK(grow_buffer(&t->order_buf, &t->order_bytes, need, st, "receiver order"));
     uint64_t* keys = static_cast<uint64_t*>(t->order_buf);
     int* slots = reinterpret_cast<int*>(keys + A);
-    k_order_keys<<<unsigned((A + 255) / 256), 256, 0, st>>>(active, A, t->N, t->inv, keys, slots);
-    note_launch();
-    int bits = 1;
-    while ((int64_t(1) << bits) <= t->N) ++bits;
-    T2_CHECK(radix_sort_u64_i32(keys, slots, A, st, bits));
+    T2_CHECK(order_receivers(t, active, A, keys, slots, st));
     a.order = slots;
   }
   const bool cells = use_cells(t, tb, theta);
@@ -1677,13 +1663,7 @@ static int launch_walk_bucket(Tree* t, Table* tb, const int64_t* active, int64_t
   int* slots = reinterpret_cast<int*>(keys + A);
   int* leaf = slots + A;
   const unsigned gb = unsigned((A + 255) / 256);
-  k_order_keys<<<gb, 256, 0, st>>>(active, A, t->N, t->inv, keys, slots);
-  note_launch();
-  if (A > 1) {
-    int bits = 1;
-    while ((int64_t(1) << bits) <= t->N) ++bits;
-    T2_CHECK(radix_sort_u64_i32(keys, slots, A, st, bits));
-  }
+  T2_CHECK(order_receivers(t, active, A, keys, slots, st));
   k_bucket_leaf<<<gb, 256, 0, st>>>(t->child, t->first, keys, A, t->N, leaf);
   note_launch();
   a.order = slots;
@@ -1759,6 +1739,10 @@ int read_status(Tree* t, cudaStream_t st) {
     set_error("trevr2_J: a bucket's p-p sphere holds more than %d particles (TREVR2_PP)",
               kPPCapacity);
     return TREVR2_EUNSUPPORTED;
+  }
+  if (s & kStatusBarrier) {
+    set_error("trevr2_J: a grid barrier of the receiver sort gave up waiting");
+    return TREVR2_ETIMEOUT;
   }
   set_error("trevr2: device status 0x%x", s);
   return TREVR2_EINTERNAL;
@@ -1976,7 +1960,8 @@ static int batch_enqueue(Batch* b, const int64_t* active, float* J, cudaStream_t
   const unsigned g = unsigned((R + 255) / 256);
   T2_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(unsigned long long), st));
   k_batch_keys<<<g, 256, 0, st>>>(b->args); note_launch();
-  T2_CHECK(radix_sort_u64_i32(b->args.keys, b->args.rows, R, st, b->key_bits, b->sort_ws));
+  T2_CHECK(radix_sort_u64_i32(b->args.keys, b->args.rows, R, st, b->trees[0]->status,
+                              b->key_bits, b->sort_ws));
   k_batch_first<<<g, 256, 0, st>>>(b->args); note_launch();
   T2_CHECK(scan_exclusive_i32(b->args.first_scan, R, b->args.n_distinct, st, b->scan_ws));
   k_batch_distinct<<<g, 256, 0, st>>>(b->args); note_launch();
