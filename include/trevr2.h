@@ -369,9 +369,10 @@ const char* trevr2_last_error(void);
 /* Sets one testing aid (EINVAL for an unknown `what` or a value out of range). */
 int trevr2_debug_set(int what, int64_t value);
 
-/* Bytes the library currently holds in the current device's default
- * stream-ordered memory pool, which only this library allocates from
- * (synchronises the device first; ECUDA if the query fails). */
+/* Bytes the library currently holds in its own stream-ordered memory pool of
+ * the current device (synchronises the device first; ECUDA if the query
+ * fails).  The pool keeps up to 2 GiB of freed memory for later calls and
+ * gives it back when an allocation fails. */
 int trevr2_debug_pool_used(uint64_t* bytes);
 
 /* The architecture the library's kernels run as on the current device

@@ -104,7 +104,7 @@ def debug_set(what: int, value: int) -> None:
 
 
 def debug_pool_used() -> int:
-    """Bytes libtrevr2 holds in the current device's default memory pool."""
+    """Bytes libtrevr2 holds in its memory pool of the current device."""
     v = C.c_uint64(0)
     _check(load_library().trevr2_debug_pool_used(C.byref(v)))
     return int(v.value)

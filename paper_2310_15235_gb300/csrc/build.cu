@@ -15,6 +15,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <string>
@@ -57,6 +58,46 @@ static bool injected_alloc_failure() {
   return false;
 }
 
+// The library's memory pool of the current device.  The default pool gives
+// every freed byte back at the next synchronisation, so that each step's trees
+// were mapped anew (about 0.4 ms of a 4k-element step, 1 ms of a 2.1M one); this
+// one keeps up to kPoolKeep free bytes (a 2.1M-element tree with its tables and
+// walk buffers; 0.7 % of the card), and gives them back when an allocation
+// fails.
+constexpr uint64_t kPoolKeep = uint64_t(2) << 30;
+constexpr int kMaxDevices = 64;
+
+static int library_pool(cudaMemPool_t* pool) {
+  static std::mutex lock;
+  static cudaMemPool_t pools[kMaxDevices] = {};
+  int dev = 0;
+  T2_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) {
+    T2_CUDA(cudaDeviceGetDefaultMemPool(pool, dev));
+    return TREVR2_OK;
+  }
+  std::lock_guard<std::mutex> hold(lock);
+  if (!pools[dev]) {
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t fresh = nullptr;
+    T2_CUDA(cudaMemPoolCreate(&fresh, &props));
+    uint64_t keep = kPoolKeep;
+    const cudaError_t e = cudaMemPoolSetAttribute(fresh, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(fresh);
+      return cuda_fail(e, "cudaMemPoolSetAttribute");
+    }
+    pools[dev] = fresh;
+  }
+  *pool = pools[dev];
+  return TREVR2_OK;
+}
+
 int device_alloc(void** p, size_t bytes, cudaStream_t st, const char* what) {
   *p = nullptr;
   if (injected_alloc_failure()) {
@@ -64,7 +105,14 @@ int device_alloc(void** p, size_t bytes, cudaStream_t st, const char* what) {
               "trevr2_debug_set)", what, bytes);
     return TREVR2_ENOMEM;
   }
-  cudaError_t e = cudaMallocAsync(p, bytes, st);
+  cudaMemPool_t pool = nullptr;
+  T2_CHECK(library_pool(&pool));
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  if (e == cudaErrorMemoryAllocation) {  // give back what the pool keeps, and try once more
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
   if (e != cudaSuccess) {
     *p = nullptr;
     cudaGetLastError();
@@ -1234,11 +1282,9 @@ int trevr2_debug_pool_used(uint64_t* bytes) {
     set_error("trevr2_debug_pool_used: bytes is NULL");
     return TREVR2_EINVAL;
   }
-  int dev = 0;
-  T2_CUDA(cudaGetDevice(&dev));
   T2_CUDA(cudaDeviceSynchronize());
-  cudaMemPool_t pool;
-  T2_CUDA(cudaDeviceGetDefaultMemPool(&pool, dev));
+  cudaMemPool_t pool = nullptr;
+  T2_CHECK(library_pool(&pool));
   uint64_t used = 0;
   T2_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
   *bytes = uint64_t(used);
