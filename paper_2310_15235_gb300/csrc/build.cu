@@ -219,8 +219,9 @@ int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws
 // ---------------------------------------------------------------------------
 // Stable sort of 64-bit keys with a 32-bit payload.
 //
-// Up to kSmallSort keys: one block, a bitonic sort of (key, input position) in
-// shared memory; the position makes the order stable.  More: one cooperative
+// Up to kSmallSort keys: one block, a merge sort in shared memory, every key
+// finding its place in the neighbouring run by a binary search (4097 keys: 14
+// us; a bitonic network's 91 steps took 75).  More: one cooperative
 // launch does every pass of an LSD radix sort (8 bits a pass), with a grid
 // barrier where a pass needs all blocks' counts or keys: a launch for each
 // step of each pass left the GPU idle between them for longer than the steps
@@ -228,60 +229,64 @@ int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws
 constexpr int kSmallSort = 8192;
 constexpr int kSmallSortThreads = 1024;
 
-__device__ __forceinline__ bool sort_after(uint64_t ka, uint32_t pa, uint64_t kb, uint32_t pb) {
-  return ka > kb || (ka == kb && pa > pb);
-}
-
 // With `active`, the receivers' order: the keys are their elements' sorted
 // positions (N for an index outside [0, N)), the payload their slots.
 __global__ void __launch_bounds__(kSmallSortThreads)
-    k_sort_small(uint64_t* keys, int* vals, int n, int n2, const int64_t* __restrict__ active,
+    k_sort_small(uint64_t* keys, int* vals, int n, const int64_t* __restrict__ active,
                  const int* __restrict__ inv, int64_t N) {
   extern __shared__ uint64_t sort_smem[];
-  uint64_t* k = sort_smem;
-  uint32_t* p = reinterpret_cast<uint32_t*>(k + n2);
-  for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-    uint64_t key = ~0ull;  // the padding comes last: its positions are beyond n
-    if (i < n) {
-      if (active) {
-        const int64_t io = active[i];
-        key = io >= 0 && io < N ? uint64_t(inv[io]) : uint64_t(N);
-      } else {
-        key = keys[i];
-      }
+  uint64_t *ka = sort_smem, *kb = ka + n;
+  uint16_t *pa = reinterpret_cast<uint16_t*>(kb + n), *pb = pa + n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    uint64_t key;
+    if (active) {
+      const int64_t io = active[i];
+      key = io >= 0 && io < N ? uint64_t(inv[io]) : uint64_t(N);
+    } else {
+      key = keys[i];
     }
-    k[i] = key;
-    p[i] = uint32_t(i);
+    ka[i] = key;
+    pa[i] = uint16_t(i);
+  }
+  for (int run = 1; run < n; run <<= 1) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const uint64_t key = ka[i];
+      const int base = i & ~(2 * run - 1);
+      const bool left = i - base < run;
+      // the other run; its equal keys go before a right one, after a left one
+      const int first = left ? base + run : base;
+      int lo = min(first, n), hi = min(first + run, n);
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const uint64_t other = ka[mid];
+        if (left ? other < key : other <= key) lo = mid + 1; else hi = mid;
+      }
+      const int at = left ? i + lo - min(first, n) : i - run + lo - first;
+      kb[at] = key;
+      pb[at] = pa[i];
+    }
+    uint64_t* const tk = ka;
+    ka = kb;
+    kb = tk;
+    uint16_t* const tp = pa;
+    pa = pb;
+    pb = tp;
   }
   __syncthreads();
-  for (int size = 2; size <= n2; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
-        const int i = 2 * t - (t & (stride - 1)), j = i + stride;
-        const uint64_t ki = k[i], kj = k[j];
-        const uint32_t pi = p[i], pj = p[j];
-        if (sort_after(ki, pi, kj, pj) == ((i & size) == 0)) {
-          k[i] = kj;
-          k[j] = ki;
-          p[i] = pj;
-          p[j] = pi;
-        }
-      }
-      __syncthreads();
-    }
-  constexpr int kPer = kSmallSort / kSmallSortThreads;
-  int v[kPer];
+  // the payload is permuted in place: read by everybody before it is written
+  int v[kSmallSort / kSmallSortThreads];
 #pragma unroll
-  for (int r = 0; r < kPer; ++r) {
+  for (int r = 0; r < kSmallSort / kSmallSortThreads; ++r) {
     const int i = threadIdx.x + r * blockDim.x;
-    if (i < n) v[r] = active ? int(p[i]) : vals[p[i]];
+    if (i < n) v[r] = active ? int(pa[i]) : vals[pa[i]];
   }
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < kPer; ++r) {
+  for (int r = 0; r < kSmallSort / kSmallSortThreads; ++r) {
     const int i = threadIdx.x + r * blockDim.x;
     if (i < n) {
-      keys[i] = k[i];
+      keys[i] = ka[i];
       vals[i] = v[r];
     }
   }
@@ -408,13 +413,12 @@ size_t radix_ws_bytes(int64_t n) {
 
 static int sort_small(uint64_t* keys, int* vals, int n, cudaStream_t st, const int64_t* active,
                       const int* inv, int64_t N) {
-  int n2 = 2;
-  while (n2 < n) n2 <<= 1;
-  const size_t smem = size_t(n2) * (sizeof(uint64_t) + sizeof(uint32_t));
+  const size_t smem = size_t(n) * 2 * (sizeof(uint64_t) + sizeof(uint16_t)) + 8;
   T2_CUDA(cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmallSort * 12));
-  k_sort_small<<<1, std::min(kSmallSortThreads, std::max(32, n2 / 2)), smem, st>>>(
-      keys, vals, n, n2, active, inv, N);
+                               kSmallSort * 20 + 8));
+  // at most kSmallSort / kSmallSortThreads keys a thread
+  const int threads = std::min(kSmallSortThreads, (n + 31) & ~31);
+  k_sort_small<<<1, threads, smem, st>>>(keys, vals, n, active, inv, N);
   note_launch();
   T2_CUDA(cudaGetLastError());
   return TREVR2_OK;
@@ -669,9 +673,10 @@ __global__ void k_gather_elements(const double* __restrict__ pos, const float* _
 // level, counts its splits, and after a grid barrier places its children
 // behind those of the blocks before it.  A node splits while it holds more
 // than `bucket` elements; nodes are numbered by depth, by prefix within a
-// depth.  Aggregates: all leaves at once, then in one cooperative launch the
-// internal nodes, deepest depth first (their children are done); runs of small
-// depths stay in block 0.  Values another block wrote are read past the L1.
+// depth.  Aggregates: the leaves' sums at once, then in one cooperative launch
+// the internal nodes' (additions only), deepest depth first; runs of small
+// depths stay in block 0; then every node's centre, B and record at once.
+// Values another block wrote are read past the L1.
 struct TreeArgs {
   const uint64_t* keys;
   int64_t N;
@@ -720,6 +725,24 @@ __device__ __forceinline__ int split_at(const TreeArgs& A, int d, int f, int c) 
   return lo;
 }
 
+// The same for one node by a whole warp: 32 probes a step instead of one.
+__device__ __forceinline__ int split_at_warp(const TreeArgs& A, int d, int f, int c) {
+  if (!(c > A.bucket && d < kMaxDepth)) return -1;
+  const int bit = kMaxDepth - 1 - d, lane = threadIdx.x & 31;
+  int lo = f, hi = f + c;  // first index with the bit set lies in [lo, hi]
+  while (lo < hi) {
+    const int step = (hi - lo + 31) >> 5;
+    const int at = lo + lane * step;  // probes lo, lo + step, ...
+    const bool set = at >= hi || ((A.keys[at] >> bit) & 1ull);
+    const unsigned m = __ballot_sync(0xffffffffu, set);
+    if (m & 1u) return lo;
+    const int k = m ? __ffs(m) - 1 : 32;  // clear at probe k - 1, set at probe k
+    hi = min(hi, lo + k * step);
+    lo = lo + (k - 1) * step + 1;
+  }
+  return lo;
+}
+
 __device__ __forceinline__ void emit_halves(const TreeArgs& A, int q, int c, int d, int f, int n,
                                             int m) {
   const uint64_t p = __ldcg(A.prefix + q);
@@ -754,93 +777,120 @@ __device__ __forceinline__ int tile_rank(bool flag, int& total) {
   return before + __popc(m & ((1u << lane) - 1u));
 }
 
-// ---------------------------------------------------------------------------
-// Bottom-up aggregates for one depth (children are done before parents).
-__device__ inline void node_box_norm(uint64_t prefix, int depth, double lo[3], double ext[3]) {
-  for (int a = 0; a < 3; ++a) {
-    uint64_t k = 0;
-    for (int l = 0; l < kKeyBits; ++l) k = (k << 1) | ((prefix >> (3 * (kKeyBits - 1 - l) + 2 - a)) & 1ull);
-    lo[a] = double(k) * (1.0 / 2097152.0);
-    ext[a] = ldexp(1.0, -splits_on_axis(depth, a));
-  }
-}
-
-__device__ void aggregate_node(const TreeArgs& A, int64_t q, bool leaf, double inv_size2) {
+// The sums of a leaf's elements: luminosity per band, L-weighted position and
+// total, bucket absorption; whether it absorbs or shines.
+__device__ __forceinline__ void leaf_sums(const TreeArgs& A, int64_t q, double inv_size2) {
   const int nb = A.nb, nbp = A.nbp;
-  const int d = __ldcg(A.depth + q);
-  double lo[3], ext[3];
-  node_box_norm(__ldcg(A.prefix + q), d, lo, ext);
-  const int c = leaf ? -1 : __ldcg(A.child + q);
-  double cs[4] = {0, 0, 0, 0};
-  uint32_t has = 0, lit = 0, half0 = 0, half1 = 0;
-  if (c < 0) {
-    const int f = __ldcg(A.first + q), n = __ldcg(A.count + q);
-    double Lb[4] = {0, 0, 0, 0}, kmb[4] = {0, 0, 0, 0};
-    for (int e = f; e < f + n; ++e) {
-      double lt = 0.0;
-      for (int b = 0; b < nb; ++b) {
-        double l = double(A.Lelem[int64_t(e) * nbp + b]);
-        Lb[b] = __dadd_rn(Lb[b], l);
-        lt = __dadd_rn(lt, l);
-        // kappa and m are float32: their FP64 product is exact
-        const int i = A.perm[e];
-        kmb[b] = __dadd_rn(kmb[b], __dmul_rn(double(A.kappa[int64_t(i) * nb + b]), double(A.mass[i])));
-      }
+  const int f = A.first[q], n = A.count[q];
+  double Lb[4] = {0, 0, 0, 0}, kmb[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0};
+  uint32_t has = 0, lit = 0;
+  for (int e = f; e < f + n; ++e) {
+    double lt = 0.0;
+    const int i = A.perm[e];
+    const double m = double(A.mass[i]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      if (b >= nb) break;
+      const double l = double(A.Lelem[int64_t(e) * nbp + b]);
+      Lb[b] = __dadd_rn(Lb[b], l);
+      lt = __dadd_rn(lt, l);
+      // kappa and m are float32: their FP64 product is exact
+      kmb[b] = __dadd_rn(kmb[b], __dmul_rn(double(A.kappa[int64_t(i) * nb + b]), m));
+    }
+    if (lt > 0.0) {  // else it adds zeros
+#pragma unroll
       for (int a = 0; a < 3; ++a) cs[a] = __dadd_rn(cs[a], __dmul_rn(lt, A.pos64[3 * int64_t(e) + a]));
       cs[3] = __dadd_rn(cs[3], lt);
-      if (lt > 0.0 && e - f < 32) lit |= 1u << (e - f);
+      if (e - f < 32) lit |= 1u << (e - f);
     }
-    const double V = ext[0] * ext[1] * ext[2];  // exact powers of two
-    for (int b = 0; b < nbp; ++b) {
-      double al = b < nb ? kmb[b] / V * inv_size2 : 0.0;
+  }
+  // 1 / V: V = 2^-depth, so the product is exact
+  const double iV = __longlong_as_double((long long)(1023 + A.depth[q]) << 52);
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    if (b < nbp) {
+      const double al = b < nb ? kmb[b] * iV * inv_size2 : 0.0;
       A.alpha_leaf[q * nbp + b] = float(al);
       if (al > 0.0) has |= kMetaHasAlpha;
     }
-    for (int b = 0; b < 4; ++b) __stcg(A.L64 + q * 4 + b, b < nb ? Lb[b] : 0.0);
-  } else {
-    for (int b = 0; b < 4; ++b)
-      __stcg(A.L64 + q * 4 + b, __dadd_rn(__ldcg(A.L64 + int64_t(c) * 4 + b), __ldcg(A.L64 + int64_t(c + 1) * 4 + b)));
-    for (int a = 0; a < 4; ++a) cs[a] = __dadd_rn(__ldcg(A.cs64 + int64_t(c) * 4 + a), __ldcg(A.cs64 + int64_t(c + 1) * 4 + a));
-    half0 = __ldcg(A.flags + c);
-    half1 = __ldcg(A.flags + c + 1);
-    has = (half0 | half1) & kMetaHasAlpha;
+    A.L64[q * 4 + b] = b < nb ? Lb[b] : 0.0;
+    A.cs64[q * 4 + b] = cs[b];
+  }
+  if (cs[3] > 0.0) has |= kMetaHasL;
+  A.flags[q] = has;
+  A.lmask[q] = lit;
+}
+
+// The sums of an internal node from its halves'.
+__device__ __forceinline__ void inner_sums(const TreeArgs& A, int64_t q) {
+  const int64_t c = __ldcg(A.child + q);
+  if (c < 0) return;
+  const double2* L = reinterpret_cast<const double2*>(A.L64 + 4 * c);
+  const double2* s = reinterpret_cast<const double2*>(A.cs64 + 4 * c);
+  const uint32_t h0 = __ldcg(A.flags + c), h1 = __ldcg(A.flags + c + 1);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double2 l0 = __ldcg(L + i), l1 = __ldcg(L + 2 + i);
+    const double2 s0 = __ldcg(s + i), s1 = __ldcg(s + 2 + i);
+    __stcg(reinterpret_cast<double2*>(A.L64 + 4 * q) + i,
+           make_double2(__dadd_rn(l0.x, l1.x), __dadd_rn(l0.y, l1.y)));
+    __stcg(reinterpret_cast<double2*>(A.cs64 + 4 * q) + i,
+           make_double2(__dadd_rn(s0.x, s1.x), __dadd_rn(s0.y, s1.y)));
+  }
+  // (a cell shines if a half does: luminosities are not negative)
+  uint32_t has = (h0 | h1) & (kMetaHasAlpha | kMetaHasL);
+  if (h0 & kMetaHasAlpha) has |= kMetaChild0Alpha;
+  if (h1 & kMetaHasAlpha) has |= kMetaChild1Alpha;
+  __stcg(A.flags + q, has);
+}
+
+// Every other bit triple of a 63-bit key from bit `shift` on: one axis's 21 bits.
+__device__ __forceinline__ uint32_t compact3(uint64_t v, int shift) {
+  v = (v >> shift) & 0x1249249249249249ull;
+  v = (v ^ (v >> 2)) & 0x10c30c30c30c30c3ull;
+  v = (v ^ (v >> 4)) & 0x100f00f00f00f00full;
+  v = (v ^ (v >> 8)) & 0x1f0000ff0000ffull;
+  v = (v ^ (v >> 16)) & 0x1f00000000ffffull;
+  v = (v ^ (v >> 32)) & 0x1fffffull;
+  return uint32_t(v);
+}
+
+// A node's record, centre and B from its sums: independent of other nodes.
+__device__ __forceinline__ void finish_node(const TreeArgs& A, int64_t q) {
+  const int nbp = A.nbp;
+  const int d = A.depth[q], c = A.child[q];
+  const uint64_t prefix = A.prefix[q];
+  const uint32_t has = A.flags[q];
+  const double cs3 = A.cs64[q * 4 + 3];
+  double lo[3], cc[3], B2 = 0.0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = double(compact3(prefix, 2 - a)) * (1.0 / 2097152.0);
+    const double ext = __longlong_as_double((long long)(1023 - splits_on_axis(d, a)) << 52);
+    cc[a] = cs3 > 0.0 ? A.cs64[q * 4 + a] / cs3 : lo[a] + 0.5 * ext;
+    // B: the farthest box corner from the centre of luminosity (Sec. 2.5.2),
+    // the farther face on each axis
+    const double d0 = __dsub_rn(lo[a], cc[a]), d1 = __dsub_rn(lo[a] + ext, cc[a]);
+    B2 = __dadd_rn(B2, fmax(__dmul_rn(d0, d0), __dmul_rn(d1, d1)));
+    A.c64[3 * q + a] = cc[a];
+  }
+  const double B = sqrt(B2);
+  A.B64[q] = B;
+  for (int b = 0; b < nbp; ++b) A.Lnode[q * nbp + b] = float(A.L64[q * 4 + b]);
+  A.csrc[q] = make_float4(float(cc[0]), float(cc[1]), float(cc[2]), float(cs3));
+  if (c >= 0) {
+    A.lmask[q] = 0;
     for (int b = 0; b < nbp; ++b) A.alpha_leaf[q * nbp + b] = 0.0f;
   }
-  for (int a = 0; a < 4; ++a) __stcg(A.cs64 + q * 4 + a, cs[a]);
-  double cc[3];
-  for (int a = 0; a < 3; ++a) cc[a] = cs[3] > 0.0 ? cs[a] / cs[3] : lo[a] + 0.5 * ext[a];
-  if (cs[3] > 0.0) has |= kMetaHasL;
-  __stcg(A.flags + q, has);
-  A.lmask[q] = lit;
-  // B: farthest box corner from the centre of luminosity (Sec. 2.5.2)
-  double B2 = 0.0;
-  for (int corner = 0; corner < 8; ++corner) {
-    double r2 = 0.0;
-    for (int a = 0; a < 3; ++a) {
-      double p = ((corner >> a) & 1) ? lo[a] + ext[a] : lo[a];
-      double dd = __dsub_rn(p, cc[a]);
-      r2 = __dadd_rn(r2, __dmul_rn(dd, dd));
-    }
-    B2 = fmax(B2, r2);
-  }
-  double B = sqrt(B2);
-  for (int a = 0; a < 3; ++a) A.c64[3 * q + a] = cc[a];
-  A.B64[q] = B;
-  for (int b = 0; b < nbp; ++b) A.Lnode[q * nbp + b] = float(__ldcg(A.L64 + q * 4 + b));
-  A.csrc[q] = make_float4(float(cc[0]), float(cc[1]), float(cc[2]), float(cs[3]));
   NodeW w;
   w.lo[0] = float(lo[0]);
   w.lo[1] = float(lo[1]);
   w.lo[2] = float(lo[2]);
   w.B = float(B);
   w.child = c;
-  w.aux = c < 0 ? __ldcg(A.first + q) : __ldcg(A.int_index + q);
-  w.count = __ldcg(A.count + q);
+  w.aux = c < 0 ? A.first[q] : A.int_index[q];
+  w.count = A.count[q];
   w.meta = uint32_t(d) | (uint32_t(d % 3) << kMetaAxisShift) | (c < 0 ? kMetaLeaf : 0u) | has;
-  if (c >= 0) {
-    if (half0 & kMetaHasAlpha) w.meta |= kMetaChild0Alpha;
-    if (half1 & kMetaHasAlpha) w.meta |= kMetaChild1Alpha;
-  }
   A.nodes[q] = w;
 }
 
@@ -870,6 +920,16 @@ __global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_consta
           d = level;
           f = __ldcg(A.first + q);
           c = __ldcg(A.count + q);
+        }
+        if (le - lb <= 4 * kTreeThreads / 32) {  // few nodes, long searches: a warp each
+          __shared__ int s_mid[4 * kTreeThreads / 32];
+          for (int i = t >> 5; i < le - lb; i += kTreeThreads / 32) {
+            const int at = split_at_warp(A, level, __ldcg(A.first + lb + i), __ldcg(A.count + lb + i));
+            if ((t & 31) == 0) s_mid[i] = at;
+          }
+          __syncthreads();
+          if (q < le) m = s_mid[t];
+        } else if (q < le) {
           m = split_at(A, d, f, c);
         }
         int tile = 0;
@@ -997,10 +1057,16 @@ __global__ void __launch_bounds__(128) k_aggregate_leaves(const __grid_constant_
   const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (A.S->need || q >= A.S->n_nodes || A.child[q] >= 0) return;
   const double size = A.S->size;
-  aggregate_node(A, q, true, 1.0 / (size * size));
+  leaf_sums(A, q, 1.0 / (size * size));
 }
 
-__global__ void __launch_bounds__(kTreeThreads, 2) k_aggregate_inner(const __grid_constant__ TreeArgs A) {
+__global__ void __launch_bounds__(128) k_finish_nodes(const __grid_constant__ TreeArgs A) {
+  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (A.S->need || q >= A.S->n_nodes) return;
+  finish_node(A, q);
+}
+
+__global__ void __launch_bounds__(kTreeThreads, 2) k_sum_levels(const __grid_constant__ TreeArgs A) {
   BuildState* S = A.S;
   if (S->need) return;
   const int blocks = gridDim.x, t = threadIdx.x;
@@ -1009,7 +1075,6 @@ __global__ void __launch_bounds__(kTreeThreads, 2) k_aggregate_inner(const __gri
   for (int i = t; i < level; i += kTreeThreads) s_begin[i] = S->level_begin[i];
   if (t == 0) s_begin[level] = S->n_nodes;
   __syncthreads();
-  const double size = S->size, inv_size2 = 1.0 / (size * size);
   const int64_t stride = int64_t(blocks) * kTreeThreads, at = int64_t(blockIdx.x) * kTreeThreads + t;
   bool together = false;  // whether the depth below was done by all blocks
   for (int d = level - 2; d >= 0; --d) {
@@ -1022,11 +1087,9 @@ __global__ void __launch_bounds__(kTreeThreads, 2) k_aggregate_inner(const __gri
     }
     together = !small;
     if (small) {
-      if (blockIdx.x == 0 && t < b1 - b0 && __ldcg(A.child + b0 + t) >= 0)
-        aggregate_node(A, b0 + t, false, inv_size2);
+      if (blockIdx.x == 0 && t < b1 - b0) inner_sums(A, b0 + t);
     } else {
-      for (int64_t q = b0 + at; q < b1; q += stride)
-        if (__ldcg(A.child + q) >= 0) aggregate_node(A, q, false, inv_size2);
+      for (int64_t q = b0 + at; q < b1; q += stride) inner_sums(A, q);
     }
   }
 }
@@ -1209,8 +1272,10 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
     k_aggregate_leaves<<<blocks_for(cap, 128), 128, 0, st>>>(A);
     note_launch();
     T2_CUDA(cudaMemsetAsync(&state.p->bar, 0, sizeof(uint32_t), st));
-    T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_aggregate_inner),
+    T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_sum_levels),
                                         dim3(unsigned(blocks_inner)), dim3(kTreeThreads), args, 0, st));
+    note_launch();
+    k_finish_nodes<<<blocks_for(cap, 128), 128, 0, st>>>(A);
     note_launch();
     uint32_t hstatus = 0;
     T2_CUDA(cudaMemcpyAsync(&S, state.p, sizeof(S), cudaMemcpyDeviceToHost, st));

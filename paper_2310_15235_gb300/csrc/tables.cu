@@ -88,6 +88,7 @@ __device__ __forceinline__ void cube_vec(int f, float a, float b, float v[3]) {
 // place is the first class (rho up to sin of the cone half-angle acos(1 -
 // (c / kConeClasses)^2)) that has it, and a class's candidates are the first
 // ones of the list.
+template <int kGroups>
 __global__ void k_beam_map(int npix, int stride, int nf, const float4* __restrict__ dirs,
                            uint8_t* __restrict__ list, uint8_t* __restrict__ count,
                            float4* __restrict__ beam_inv) {
@@ -114,7 +115,6 @@ __global__ void k_beam_map(int npix, int stride, int nf, const float4* __restric
     cube_vec(f, -1.0f + (i + (q & 1)) * w, -1.0f + (j + (q >> 1)) * w, v);
     for (int a = 0; a < 3; ++a) wide[a] = fmaxf(wide[a], fabsf(v[a] - c[a]) + 1e-4f);
   }
-  constexpr int kGroups = (12 * kCellNside * kCellNside + 31) / 32;
   int first[kGroups];
 #pragma unroll
   for (int g = 0; g < kGroups; ++g) {
@@ -177,15 +177,16 @@ __device__ __forceinline__ float combine_alpha(float a1, float a2, float w1, flo
     if (w12 > 0.0f) S += w12 * expf(-(x12 - m));
     lnT = -m + logf(S);
   } else {
-    float S = 0.0f;
-    if (w1 > 0.0f) S += w1 * (expf(-x1) + expf(-x2));
-    if (w12 > 0.0f) S += w12 * expf(-x12);
-    if (S > 0.5f) {
-      float e = 0.0f;
-      if (w1 > 0.0f) e += w1 * (expm1f(-x1) + expm1f(-x2));
-      if (w12 > 0.0f) e += w12 * expm1f(-x12);
+    // sum_j w_j = 1, so T - 1 comes without T
+    float e = 0.0f;
+    if (w1 > 0.0f) e += w1 * (expm1f(-x1) + expm1f(-x2));
+    if (w12 > 0.0f) e += w12 * expm1f(-x12);
+    if (e > -0.5f) {
       lnT = log1pf(e);
     } else {
+      float S = 0.0f;
+      if (w1 > 0.0f) S += w1 * (expf(-x1) + expf(-x2));
+      if (w12 > 0.0f) S += w12 * expf(-x12);
       lnT = logf(S);
     }
   }
@@ -286,8 +287,10 @@ int ensure_beam_map(Table* tb, cudaStream_t st) {
                         inv_bytes + squares * (stride + kConeClasses + 1), st, "beam map"));
   uint8_t* list = map.p + inv_bytes;
   uint8_t* count = list + squares * stride;
-  k_beam_map<<<unsigned((squares + 7) / 8), 256, 0, st>>>(npix, stride, nf, tb->dirs, list, count,
-                                                          reinterpret_cast<float4*>(map.p));
+  // beams in groups of a warp's lanes: up to 64 (nside 1, 2) or 192 of them
+  const auto fn = npix <= 64 ? &k_beam_map<2> : &k_beam_map<6>;
+  fn<<<unsigned((squares + 7) / 8), 256, 0, st>>>(npix, stride, nf, tb->dirs, list, count,
+                                                  reinterpret_cast<float4*>(map.p));
   note_launch();
   T2_CUDA(cudaGetLastError());
   tb->beam_inv = reinterpret_cast<float4*>(map.p);
