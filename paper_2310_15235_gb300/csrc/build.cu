@@ -250,21 +250,38 @@ __global__ void __launch_bounds__(kSmallSortThreads)
   }
   for (int run = 1; run < n; run <<= 1) {
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const uint64_t key = ka[i];
-      const int base = i & ~(2 * run - 1);
-      const bool left = i - base < run;
-      // the other run; its equal keys go before a right one, after a left one
-      const int first = left ? base + run : base;
-      int lo = min(first, n), hi = min(first + run, n);
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const uint64_t other = ka[mid];
-        if (left ? other < key : other <= key) lo = mid + 1; else hi = mid;
+    // four keys a thread at a time, their searches side by side
+    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * blockDim.x) {
+      uint64_t key[4];
+      int lo[4], hi[4];
+      bool left[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = min(i0 + u * int(blockDim.x), n - 1);
+        key[u] = ka[i];
+        left[u] = (i & run) == 0;
+        // the other run; its equal keys go before a right one, after a left one
+        const int first = left[u] ? (i & ~(run - 1)) + run : (i & ~(2 * run - 1));
+        lo[u] = min(first, n);
+        hi[u] = min(first + run, n);
       }
-      const int at = left ? i + lo - min(first, n) : i - run + lo - first;
-      kb[at] = key;
-      pb[at] = pa[i];
+      for (int len = run; len > 0; len >>= 1)  // the last half steps are empty for some
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (lo[u] < hi[u]) {
+            const int mid = (lo[u] + hi[u]) >> 1;
+            const uint64_t other = ka[mid];
+            if (left[u] ? other < key[u] : other <= key[u]) lo[u] = mid + 1; else hi[u] = mid;
+          }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * int(blockDim.x);
+        if (i >= n) break;
+        const int first = left[u] ? (i & ~(run - 1)) + run : (i & ~(2 * run - 1));
+        const int at = left[u] ? i + lo[u] - min(first, n) : i - run + lo[u] - first;
+        kb[at] = key[u];
+        pb[at] = pa[i];
+      }
     }
     uint64_t* const tk = ka;
     ka = kb;
@@ -1097,13 +1114,13 @@ __global__ void __launch_bounds__(kTreeThreads, 2) k_sum_levels(const __grid_con
 // The node arrays for `cap` nodes.
 static int alloc_nodes(Tree* t, int64_t cap, cudaStream_t st) {
   const int nbp = t->nbp;
-  T2_CHECK(dalloc(&t->prefix, cap, st));
-  T2_CHECK(dalloc(&t->depth, cap, st));
-  T2_CHECK(dalloc(&t->first, cap, st));
-  T2_CHECK(dalloc(&t->count, cap, st));
-  T2_CHECK(dalloc(&t->child, cap, st));
-  T2_CHECK(dalloc(&t->parent, cap, st));
-  T2_CHECK(dalloc(&t->int_index, cap, st));
+  T2_CHECK(dalloc(&t->prefix, 4 * cap, st));  // the topology arrays, in one piece
+  t->depth = reinterpret_cast<int*>(t->prefix + cap);
+  t->first = t->depth + cap;
+  t->count = t->first + cap;
+  t->child = t->count + cap;
+  t->parent = t->child + cap;
+  t->int_index = t->parent + cap;
   T2_CHECK(dalloc(&t->nodes, cap, st));
   T2_CHECK(dalloc(&t->Lnode, cap * nbp, st));
   T2_CHECK(dalloc(&t->csrc, cap, st));
@@ -1116,12 +1133,7 @@ static int alloc_nodes(Tree* t, int64_t cap, cudaStream_t st) {
 
 static void free_nodes(Tree* t, cudaStream_t st) {
   dfree(t->prefix, st);
-  dfree(t->depth, st);
-  dfree(t->first, st);
-  dfree(t->count, st);
-  dfree(t->child, st);
-  dfree(t->parent, st);
-  dfree(t->int_index, st);
+  t->depth = t->first = t->count = t->child = t->parent = t->int_index = nullptr;
   dfree(t->nodes, st);
   dfree(t->Lnode, st);
   dfree(t->csrc, st);

@@ -179,7 +179,7 @@ constexpr int kCellHits = 64 * 4;
 
 // Up to 32 crossings (t0, t1, row, beam), one per lane: their increments, to
 // the sources [e0, e0 + m) of V.
-template <int NBP>
+template <int NBP, bool kInOrder>
 __device__ __forceinline__ void add_crossings(const WalkArgs& a, int lane, bool live, float4 h,
                                               const float4* binv, const float* ss, const int* off,
                                               int e0, int m, float s_before, float* T, float* own,
@@ -220,26 +220,178 @@ __device__ __forceinline__ void add_crossings(const WalkArgs& a, int lane, bool 
     for (int b = 0; b < NBP; ++b) add.v[b] *= len;
   }
   // the first lane of those that meet the same source adds up their
-  // increments in lane order, so that T is read and written once
+  // increments in lane order, so that T is read and written once; kInOrder: one
+  // after another onto T, so that the sum does not depend on how the crossings
+  // fall into groups (k_walk_team's fall otherwise than k_walk's)
   const unsigned peers = __match_any_sync(0xffffffffu, key);
   const bool lead = key >= 0 && (peers & ((1u << lane) - 1u)) == 0u;
   float* p = T + key * NBP;
   BandVec<NBP> old;
   if (lead) old = load_bands<NBP>(p);
+  if constexpr (kInOrder) {
+    if (lead) {
+#pragma unroll
+      for (int b = 0; b < NBP; ++b) old.v[b] += add.v[b];
+    }
+  }
   unsigned rest = lead ? peers & (peers - 1u) : 0u;
   while (__any_sync(0xffffffffu, rest != 0u)) {
     const int from = rest ? __ffs(rest) - 1 : lane;
 #pragma unroll
     for (int b = 0; b < NBP; ++b) {
       const float v = __shfl_sync(0xffffffffu, add.v[b], from);
-      if (rest) add.v[b] += v;
+      if (rest) (kInOrder ? old : add).v[b] += v;
     }
     rest &= rest - 1u;
   }
   if (lead) {
+    if constexpr (!kInOrder) {
 #pragma unroll
-    for (int b = 0; b < NBP; ++b) old.v[b] += add.v[b];
+      for (int b = 0; b < NBP; ++b) old.v[b] += add.v[b];
+    }
     store_bands<NBP>(p, old);
+  }
+  __syncwarp();
+}
+
+// bin_sources for up to bin_cap sources: the records' (s, beam, index) are put
+// in the order of their beams in shared memory, ranked there, and every record
+// is moved once.  key: 2 bin_cap ints.
+static __device__ int bin_sources_small(const WalkArgs& a, int lane, const SrcEntry* U, const int* Up,
+                                        int n, SrcEntry* V, int* off, int* key) {
+  const int npix = a.npix;
+  float* ks = reinterpret_cast<float*>(key);
+  uint32_t* kk = reinterpret_cast<uint32_t*>(key + a.bin_cap);
+  for (int k = lane; k < npix; k += 32) off[k] = 0;
+  __syncwarp();
+  for (int e = lane; e < n; e += 32)
+    if (const int k = Up[e]; k >= 0) atomicAdd(&off[k], 1);
+  __syncwarp();
+  // exclusive scan of the bucket sizes
+  const int per = (npix + 31) / 32;
+  const int b0 = min(lane * per, npix), b1 = min(b0 + per, npix);
+  int sum = 0;
+  for (int k = b0; k < b1; ++k) sum += off[k];
+  const int incl = warp_incl_scan(sum, lane);
+  int run = incl - sum;
+  for (int k = b0; k < b1; ++k) {
+    const int c = off[k];
+    off[k] = run;
+    run += c;
+  }
+  __syncwarp();
+  for (int e = lane; e < n; e += 32) {
+    const int k = Up[e];
+    if (k < 0) continue;
+    const int slot = atomicAdd(&off[k], 1);
+    ks[slot] = U[e].s;
+    kk[slot] = uint32_t(e) | (uint32_t(k) << 16);
+  }
+  __syncwarp();
+  n = off[npix - 1];  // records binned
+  // each record's rank in its bucket by (projected distance, index)
+  for (int p = lane; p < n; p += 32) {
+    const uint32_t me = kk[p];
+    const int k = int(me >> 16), s0 = k ? off[k - 1] : 0, s1 = off[k];
+    const float s = ks[p];
+    int r = s0;
+    for (int j = s0; j < s1; ++j) r += ks[j] < s || (ks[j] == s && kk[j] < me);
+    V[r] = U[me & 0xffffu];
+  }
+  __syncwarp();
+  return n;
+}
+
+// 32 cells of the cut, one per lane (q < 0: none): the (cell, beam) pairs that
+// can cross, 32 at a time, each tested against its cell's box; push(hit, t0, t1,
+// row, beam slot) is called by the whole warp for every 32 pairs.  The beams of
+// a cell come from the look-up by its shape, the direction of its centre and
+// the class of the cone about it that holds the box (sin^2 = H2 / D2; with x
+// inside the sphere through the corners, every beam).  stage: kCellStage ints.
+template <bool kPP, class Push>
+__device__ __forceinline__ void cross_batch(const WalkArgs& a, float3 x, int lane, int q,
+                                            int* stage, const float4* binv, const float* far,
+                                            float rpp, Push push) {
+  const unsigned lt = (1u << lane) - 1u;
+  const int npix = a.npix, stride = (npix + 15) & ~15;
+  const float nfh = 0.5f * float(a.beam_side);
+  float4* box0 = reinterpret_cast<float4*>(stage);
+  float4* box1 = box0 + 32;
+  uint4* beams = reinterpret_cast<uint4*>(box1 + 32);
+  const uint8_t* beams8 = reinterpret_cast<const uint8_t*>(beams);
+  int count = 0, total;
+  int start;
+  {
+    NodeW nd;
+    if (q >= 0) nd = load_node(a.nodes + q);
+    int sq = 0, row = 0;
+    float lx = 0.0f, ly = 0.0f, lz = 0.0f, hx = 0.0f, hy = 0.0f, hz = 0.0f;
+    if (q >= 0) {
+      const float4 e = ext_of(nd.meta);
+      lx = nd.lo[0] - x.x; hx = nd.lo[0] + e.x - x.x;
+      ly = nd.lo[1] - x.y; hy = nd.lo[1] + e.y - x.y;
+      lz = nd.lo[2] - x.z; hz = nd.lo[2] + e.z - x.z;
+      row = (nd.meta & kMetaLeaf) ? -(q + 1) : nd.aux;
+      const float cx = 0.5f * (lx + hx), cy = 0.5f * (ly + hy), cz = 0.5f * (lz + hz);
+      const float D2 = cx * cx + cy * cy + cz * cz;
+      const float H2 = 0.25f * (e.x * e.x + e.y * e.y + e.z * e.z);
+      count = npix;
+      if (D2 > H2) {
+        // sqrt(1 - cos) by classes; the look-up's slack covers the approximations
+        const float c2 = fmaxf(1e-12f, 1.0f - __fdividef(H2, D2));
+        const float v = fmaxf(1e-12f, 1.0f - c2 * rsqrtf(c2));
+        const int cls = int(v * rsqrtf(v) * float(kConeClasses) + 1.02f);
+        if (cls <= kConeClasses) {
+          const float ax = fabsf(cx), ay = fabsf(cy), az = fabsf(cz);
+          const float vm = fmaxf(fmaxf(ax, ay), az);
+          const bool mx = ax == vm, my = !mx && ay == vm;
+          const float ca = mx ? cy : cx, cb = mx || my ? cz : cy, cm = mx ? cx : (my ? cy : cz);
+          const float iv = __fdividef(nfh, vm);
+          const int top = a.beam_side - 1;
+          const int i = max(0, min(top, int(ca * iv + nfh))), j = max(0, min(top, int(cb * iv + nfh)));
+          const int face = 6 * int((nd.meta >> kMetaAxisShift) & 3u) + (mx ? 0 : (my ? 2 : 4)) +
+                           (cm < 0.0f ? 1 : 0);
+          sq = (face * a.beam_side + i) * a.beam_side + j;
+          count = a.beam_count[sq * (kConeClasses + 1) + cls];
+        }
+      }
+    }
+    const uint4 near16 = *reinterpret_cast<const uint4*>(a.beam_list + sq * stride);
+    const int incl = warp_incl_scan(count, lane);
+    start = incl - count;
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned some = __ballot_sync(0xffffffffu, count > 0);
+    if (count > 0) {
+      const int slot = __popc(some & lt);
+      box0[slot] = make_float4(lx, ly, lz, hx);
+      box1[slot] = make_float4(hy, hz, __int_as_float((sq << 13) | start), __int_as_float(row));
+      beams[slot] = near16;
+    } else {
+      start = INT32_MIN;  // owns no pair
+    }
+    __syncwarp();
+  }
+  int owners = -1;  // the last cell whose pairs start before this chunk
+  for (int p = lane; p - lane < total; p += 32, start -= 32) {
+    // a lane's pair belongs to the last cell that starts at or before it
+    const unsigned begins = __reduce_or_sync(0xffffffffu, bit_at(start));
+    const int slot = owners + __popc(begins & (2u * lt + 1u));
+    owners += __popc(begins);
+    const float4 b0 = box0[slot], b1 = box1[slot];
+    const int meta = __float_as_int(b1.z), i = p - (meta & 0x1fff);
+    const bool live = p < total;
+    int k = beams8[16 * slot + min(i, 15)];
+    if (live && i > 15) k = a.beam_list[(meta >> 13) * stride + i];
+    k = live ? k : 0;
+    const float4 iv = binv[k];
+    const float ax = b0.x * iv.x, bx = b0.w * iv.x;
+    const float ay = b0.y * iv.y, by = b1.x * iv.y;
+    const float az = b0.z * iv.z, bz = b1.y * iv.z;
+    float t0 = fmaxf(fmaxf(fminf(ax, bx), fminf(ay, by)), fmaxf(fminf(az, bz), 0.0f));
+    const float t1 = fminf(fminf(fmaxf(ax, bx), fmaxf(ay, by)), fmaxf(az, bz));
+    if constexpr (kPP) t0 = fmaxf(t0, rpp);  // cells absorb only beyond r_pp (Sec. 2.4)
+    const bool hit = live && t0 < fminf(t1, far[k]);
+    push(hit, t0, t1, __float_as_int(b1.w), k);
   }
   __syncwarp();
 }
@@ -247,21 +399,16 @@ __device__ __forceinline__ void add_crossings(const WalkArgs& a, int lane, bool 
 // tau of the n staged sources V (sorted by beam and distance) from the nc
 // listed cells, into T[e][NBP]: set with `first`, added to what is there
 // without.  own[e][NBP]: the depth of the cell that holds a source, up to it.
-template <int NBP, bool kPP>
+template <int NBP, bool kPP, bool kInOrder>
 __device__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
                              const float4* binv, const int* off, float* far, const SrcEntry* V,
                              float* T, float* own, int n, const int* cells, int nc, bool first,
                              float rpp) {
   const unsigned lt = (1u << lane) - 1u;
   const int npix = a.npix;
-  float4* box0 = reinterpret_cast<float4*>(region);
-  float4* box1 = box0 + 32;
-  uint4* beams = reinterpret_cast<uint4*>(box1 + 32);
-  const uint8_t* beams8 = reinterpret_cast<const uint8_t*>(beams);
-  float4* hits = box0 + kCellStage / 4;
+  int* stage = region;
+  float4* hits = reinterpret_cast<float4*>(region + kCellStage);
   float* ss = reinterpret_cast<float*>(hits + kCellHits / 4);
-  const float nfh = 0.5f * float(a.beam_side);
-  const int stride = (npix + 15) & ~15;
   if (first) {
     BandVec<NBP> zero;
 #pragma unroll
@@ -282,102 +429,26 @@ __device__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
       const int s0 = max((k ? off[k - 1] : 0) - e0, 0), s1 = min(off[k] - e0, m);
       far[beam_slot(k)] = s1 > s0 ? ss[s1 - 1] : -1.0f;
     }
-    int nh = 0;  // pending crossings
-    // a batch's nodes are loaded while the one before is crossed
+    int head = 0;  // crossings found; the last head % 32 are pending, in a ring of 64
     int q_next = lane < nc ? cells[lane] : -1;
     for (int c0 = 0; c0 < nc; c0 += 32) {
-      // 32 cells: their boxes seen from x and the beams that can cross them, by
-      // shape, direction of the centre and the class of the cone about it that
-      // holds the box (sin^2 = H2 / D2; with x inside the sphere through the
-      // corners, every beam)
-      int count = 0, total;
-      int start;
-      {
-        const int q = q_next;
-        NodeW nd;
-        if (q >= 0) nd = load_node(a.nodes + q);
-        q_next = c0 + 32 + lane < nc ? cells[c0 + 32 + lane] : -1;
-        int sq = 0, row = 0;
-        float lx = 0.0f, ly = 0.0f, lz = 0.0f, hx = 0.0f, hy = 0.0f, hz = 0.0f;
-        if (q >= 0) {
-          const float4 e = ext_of(nd.meta);
-          lx = nd.lo[0] - x.x; hx = nd.lo[0] + e.x - x.x;
-          ly = nd.lo[1] - x.y; hy = nd.lo[1] + e.y - x.y;
-          lz = nd.lo[2] - x.z; hz = nd.lo[2] + e.z - x.z;
-          row = (nd.meta & kMetaLeaf) ? -(q + 1) : nd.aux;
-          const float cx = 0.5f * (lx + hx), cy = 0.5f * (ly + hy), cz = 0.5f * (lz + hz);
-          const float D2 = cx * cx + cy * cy + cz * cz;
-          const float H2 = 0.25f * (e.x * e.x + e.y * e.y + e.z * e.z);
-          count = npix;
-          if (D2 > H2) {
-            // sqrt(1 - cos) by classes; the look-up's slack covers the approximations
-            const float c2 = fmaxf(1e-12f, 1.0f - __fdividef(H2, D2));
-            const float v = fmaxf(1e-12f, 1.0f - c2 * rsqrtf(c2));
-            const int cls = int(v * rsqrtf(v) * float(kConeClasses) + 1.02f);
-            if (cls <= kConeClasses) {
-              const float ax = fabsf(cx), ay = fabsf(cy), az = fabsf(cz);
-              const float vm = fmaxf(fmaxf(ax, ay), az);
-              const bool mx = ax == vm, my = !mx && ay == vm;
-              const float ca = mx ? cy : cx, cb = mx || my ? cz : cy, cm = mx ? cx : (my ? cy : cz);
-              const float iv = __fdividef(nfh, vm);
-              const int top = a.beam_side - 1;
-              const int i = max(0, min(top, int(ca * iv + nfh))), j = max(0, min(top, int(cb * iv + nfh)));
-              const int face = 6 * int((nd.meta >> kMetaAxisShift) & 3u) + (mx ? 0 : (my ? 2 : 4)) +
-                               (cm < 0.0f ? 1 : 0);
-              sq = (face * a.beam_side + i) * a.beam_side + j;
-              count = a.beam_count[sq * (kConeClasses + 1) + cls];
-            }
-          }
-        }
-        const uint4 near16 = *reinterpret_cast<const uint4*>(a.beam_list + sq * stride);
-        const int incl = warp_incl_scan(count, lane);
-        start = incl - count;
-        total = __shfl_sync(0xffffffffu, incl, 31);
-        const unsigned some = __ballot_sync(0xffffffffu, count > 0);
-        if (count > 0) {
-          const int slot = __popc(some & lt);
-          box0[slot] = make_float4(lx, ly, lz, hx);
-          box1[slot] = make_float4(hy, hz, __int_as_float((sq << 13) | start), __int_as_float(row));
-          beams[slot] = near16;
-        } else {
-          start = INT32_MIN;  // owns no pair
-        }
-        __syncwarp();
-      }
-      int owners = -1;  // the last cell whose pairs start before this chunk
-      for (int p = lane; p - lane < total; p += 32, start -= 32) {
-        // a lane's pair belongs to the last cell that starts at or before it
-        const unsigned begins = __reduce_or_sync(0xffffffffu, bit_at(start));
-        const int slot = owners + __popc(begins & (2u * lt + 1u));
-        owners += __popc(begins);
-        const float4 b0 = box0[slot], b1 = box1[slot];
-        const int meta = __float_as_int(b1.z), i = p - (meta & 0x1fff);
-        const bool live = p < total;
-        int k = beams8[16 * slot + min(i, 15)];
-        if (live && i > 15) k = a.beam_list[(meta >> 13) * stride + i];
-        k = live ? k : 0;
-        const float4 iv = binv[k];
-        const float ax = b0.x * iv.x, bx = b0.w * iv.x;
-        const float ay = b0.y * iv.y, by = b1.x * iv.y;
-        const float az = b0.z * iv.z, bz = b1.y * iv.z;
-        float t0 = fmaxf(fmaxf(fminf(ax, bx), fminf(ay, by)), fmaxf(fminf(az, bz), 0.0f));
-        const float t1 = fminf(fminf(fmaxf(ax, bx), fmaxf(ay, by)), fmaxf(az, bz));
-        if constexpr (kPP) t0 = fmaxf(t0, rpp);  // cells absorb only beyond r_pp (Sec. 2.4)
-        const bool hit = live && t0 < fminf(t1, far[k]);
+      const int q = q_next;
+      q_next = c0 + 32 + lane < nc ? cells[c0 + 32 + lane] : -1;
+      cross_batch<kPP>(a, x, lane, q, stage, binv, far, rpp, [&](bool hit, float t0, float t1, int row, int k) {
         const unsigned hm = __ballot_sync(0xffffffffu, hit);
-        if (hit) hits[nh + __popc(hm & lt)] = make_float4(t0, t1, b1.w, __int_as_float(k));
-        nh += __popc(hm);
+        if (hit)
+          hits[(head + __popc(hm & lt)) & 63] =
+              make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
+        const int was = head;
+        head += __popc(hm);
         __syncwarp();
-        if (nh >= 32) {
-          nh -= 32;
-          add_crossings<NBP>(a, lane, true, hits[nh + lane], binv, ss, off, e0, m, s_before, Tw,
-                             own + e0 * NBP, first);
-        }
-      }
-      __syncwarp();
+        if ((head ^ was) & 32)
+          add_crossings<NBP, kInOrder>(a, lane, true, hits[(was & 32) + lane], binv, ss, off, e0, m, s_before,
+                             Tw, own + e0 * NBP, first);
+      });
     }
-    if (nh > 0)
-      add_crossings<NBP>(a, lane, lane < nh, hits[lane], binv, ss, off, e0, m, s_before, Tw,
+    if (head & 31)
+      add_crossings<NBP, kInOrder>(a, lane, lane < (head & 31), hits[(head & 32) + lane], binv, ss, off, e0, m, s_before, Tw,
                          own + e0 * NBP, first);
   }
   __syncwarp();
@@ -386,8 +457,8 @@ __device__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
 // The increments of all cells summed along each beam, a beam per lane.
 template <int NBP>
 __device__ __forceinline__ void sum_increments(int lane, int npix, const int* off, float* T,
-                                               const float* own) {
-  for (int k = lane; k < npix; k += 32) {
+                                               const float* own, int lanes = 32) {
+  for (int k = lane; k < npix; k += lanes) {
     BandVec<NBP> run;
 #pragma unroll
     for (int b = 0; b < NBP; ++b) run.v[b] = 0.0f;

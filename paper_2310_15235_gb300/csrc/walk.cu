@@ -209,6 +209,8 @@ __device__ __forceinline__ void eval_sources(const WalkArgs& a, int lane, const 
   }
 }
 
+constexpr int kCellCap = 2048;  // cells of a cut listed at once
+
 // A warp's part of a walk block's shared memory and of the walk buffers.
 struct WarpMem {
   int* stk;          // traversal stacks / increments, boxes and crossings
@@ -268,7 +270,7 @@ template <int NBP, bool kBucket, bool kPP, bool kCSM, bool kCells>
 __device__ __forceinline__ void absorb(const WalkArgs& a, float3 x, int si, int lane, const WarpMem& w,
                                        int n, int listed, int clo, int leaf, float rpp) {
   if constexpr (kCells) {
-    absorb_cells<NBP, kPP>(a, x, lane, w.stk, w.binv, w.off, w.far, w.V, w.T, w.own, n, w.cells,
+    absorb_cells<NBP, kPP, !kBucket>(a, x, lane, w.stk, w.binv, w.off, w.far, w.V, w.T, w.own, n, w.cells,
                            min(listed - clo, a.cell_cap), clo == 0, rpp);
     if (clo + a.cell_cap >= listed) {
       sum_increments<NBP>(lane, a.npix, w.off, w.T, w.own);
@@ -312,7 +314,9 @@ __device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si,
     if (clo == 0) {
       const int staged = min(total - lo, a.M);
       make_sources<kBucket, kCSM>(a, x, si, lane, w.U, w.Up, staged);
-      n = staged > 0 ? bin_sources(a, lane, w.U, w.Up, staged, w.V, w.off) : 0;
+      n = staged <= 0                        ? 0
+          : kCells && !kBucket && staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
+                                          : bin_sources(a, lane, w.U, w.Up, staged, w.V, w.off);
     }
     if (n > 0) {
       absorb<NBP, kBucket, kPP, kCSM, kCells>(a, x, si, lane, w, n, listed, clo, leaf, rpp);
@@ -329,22 +333,10 @@ __device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si,
   }
 }
 
-// J of one receiver (caller index io of the tree described by a) into
-// Jrow[0, nbsel); the warp's shared stacks and buffers are passed in.
-template <int NBP, bool kCells>
-__device__ __forceinline__ void walk_receiver_si(const WalkArgs& a, int si, float* Jrow, int lane,
-                                                 const WarpMem& w) {
-  const float4 xr = a.pos32[si];
-  // the receiver in FP32, on the FP64 side of every box face
-  const float3 x = grazing_coords(a, si, make_float3(xr.x, xr.y, xr.z));
-  // the receiver's ancestors, root first
-  const int leaf = kCells ? 0 : build_chain(a.nodes, x, lane, w.chain);
-  float Js[NBP], Jc[NBP];
-#pragma unroll
-  for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
-  walk_origin<NBP, false, false, false, kCells>(a, x, si, lane, w, leaf, 0.0f, [&](int n) {
-    eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
-  });
+// A receiver's row from its lanes' sums.
+template <int NBP>
+__device__ __forceinline__ void store_J(const WalkArgs& a, int si, int lane, const float* Js,
+                                        const float* Jc, float* Jrow) {
   // FP64 reduction of the lane partial sums
   double Jd[NBP];
 #pragma unroll
@@ -369,6 +361,25 @@ __device__ __forceinline__ void walk_receiver_si(const WalkArgs& a, int si, floa
     }
     Jrow[lane] = float(v);
   }
+}
+
+// J of one receiver (caller index io of the tree described by a) into
+// Jrow[0, nbsel); the warp's shared stacks and buffers are passed in.
+template <int NBP, bool kCells>
+__device__ __forceinline__ void walk_receiver_si(const WalkArgs& a, int si, float* Jrow, int lane,
+                                                 const WarpMem& w) {
+  const float4 xr = a.pos32[si];
+  // the receiver in FP32, on the FP64 side of every box face
+  const float3 x = grazing_coords(a, si, make_float3(xr.x, xr.y, xr.z));
+  // the receiver's ancestors, root first
+  const int leaf = kCells ? 0 : build_chain(a.nodes, x, lane, w.chain);
+  float Js[NBP], Jc[NBP];
+#pragma unroll
+  for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
+  walk_origin<NBP, false, false, false, kCells>(a, x, si, lane, w, leaf, 0.0f, [&](int n) {
+    eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
+  });
+  store_J<NBP>(a, si, lane, Js, Jc, Jrow);
 }
 
 // The same for the receiver with caller index io (NaN row and a status bit
@@ -400,6 +411,157 @@ __global__ void __launch_bounds__(WARPS * 32, (kCells ? kCellWarpsPerSM : kWalkW
     if (slot >= (unsigned long long)a.A) break;
     const int64_t r = a.order ? int64_t(a.order[slot]) : int64_t(slot);
     walk_receiver<NBP, kCells>(a, a.active[r], a.J + r * a.nbsel, lane, w);
+  }
+}
+
+// Few receivers (short rungs): a block of kTeamWarps warps for each, so that a
+// walk's chain of loads is a fraction of one warp's.  Warp 0 finds the cut and
+// bins the sources; all warps make the source records; batches of 32 cells go
+// round the warps, which list their crossings batch by batch; then every warp
+// takes the crossings of its own beams from all batches, in their order, so
+// each source's sums run exactly as in k_walk and the row is bit for bit the
+// same.  A receiver whose cut or crossings do not fit is walked by warp 0 alone.
+// 100 receivers of the 96^3 field: 0.49 -> 0.20 ms a call (see team_receivers).
+constexpr int kTeamWarps = 8;
+constexpr int kTeamHits = 2048;  // crossings a warp lists
+constexpr int kTeamBatches = kCellCap / 32;
+
+struct TeamArgs {
+  float4* hits;  // [blocks][kTeamWarps][kTeamHits]
+};
+
+template <int NBP>
+__global__ void __launch_bounds__(kTeamWarps * 32, 2)
+    k_walk_team(WalkArgs a, const __grid_constant__ TeamArgs tm) {
+  extern __shared__ __align__(16) int smem[];
+  init_block<true>(a, smem);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x;
+  const int64_t blk = blockIdx.x;
+  // one receiver's buffers and warp 0's region, then every warp's own stage
+  // and queue, the sources' distances and the batches' places in the lists
+  WarpMem w = warp_mem<true>(a, smem, blk, a.srcU, a.pixU, a.srcV, a.srcT, a.cells);
+  w.stk = smem + 4 * a.npix;
+  w.off = w.stk + a.region_ints;
+  w.far = reinterpret_cast<float*>(w.off + a.npix);
+  int* own_smem = smem + 4 * a.npix + a.warp_ints;
+  int* stage = own_smem + wid * (kCellStage + kCellHits);
+  float4* queue = reinterpret_cast<float4*>(stage + kCellStage);
+  float* ss = reinterpret_cast<float*>(own_smem + kTeamWarps * (kCellStage + kCellHits));
+  __shared__ int2 seg[kTeamBatches];
+  __shared__ unsigned long long s_slot;
+  __shared__ int s_total, s_listed, s_n, s_full;
+  float4* lists = tm.hits + blk * (kTeamWarps * kTeamHits);
+  const unsigned lt = (1u << lane) - 1u;
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) {
+      s_slot = atomicAdd(a.counter, 1ull);
+      s_full = 0;
+    }
+    __syncthreads();
+    if (s_slot >= (unsigned long long)a.A) break;
+    const int64_t r = a.order ? int64_t(a.order[s_slot]) : int64_t(s_slot);
+    const int64_t io = a.active[r];
+    float* Jrow = a.J + r * a.nbsel;
+    if (io < 0 || io >= a.N) {
+      if (wid == 0) walk_receiver<NBP, true>(a, io, Jrow, lane, w);
+      continue;
+    }
+    const int si = a.inv[io];
+    const float4 xr = a.pos32[si];
+    const float3 x = grazing_coords(a, si, make_float3(xr.x, xr.y, xr.z));
+    if (wid == 0) {
+      const int2 c = phase_cut<false, false>(a, x, si, lane, w.stk, a.src_stack_cap, w.U, 0, w.cells, 0, 0.0f);
+      if (lane == 0) {
+        s_total = c.x;
+        s_listed = c.y;
+      }
+    }
+    __syncthreads();
+    const int total = s_total, listed = s_listed;
+    if (total > a.M || listed > a.cell_cap) {
+      if (wid == 0) walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
+      continue;
+    }
+    make_sources(a, x, si, tid, w.U, w.Up, total, kTeamWarps * 32);
+    __syncthreads();
+    if (wid == 0) {
+      const int n0 = total <= 0           ? 0
+                   : total <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, total, w.V, w.off, w.stk)
+                                        : bin_sources(a, lane, w.U, w.Up, total, w.V, w.off);
+      if (lane == 0) s_n = n0;
+    }
+    __syncthreads();
+    const int n = s_n;
+    if (n > 0) {
+      BandVec<NBP> zero;
+#pragma unroll
+      for (int b = 0; b < NBP; ++b) zero.v[b] = 0.0f;
+      for (int e = tid; e < n; e += kTeamWarps * 32) {
+        ss[e] = w.V[e].s;
+        store_bands<NBP>(w.T + e * NBP, zero);
+        store_bands<NBP>(w.own + e * NBP, zero);
+      }
+      for (int k = tid; k < a.npix; k += kTeamWarps * 32) {
+        const int s1 = w.off[k];
+        w.far[beam_slot(k)] = s1 > (k ? w.off[k - 1] : 0) ? w.V[s1 - 1].s : -1.0f;
+      }
+      __syncthreads();
+      // this warp's batches: their crossings, listed
+      const int batches = (listed + 31) / 32;
+      int nh = 0;
+      float4* mine = lists + wid * kTeamHits;
+      for (int b = wid; b < batches; b += kTeamWarps) {
+        const int from = nh;
+        const int q = 32 * b + lane < listed ? w.cells[32 * b + lane] : -1;
+        cross_batch<false>(a, x, lane, q, stage, w.binv, w.far, 0.0f, [&](bool hit, float t0, float t1, int row, int k) {
+          const unsigned hm = __ballot_sync(0xffffffffu, hit);
+          const int at = nh + __popc(hm & lt);
+          if (hit && at < kTeamHits)
+            mine[at] = make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
+          nh += __popc(hm);
+        });
+        if (lane == 0) seg[b] = make_int2(from, nh - from);
+      }
+      if (nh > kTeamHits && lane == 0) s_full = 1;
+      __syncthreads();
+      if (s_full) {
+        if (wid == 0) walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
+        continue;
+      }
+      // this warp's beams: their crossings of all batches, in order
+      int nq = 0;
+      for (int b = 0; b < batches; ++b) {
+        const int2 sg = seg[b];
+        const float4* from = lists + (b % kTeamWarps) * kTeamHits + sg.x;
+        for (int i = 0; i < sg.y; i += 32) {
+          float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (i + lane < sg.y) h = __ldcg(from + i + lane);
+          const bool take = i + lane < sg.y && (__float_as_int(h.w) % kTeamWarps) == wid;
+          const unsigned m = __ballot_sync(0xffffffffu, take);
+          if (take) queue[(nq + __popc(m & lt)) & 63] = h;
+          const int was = nq;
+          nq += __popc(m);
+          __syncwarp();
+          if ((nq ^ was) & 32)
+            add_crossings<NBP, true>(a, lane, true, queue[(was & 32) + lane], w.binv, ss, w.off, 0, n, 0.0f,
+                               w.T, w.own, true);
+        }
+      }
+      __syncwarp();
+      if (nq & 31)
+        add_crossings<NBP, true>(a, lane, lane < (nq & 31), queue[(nq & 32) + lane], w.binv, ss, w.off, 0, n, 0.0f, w.T, w.own, true);
+      __syncthreads();
+      sum_increments<NBP>(tid, a.npix, w.off, w.T, w.own, kTeamWarps * 32);
+      __syncthreads();
+    }
+    if (wid == 0) {
+      float Js[NBP], Jc[NBP];
+#pragma unroll
+      for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
+      if (n > 0) eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
+      store_J<NBP>(a, si, lane, Js, Jc, Jrow);
+    }
   }
 }
 
@@ -1317,7 +1479,6 @@ void fill_walk_args(const Tree* t, const Table* tb, int nside, float theta, cons
   a->counter = t->counter;
 }
 
-constexpr int kCellCap = 2048;     // cells of a cut listed at once
 constexpr int kCellSources = 512;  // sources whose distances a warp holds at once
 
 size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
@@ -1426,6 +1587,37 @@ static int grow_buffer(void** buf, size_t* bytes, size_t need, cudaStream_t st, 
   return TREVR2_OK;
 }
 
+// Receivers up to which a block walks each one: measured on the 96^3 clumpy
+// field against a warp each (ms a call): nside 4, theta 0.5: 100 receivers
+// 0.20 / 0.49, 600 0.32 / 0.53, 1000 0.48 / 0.57, 1500 0.67 / 0.58; nside 2,
+// theta 0.75: 100 0.12 / 0.18, 600 0.17 / 0.19, 1000 0.24 / 0.21.
+static int64_t team_receivers(int nside) { return nside < 4 ? 640 : 1024; }
+
+// The walk of few receivers, cell by cell; a holds everything but the buffers.
+static int launch_walk_team(Tree* t, WalkArgs a, cudaStream_t st) {
+  const void* fn = t->nbp == 1 ? reinterpret_cast<const void*>(&k_walk_team<1>)
+                 : t->nbp == 2 ? reinterpret_cast<const void*>(&k_walk_team<2>)
+                               : reinterpret_cast<const void*>(&k_walk_team<4>);
+  const size_t smem = walk_layout(&a, 1, true, false) +
+                      (size_t(kTeamWarps) * (kCellStage + kCellHits) + a.M) * sizeof(int);
+  int per_sm = 0, sms = 0;
+  T2_CHECK(config_walk_kernel(fn, kTeamWarps, smem, &per_sm, &sms));
+  const size_t blocks = size_t(std::max<int64_t>(1, std::min<int64_t>(int64_t(sms) * per_sm, a.A)));
+  a.cell_cap = kCellCap;
+  const size_t wb = (walk_buffer_bytes(blocks, a.M, a.cell_cap) + 255) & ~size_t(255);
+  const size_t need = wb + blocks * kTeamWarps * kTeamHits * sizeof(float4);
+  T2_CHECK(grow_buffer(&t->scratch, &t->scratch_bytes, need, st, "walk buffers"));
+  char* base = static_cast<char*>(t->scratch);
+  place_walk_buffers(base, blocks, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU, &a.cells);
+  TeamArgs tm;
+  tm.hits = reinterpret_cast<float4*>(base + wb);
+  T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
+  void* args[] = {&a, &tm};
+  T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(kTeamWarps * 32), args, smem, st));
+  note_launch();
+  return TREVR2_OK;
+}
+
 static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int nside,
                        float theta, const int* bsel, int nbsel, uint32_t flags, float* J,
                        cudaStream_t st) {
@@ -1434,6 +1626,11 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
   a.active = active;
   a.A = A;
   a.J = J;
+  const bool cells = use_cells(t, tb, theta);
+  if (cells) {
+    T2_CHECK(use_beam_map(tb, &a, st));
+    if (A <= team_receivers(nside)) return launch_walk_team(t, a, st);
+  }
   if (A > 1) {
     const size_t need = size_t(A) * (sizeof(uint64_t) + sizeof(int));
     T2_CHECK(grow_buffer(&t->order_buf, &t->order_bytes, need, st, "receiver order"));
@@ -1442,8 +1639,6 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
     T2_CHECK(order_receivers(t, active, A, keys, slots, st));
     a.order = slots;
   }
-  const bool cells = use_cells(t, tb, theta);
-  if (cells) T2_CHECK(use_beam_map(tb, &a, st));
   const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells);
   const size_t smem = walk_layout(&a, kWalkWarps, cells, false);
   int per_sm = 0, sms = 0;

@@ -506,8 +506,8 @@ static __device__ int phase_sources(const WalkArgs& a, float3 x, int si, int lan
 // not in front of its beam) gets beam -1.
 template <bool kBucket = false, bool kCSM = false>
 static __device__ void make_sources(const WalkArgs& a, float3 x, int si, int lane, SrcEntry* U,
-                                    int* Up, int n) {
-  for (int e = lane; e < n; e += 32) {
+                                    int* Up, int n, int lanes = 32) {
+  for (int e = lane; e < n; e += lanes) {
     const int ref = U[e].ref;
     float3 p;
     const double* p64;
