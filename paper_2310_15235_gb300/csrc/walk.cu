@@ -315,7 +315,7 @@ __device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si,
       const int staged = min(total - lo, a.M);
       make_sources<kBucket, kCSM>(a, x, si, lane, w.U, w.Up, staged);
       n = staged <= 0                        ? 0
-          : kCells && !kBucket && staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
+          : kCells && staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
                                           : bin_sources(a, lane, w.U, w.Up, staged, w.V, w.off);
     }
     if (n > 0) {
@@ -396,8 +396,8 @@ __device__ __forceinline__ void walk_receiver(const WalkArgs& a, int64_t io, flo
 }
 
 // One warp per receiver, receivers from a global counter.
-template <int NBP, int WARPS, bool kCells>
-__global__ void __launch_bounds__(WARPS * 32, (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
+template <int NBP, int WARPS, bool kCells, int kWarpsPerSM>
+__global__ void __launch_bounds__(WARPS * 32, kWarpsPerSM / WARPS)
     k_walk(WalkArgs a) {
   extern __shared__ __align__(16) int smem[];
   init_block<kCells>(a, smem);
@@ -1178,7 +1178,7 @@ __device__ void walk_bucket(const WalkArgs& a, const BucketArgs& bk, int64_t p0,
 constexpr int kPPBlocksPerSM = 5;
 
 template <int NBP, int WARPS, bool kPP, bool kCSM, bool kCells>
-__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
+__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellBucketWarpsPerSM : kWalkWarpsPerSM) / WARPS)
     k_walk_bucket(WalkArgs a, const __grid_constant__ BucketArgs bk) {
   extern __shared__ __align__(16) int smem[];
   init_block<kCells>(a, smem);
@@ -1346,8 +1346,8 @@ __global__ void k_batch_tree_range(const __grid_constant__ BatchArgs B) {
 // One launch per tree (its walk arguments are this launch's own parameter,
 // so the walk reads them as directly as k_walk does): one warp per distinct
 // key of the tree, keys from a global counter.
-template <int NBP, int WARPS, bool kCells>
-__global__ void __launch_bounds__(WARPS * 32, (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
+template <int NBP, int WARPS, bool kCells, int kWarpsPerSM>
+__global__ void __launch_bounds__(WARPS * 32, kWarpsPerSM / WARPS)
     k_walk_batched(WalkArgs a, const __grid_constant__ BatchSlice S) {
   extern __shared__ __align__(16) int smem[];
   init_block<kCells>(a, smem);
@@ -1395,7 +1395,7 @@ __global__ void k_batch_leaf(const __grid_constant__ BatchArgs B,
 // k_walk_batched; slots from a global counter, a bucket walked by the warp
 // that takes its first slot.
 template <int NBP, int WARPS, bool kPP, bool kCSM, bool kCells>
-__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellWarpsPerSM : kWalkWarpsPerSM) / WARPS)
+__global__ void __launch_bounds__(WARPS * 32, kPP ? kPPBlocksPerSM : (kCells ? kCellBucketWarpsPerSM : kWalkWarpsPerSM) / WARPS)
     k_walk_bucket_batched(WalkArgs a, const __grid_constant__ BucketArgs bk,
                           const __grid_constant__ BatchSlice S) {
   extern __shared__ __align__(16) int smem[];
@@ -1490,7 +1490,9 @@ size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
     // the search for p-p particles needs the larger stack, phase_cut half of it
     if (!pp) a->stack_ints = 32 * (a->max_depth + 2);
     a->bin_cap = kCellSources;
-    a->region_ints = std::max(a->stack_ints, kCellStage + kCellHits + a->bin_cap);
+    // the cut's stack, then bin_sources_small's keys, then boxes, crossings and
+    // distances share the region
+    a->region_ints = std::max({a->stack_ints, 2 * a->bin_cap, kCellStage + kCellHits + a->bin_cap});
     a->warp_ints = a->region_ints + 2 * a->npix + 36;
   }
   a->src_stack_cap = a->stack_ints;
@@ -1522,22 +1524,25 @@ static int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st) {
   return TREVR2_OK;
 }
 
-template <int NBP, bool kCells>
+template <int NBP, bool kCells, int kWarpsPerSM>
 static const void* walk_kernel_nbp(int warps, bool batched) {
   if (batched)
-    return warps == 4 ? reinterpret_cast<const void*>(&k_walk_batched<NBP, 4, kCells>)
-                      : reinterpret_cast<const void*>(&k_walk_batched<NBP, 8, kCells>);
-  return reinterpret_cast<const void*>(&k_walk<NBP, kWalkWarps, kCells>);
+    return warps == 4 ? reinterpret_cast<const void*>(&k_walk_batched<NBP, 4, kCells, kWarpsPerSM>)
+                      : reinterpret_cast<const void*>(&k_walk_batched<NBP, 8, kCells, 24>);
+  return reinterpret_cast<const void*>(&k_walk<NBP, kWalkWarps, kCells, kWarpsPerSM>);
 }
 
-static const void* walk_kernel(int nbp, int warps, bool batched, bool cells) {
-  if (cells)
-    return nbp == 1 ? walk_kernel_nbp<1, true>(warps, batched)
-         : nbp == 2 ? walk_kernel_nbp<2, true>(warps, batched)
-                    : walk_kernel_nbp<4, true>(warps, batched);
-  return nbp == 1 ? walk_kernel_nbp<1, false>(warps, batched)
-       : nbp == 2 ? walk_kernel_nbp<2, false>(warps, batched)
-                  : walk_kernel_nbp<4, false>(warps, batched);
+template <int NBP>
+static const void* walk_kernel_of(int warps, bool batched, bool cells, int nside) {
+  if (!cells) return walk_kernel_nbp<NBP, false, kWalkWarpsPerSM>(warps, batched);
+  return nside < 4 ? walk_kernel_nbp<NBP, true, kCellWarpsPerSM>(warps, batched)
+                   : walk_kernel_nbp<NBP, true, kCellFineWarpsPerSM>(warps, batched);
+}
+
+static const void* walk_kernel(int nbp, int warps, bool batched, bool cells, int nside) {
+  return nbp == 1 ? walk_kernel_of<1>(warps, batched, cells, nside)
+       : nbp == 2 ? walk_kernel_of<2>(warps, batched, cells, nside)
+                  : walk_kernel_of<4>(warps, batched, cells, nside);
 }
 
 // Shared memory attribute and resident blocks per SM of a walk kernel.
@@ -1639,7 +1644,7 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
     T2_CHECK(order_receivers(t, active, A, keys, slots, st));
     a.order = slots;
   }
-  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells);
+  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells, nside);
   const size_t smem = walk_layout(&a, kWalkWarps, cells, false);
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kWalkWarps, smem, &per_sm, &sms));
@@ -2088,7 +2093,7 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
     b->args.tree[i].cell_cap = c ? kCellCap : 0;
     if (fn[c]) continue;
     fn[c] = b->bucket ? bucket_batched_kernel(b->nbp, b->pp, b->csm, c != 0)
-                      : walk_kernel(b->nbp, warps, true, c != 0);
+                      : walk_kernel(b->nbp, warps, true, c != 0, b->nside);
     int per_sm = 0, sms = 0;
     T2_CHECK(config_walk_kernel(fn[c], warps, smem[c], &per_sm, &sms));
     const int64_t g = std::min<int64_t>(int64_t(sms) * per_sm, (limit + warps - 1) / warps);
@@ -2528,7 +2533,7 @@ extern "C" int trevr2_kernel_binary_version(int* version) {
     return TREVR2_EINVAL;
   }
   cudaFuncAttributes attr;
-  T2_CUDA(cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(&k_walk<4, kWalkWarps, true>)));
+  T2_CUDA(cudaFuncGetAttributes(&attr, reinterpret_cast<const void*>(&k_walk<4, kWalkWarps, true, kCellFineWarpsPerSM>)));
   *version = attr.binaryVersion;
   return TREVR2_OK;
 }
@@ -2601,7 +2606,7 @@ static int launch_walk_noalloc(Tree* t, Table* tb, const int64_t* active, int64_
   // beam by beam: walking cell by cell needs larger buffers, which would leave
   // room for fewer warps in the fixed array
   const bool cells = false;
-  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells);
+  const void* fn = walk_kernel(t->nbp, kWalkWarps, false, cells, nside);
   const size_t smem = walk_layout(&a, kWalkWarps, cells, false);
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kWalkWarps, smem, &per_sm, &sms));
