@@ -38,6 +38,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "cells.cuh"
 #include "walk.cuh"
 
 namespace trevr2 {
@@ -429,12 +430,12 @@ __device__ void adjoint_stage3(const AdjArgs& g, float3 x, int si, int lane, int
   }
 }
 
-template <int NBP>
-__device__ __forceinline__ void adjoint_receiver(const AdjArgs& g, int64_t slot, int lane, int* stk,
-                                                 int* off, uint32_t* binfo, int* next_beam,
-                                                 int* lstk, SrcEntry* U, int* Up, SrcEntry* V,
-                                                 float* T, float* Q, float4* S) {
+// One receiver's share of the gradients: its upstream gradient and factors, the
+// walk (walk(x, si, gJf, Js, Jc)), and Eq. taucorr's own term.
+template <int NBP, class Walk>
+__device__ __forceinline__ void adjoint_row(const AdjArgs& g, int64_t turn, int lane, Walk walk) {
   const WalkArgs& a = g.w;
+  const int64_t slot = a.order ? int64_t(a.order[turn]) : turn;
   const int64_t io = a.active[slot];
   if (io < 0 || io >= a.N) {
     if (lane == 0) atomicOr(a.status, kStatusBadActive);
@@ -468,11 +469,35 @@ __device__ __forceinline__ void adjoint_receiver(const AdjArgs& g, int64_t slot,
   float Js[NBP], Jc[NBP];
 #pragma unroll
   for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
+  walk(x, si, gJf, Js, Jc);
+  if (!thick) return;
+  // Eq. taucorr: J = F0 Jraw f(tau_i), tau_i = kappa_i m_i / h_i^2
+#pragma unroll
+  for (int b = 0; b < NBP; ++b) {
+    double v = double(Js[b]) - double(Jc[b]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == b && b < a.nb && gJb[b] != 0.0f) {
+      const double tau = double(a.km[int64_t(si) * NBP + b]) / (h * h);
+      // dtau/dkappa = m / h^2; the element kernel applies the mass
+      const double dk = double(gJb[b]) * a.inv_size2 * v * thick_factor_deriv(tau) / (h * h);
+      atomicAdd(g.g_thick + int64_t(si) * NBP + b, float(dk));
+    }
+  }
+}
+
+template <int NBP>
+__device__ __forceinline__ void adjoint_receiver(const AdjArgs& g, int64_t slot, int lane, int* stk,
+                                                 int* off, uint32_t* binfo, int* next_beam,
+                                                 int* lstk, SrcEntry* U, int* Up, SrcEntry* V,
+                                                 float* T, float* Q, float4* S) {
+  const WalkArgs& a = g.w;
+  adjoint_row<NBP>(g, slot, lane, [&](float3 x, int si, const float* gJf, float* Js, float* Jc) {
   for (int lo = 0;; lo += a.M) {
     const int total = phase_sources(a, x, si, lane, stk, a.src_stack_cap, U, Up, lo);
     const int staged = min(total - lo, a.M);
     make_sources(a, x, si, lane, U, Up, staged);
-    const int n = staged > 0 ? bin_sources(a, lane, U, Up, staged, V, off) : 0;
+    const int n = staged > 0 ? bin_sources(a.npix, lane, U, Up, staged, V, off) : 0;
     if (n > 0) {
       // bin_sources leaves the beams in Up unsorted: put them in V's order
       for (int e = lane; e < a.npix; e += 32) {
@@ -493,20 +518,7 @@ __device__ __forceinline__ void adjoint_receiver(const AdjArgs& g, int64_t slot,
     }
     if (lo + a.M >= total) break;
   }
-  if (!thick) return;
-  // Eq. taucorr: J = F0 Jraw f(tau_i), tau_i = kappa_i m_i / h_i^2
-#pragma unroll
-  for (int b = 0; b < NBP; ++b) {
-    double v = double(Js[b]) - double(Jc[b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == b && b < a.nb && gJb[b] != 0.0f) {
-      const double tau = double(a.km[int64_t(si) * NBP + b]) / (h * h);
-      // dtau/dkappa = m / h^2; the element kernel applies the mass
-      const double dk = double(gJb[b]) * a.inv_size2 * v * thick_factor_deriv(tau) / (h * h);
-      atomicAdd(g.g_thick + int64_t(si) * NBP + b, float(dk));
-    }
-  }
+  });
 }
 
 // Shared memory of an adjoint block: per warp the stacks, the beam offsets,
@@ -542,6 +554,212 @@ __global__ void __launch_bounds__(WARPS * 32, kAdjBlocksPerSM) k_walk_adjoint(co
     if (slot >= (unsigned long long)a.A) break;
     adjoint_receiver<NBP>(g, int64_t(slot), lane, stk, off, binfo, next_beam, lstk, U, Up, V, T, Q,
                           S);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The adjoint walk cell by cell (as k_walk's, see cells.cuh): the crossings are
+// found twice.  First they build tau and the absorption at every source; then,
+// with S_j = sum of q over the sources of the beam from j on, each crossing
+// [t0, t1) adds
+//   dLoss/dalpha -= S_(first s >= t1) (t1 - t0) + sum_{t0 <= s < t1} q (s - t0)
+// to its cell.  No order along the beam and no record of segments is needed.
+// 64^3 field, nside 2, 2 bands: 11.1 ms beam by beam.
+constexpr int kAdjCellWarps = 4;
+// As k_walk: 28 warps per SM at nside 1 and 2 (64^3 gradient 17.9 -> 16.6 ms), 24
+// at nside 4.
+constexpr int kAdjCellBlocksPerSM = 7;
+constexpr int kAdjCellFineBlocksPerSM = 6;
+
+// Up to 32 crossings, one per lane: their cells' gradients from the sources
+// [e0, e0 + m) (S and Q start at e0).
+template <int NBP>
+__device__ __forceinline__ void crossing_gradients(const AdjArgs& g, bool live, float4 h,
+                                                   const float4* binv, const float* ss,
+                                                   const int* off, int e0, int m, const float* S,
+                                                   const float* Q) {
+  const WalkArgs& a = g.w;
+  if (!live) return;
+  const float t0 = h.x, t1 = h.y;
+  const int row = __float_as_int(h.z), at = __float_as_int(h.w), k = beam_slot(at);
+  const int je = min(off[k] - e0, m);
+  int j = max((k ? off[k - 1] : 0) - e0, 0);
+  for (int b = je; j < b;) {  // the first source of the beam at or beyond t0
+    const int mid = (j + b) >> 1;
+    if (ss[mid] < t0) j = mid + 1; else b = mid;
+  }
+  float ga[NBP];
+#pragma unroll
+  for (int b = 0; b < NBP; ++b) ga[b] = 0.0f;
+  for (; j < je && ss[j] < t1; ++j) {
+    const float ds = ss[j] - t0;
+    const BandVec<NBP> q = load_bands<NBP>(Q + j * NBP);
+#pragma unroll
+    for (int b = 0; b < NBP; ++b) ga[b] -= q.v[b] * ds;
+  }
+  if (j < je) {
+    const BandVec<NBP> W = load_bands<NBP>(S + j * NBP);
+    const float len = t1 - t0;
+#pragma unroll
+    for (int b = 0; b < NBP; ++b) ga[b] -= W.v[b] * len;
+  }
+  bool any = false;
+#pragma unroll
+  for (int b = 0; b < NBP; ++b) any |= ga[b] != 0.0f;
+  if (any)
+    add_bands<NBP>(row < 0 ? g.g_aleaf + int64_t(-(row + 1)) * NBP
+                           : g.g_atab + (int64_t(row) * a.P + __float_as_int(binv[at].w)) * NBP, ga);
+}
+
+// The nc listed cells against the n staged sources: the forward (back = false:
+// tau increments to T and w.own, alpha at the sources inside cells to Q), or the
+// cells' gradients (back: S = w.own is scratch, Q holds q).  One piece of code
+// for both, so that the loops stay in the instruction cache.
+template <int NBP>
+__device__ __forceinline__ void run_cells(const AdjArgs& g, float3 x, int lane, const WarpMem& w,
+                                          float* T, float* Q, int n, int nc, bool first, bool back) {
+  const WalkArgs& a = g.w;
+  const unsigned lt = (1u << lane) - 1u;
+  int* stage = w.stk;
+  float4* hits = reinterpret_cast<float4*>(stage + kCellStage);
+  float* ss = reinterpret_cast<float*>(hits + kCellHits / 4);
+  float* own = w.own;
+  if (!back && first) {
+    BandVec<NBP> zero;
+#pragma unroll
+    for (int b = 0; b < NBP; ++b) zero.v[b] = 0.0f;
+    for (int e = lane; e < n; e += 32) {
+      store_bands<NBP>(T + e * NBP, zero);
+      store_bands<NBP>(own + e * NBP, zero);
+      store_bands<NBP>(Q + e * NBP, zero);
+    }
+  }
+  for (int e0 = 0; e0 < n; e0 += a.bin_cap) {
+    const int m = min(a.bin_cap, n - e0);
+    const float s_before = e0 ? w.V[e0 - 1].s : 0.0f;
+    __syncwarp();
+    for (int e = lane; e < m; e += 32) ss[e] = w.V[e0 + e].s;
+    __syncwarp();
+    for (int k = lane; k < a.npix; k += 32) {
+      const int s0 = max((k ? w.off[k - 1] : 0) - e0, 0), s1 = min(w.off[k] - e0, m);
+      w.far[beam_slot(k)] = s1 > s0 ? ss[s1 - 1] : -1.0f;
+      if (!back) continue;
+      BandVec<NBP> run;
+#pragma unroll
+      for (int b = 0; b < NBP; ++b) run.v[b] = 0.0f;
+      for (int j = s1 - 1; j >= s0; --j) {  // farthest first
+        const BandVec<NBP> q = load_bands<NBP>(Q + (e0 + j) * NBP);
+#pragma unroll
+        for (int b = 0; b < NBP; ++b) run.v[b] += q.v[b];
+        store_bands<NBP>(own + (e0 + j) * NBP, run);
+      }
+    }
+    __syncwarp();
+    auto take = [&](bool live, float4 h) {
+      if (back)
+        crossing_gradients<NBP>(g, live, h, w.binv, ss, w.off, e0, m, own + e0 * NBP, Q + e0 * NBP);
+      else
+        add_crossings<NBP, true>(a, lane, live, h, w.binv, ss, w.off, e0, m, s_before, T + e0 * NBP,
+                                 own + e0 * NBP, first, [&](int j, const BandVec<NBP>& al) {
+                                   store_bands<NBP>(Q + (e0 + j) * NBP, al);
+                                 });
+      __syncwarp();
+    };
+    int head = 0;  // crossings found; the last head % 32 are pending, in a ring of 64
+    int q_next = lane < nc ? w.cells[lane] : -1;
+    for (int c0 = 0; c0 < nc; c0 += 32) {
+      const int q = q_next;
+      q_next = c0 + 32 + lane < nc ? w.cells[c0 + 32 + lane] : -1;
+      cross_batch<false>(a, x, lane, q, stage, w.binv, w.far, 0.0f, [&](bool hit, float t0, float t1, int row, int k) {
+        const unsigned hm = __ballot_sync(0xffffffffu, hit);
+        if (hit)
+          hits[(head + __popc(hm & lt)) & 63] =
+              make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
+        const int was = head;
+        head += __popc(hm);
+        __syncwarp();
+        if ((head ^ was) & 32) take(true, hits[(was & 32) + lane]);
+      });
+    }
+    if (head & 31) take(lane < (head & 31), hits[(head & 32) + lane]);
+  }
+  __syncwarp();
+}
+
+// The sources and cells of one receiver, in passes of M sources; per pass the
+// forward over all windows of cells, the sources' terms, and the gradients over
+// all windows again.
+template <int NBP>
+__device__ __forceinline__ void adjoint_cells(const AdjArgs& g, float3 x, int si, int lane,
+                                              const WarpMem& w, float* T, float* Q,
+                                              const float* gJf, float* Js, float* Jc) {
+  const WalkArgs& a = g.w;
+  int n = 0, total = 0, listed = 0;
+  bool back = false;   // the pass's second run over the cells
+  bool at_hand = false;  // w.cells holds the window to run over
+  for (int lo = 0, clo = 0;;) {
+    if (!at_hand) {
+      // a later window only lists cells: no source has an index that high
+      const bool stage = clo == 0 && !back;
+      const int2 c = phase_cut<false, false>(a, x, si, lane, w.stk, a.src_stack_cap, w.U,
+                                             stage ? lo : INT32_MAX, w.cells, clo, 0.0f);
+      total = c.x;
+      listed = c.y;
+      if (stage) {
+        const int staged = min(total - lo, a.M);
+        make_sources(a, x, si, lane, w.U, w.Up, staged);
+        n = staged <= 0              ? 0
+            : staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
+                                  : bin_sources(a.npix, lane, w.U, w.Up, staged, w.V, w.off);
+      }
+    }
+    at_hand = false;
+    if (n > 0) {
+      run_cells<NBP>(g, x, lane, w, T, Q, n, min(listed - clo, a.cell_cap), clo == 0, back);
+      if (clo + a.cell_cap < listed) {
+        clo += a.cell_cap;
+        continue;
+      }
+      if (!back) {
+        sum_increments<NBP>(lane, a.npix, w.off, T, w.own);
+        // the beams of the records, in V's order
+        for (int k = lane; k < a.npix; k += 32)
+          for (int j = k ? w.off[k - 1] : 0; j < w.off[k]; ++j) w.Up[j] = k;
+        __syncwarp();
+        adjoint_stage2<NBP>(g, x, si, lane, w.V, w.Up, T, Q, n, gJf, Js, Jc);
+        __syncwarp();
+        back = true;
+        at_hand = clo == 0;  // one window: its cells are still listed
+        clo = 0;
+        continue;
+      }
+    }
+    back = false;
+    clo = 0;
+    lo += a.M;
+    if (lo >= total) break;
+  }
+}
+
+template <int NBP, int kBlocksPerSM>
+__global__ void __launch_bounds__(kAdjCellWarps * 32, kBlocksPerSM)
+    k_walk_adjoint_cells(const __grid_constant__ AdjArgs g) {
+  extern __shared__ __align__(16) int smem[];
+  const WalkArgs& a = g.w;
+  init_block<true>(a, smem);
+  const int lane = threadIdx.x & 31;
+  const int64_t gw = int64_t(blockIdx.x) * kAdjCellWarps + (threadIdx.x >> 5);
+  const WarpMem w = warp_mem<true>(a, smem, gw, a.srcU, a.pixU, a.srcV, g.T, a.cells);
+  float* T = g.T + gw * a.M * NBP;
+  float* Q = g.Q + gw * a.M * NBP;
+  for (;;) {
+    unsigned long long slot = 0;
+    if (lane == 0) slot = atomicAdd(a.counter, 1ull);
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    if (slot >= (unsigned long long)a.A) break;
+    adjoint_row<NBP>(g, int64_t(slot), lane, [&](float3 x, int si, const float* gJf, float* Js, float* Jc) {
+      adjoint_cells<NBP>(g, x, si, lane, w, T, Q, gJf, Js, Jc);
+    });
   }
 }
 
@@ -651,8 +869,10 @@ __global__ void k_grad_elements(int64_t N, int nb, double inv_size2, const int* 
 }
 
 template <int NBP>
-const void* adjoint_kernel() {
-  return reinterpret_cast<const void*>(&k_walk_adjoint<NBP, kAdjWarps>);
+const void* adjoint_kernel(bool cells, int nside) {
+  return cells && nside < 4 ? reinterpret_cast<const void*>(&k_walk_adjoint_cells<NBP, kAdjCellBlocksPerSM>)
+       : cells ? reinterpret_cast<const void*>(&k_walk_adjoint_cells<NBP, kAdjCellFineBlocksPerSM>)
+               : reinterpret_cast<const void*>(&k_walk_adjoint<NBP, kAdjWarps>);
 }
 
 }  // namespace
@@ -724,13 +944,20 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
   fill_walk_args(t, tb, nside, theta, bsel, nbsel, flags & ~TREVR2_ASYNC, kSrcCapacity, &wa);
   wa.A = A;
   wa.active = active;
-  const void* fn = nbp == 1 ? adjoint_kernel<1>() : nbp == 2 ? adjoint_kernel<2>() : adjoint_kernel<4>();
-  const size_t smem = adjoint_smem(kAdjWarps, wa.stack_ints, wa.npix);
+  const bool cells = use_cells(t, tb, theta);
+  if (cells) T2_CHECK(use_beam_map(tb, &wa, st));
+  const int bw = cells ? kAdjCellWarps : kAdjWarps;  // warps per block
+  const void* fn = nbp == 1 ? adjoint_kernel<1>(cells, nside)
+                 : nbp == 2 ? adjoint_kernel<2>(cells, nside)
+                            : adjoint_kernel<4>(cells, nside);
+  const size_t smem = cells ? walk_layout(&wa, bw, true, false)
+                            : adjoint_smem(bw, wa.stack_ints, wa.npix);
+  wa.cell_cap = cells ? kCellCap : 0;
   int per_sm = 0, sms = 0;
-  T2_CHECK(config_walk_kernel(fn, kAdjWarps, smem, &per_sm, &sms));
+  T2_CHECK(config_walk_kernel(fn, bw, smem, &per_sm, &sms));
   int64_t blocks = int64_t(sms) * per_sm;
-  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (A + kAdjWarps - 1) / kAdjWarps));
-  const size_t warps = size_t(blocks) * kAdjWarps;
+  blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (A + bw - 1) / bw));
+  const size_t warps = size_t(blocks) * bw;
 
   // one allocation: gradient buffers (zeroed), leaf map, walk buffers
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
@@ -745,12 +972,15 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
   const size_t b_Q = up(sizeof(float) * warps * wa.M * nbp);
   const size_t b_T = b_Q;
   // segment records address the table by a 32-bit row index
-  const int seg_cap = int64_t(std::max<int64_t>(t->n_internal, 1)) * P < INT32_MAX ? kSegCap : 0;
+  const int seg_cap = !cells && int64_t(std::max<int64_t>(t->n_internal, 1)) * P < INT32_MAX ? kSegCap : 0;
   const size_t b_seg = up(sizeof(float4) * warps * size_t(seg_cap) * 32);
-  const size_t b_walk = warps * size_t(wa.M) * (2 * sizeof(SrcEntry) + sizeof(int));
+  const size_t b_walk = up(warps * size_t(wa.M) * (2 * sizeof(SrcEntry) + sizeof(int)));
+  const size_t b_cells = cells ? warps * (size_t(kCellCap) + 4 * size_t(wa.M)) * sizeof(int) : 0;
+  // receivers in the tree's order, so that neighbouring walks share its nodes
+  const size_t b_keys = up(sizeof(uint64_t) * size_t(A)), b_slots = up(sizeof(int) * size_t(A));
   char* base = nullptr;
   T2_CHECK(device_alloc(reinterpret_cast<void**>(&base),
-                        zeroed + b_leaf + b_T + b_Q + b_seg + b_walk, st, "adjoint buffers"));
+                        zeroed + b_leaf + b_T + b_Q + b_seg + b_walk + up(b_cells) + b_keys + b_slots, st, "adjoint buffers"));
   AdjArgs g;
   std::memset(&g, 0, sizeof(g));
   g.w = wa;
@@ -770,13 +1000,18 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
   g.w.srcU = reinterpret_cast<SrcEntry*>(p);
   g.w.srcV = reinterpret_cast<SrcEntry*>(p + warps * wa.M * sizeof(SrcEntry));
   g.w.pixU = reinterpret_cast<int*>(p + 2 * warps * wa.M * sizeof(SrcEntry));
+  g.w.cells = reinterpret_cast<int*>(p + b_walk);
+  uint64_t* keys = reinterpret_cast<uint64_t*>(p + b_walk + up(b_cells));
+  int* slots = reinterpret_cast<int*>(p + b_walk + up(b_cells) + b_keys);
+  if (A > 1) g.w.order = slots;
   int rc = TREVR2_OK;
   auto run = [&]() -> int {
     T2_CUDA(cudaMemsetAsync(base, 0, zeroed, st));
     if (A > 0) {
+      if (A > 1) T2_CHECK(order_receivers(t, active, A, keys, slots, st));
       T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
       void* args[] = {&g};
-      T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(kAdjWarps * 32), args, smem, st));
+      T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(bw * 32)), args, smem, st));
       note_launch();
     }
     for (int d = 0; d < t->max_depth; ++d) {

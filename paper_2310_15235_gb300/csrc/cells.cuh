@@ -179,11 +179,12 @@ constexpr int kCellHits = 64 * 4;
 
 // Up to 32 crossings (t0, t1, row, beam), one per lane: their increments, to
 // the sources [e0, e0 + m) of V.
-template <int NBP, bool kInOrder>
+// inside(j, alpha) is called for every source inside its crossing's cell.
+template <int NBP, bool kInOrder, class Inside>
 __device__ __forceinline__ void add_crossings(const WalkArgs& a, int lane, bool live, float4 h,
                                               const float4* binv, const float* ss, const int* off,
                                               int e0, int m, float s_before, float* T, float* own,
-                                              bool first) {
+                                              bool first, Inside inside) {
   BandVec<NBP> add;
 #pragma unroll
   for (int b = 0; b < NBP; ++b) add.v[b] = 0.0f;
@@ -202,6 +203,7 @@ __device__ __forceinline__ void add_crossings(const WalkArgs& a, int lane, bool 
     }
     for (; j < je && ss[j] < t1; ++j) {  // sources inside the cell
       const float ds = ss[j] - t0;
+      inside(j, add);
       BandVec<NBP> tk;
 #pragma unroll
       for (int b = 0; b < NBP; ++b) tk.v[b] = add.v[b] * ds;
@@ -399,11 +401,11 @@ __device__ __forceinline__ void cross_batch(const WalkArgs& a, float3 x, int lan
 // tau of the n staged sources V (sorted by beam and distance) from the nc
 // listed cells, into T[e][NBP]: set with `first`, added to what is there
 // without.  own[e][NBP]: the depth of the cell that holds a source, up to it.
-template <int NBP, bool kPP, bool kInOrder>
-__device__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
+template <int NBP, bool kPP, bool kInOrder, class Inside>
+__device__ __forceinline__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
                              const float4* binv, const int* off, float* far, const SrcEntry* V,
                              float* T, float* own, int n, const int* cells, int nc, bool first,
-                             float rpp) {
+                             float rpp, Inside inside) {
   const unsigned lt = (1u << lane) - 1u;
   const int npix = a.npix;
   int* stage = region;
@@ -443,13 +445,15 @@ __device__ void absorb_cells(const WalkArgs& a, float3 x, int lane, int* region,
         head += __popc(hm);
         __syncwarp();
         if ((head ^ was) & 32)
-          add_crossings<NBP, kInOrder>(a, lane, true, hits[(was & 32) + lane], binv, ss, off, e0, m, s_before,
-                             Tw, own + e0 * NBP, first);
+          add_crossings<NBP, kInOrder>(a, lane, true, hits[(was & 32) + lane], binv, ss, off, e0, m,
+                                       s_before, Tw, own + e0 * NBP, first,
+                                       [&](int j, const BandVec<NBP>& al) { inside(e0 + j, al); });
       });
     }
     if (head & 31)
-      add_crossings<NBP, kInOrder>(a, lane, lane < (head & 31), hits[(head & 32) + lane], binv, ss, off, e0, m, s_before, Tw,
-                         own + e0 * NBP, first);
+      add_crossings<NBP, kInOrder>(a, lane, lane < (head & 31), hits[(head & 32) + lane], binv, ss,
+                                   off, e0, m, s_before, Tw, own + e0 * NBP, first,
+                                   [&](int j, const BandVec<NBP>& al) { inside(e0 + j, al); });
   }
   __syncwarp();
 }
@@ -473,6 +477,60 @@ __device__ __forceinline__ void sum_increments(int lane, int npix, const int* of
       store_bands<NBP>(T + j * NBP, o);
     }
   }
+}
+
+constexpr int kCellCap = 2048;  // cells of a cut listed at once
+
+// A warp's part of a walk block's shared memory and of the walk buffers.
+struct WarpMem {
+  int* stk;          // traversal stacks / increments, boxes and crossings
+  int* lstk;         // this lane's stack (beam by beam)
+  int* off;          // [npix] ends of the beams' buckets, then scratch
+  int* order;        // [npix] beams by distance (beam by beam)
+  int* next_beam;
+  NodeW* chain;      // the receiver's ancestors (beam by beam)
+  float* far;        // [npix] the beams' farthest sources (cell by cell)
+  const float4* binv;  // [npix] the block's copy of 1 / direction (cell by cell)
+  SrcEntry* U;
+  int* Up;
+  SrcEntry* V;
+  float* T;
+  float* own;        // [M][4] depth inside the cell that holds a source (cell by cell)
+  int* cells;
+};
+
+template <bool kCells>
+__device__ __forceinline__ WarpMem warp_mem(const WalkArgs& a, int* smem, int64_t gw,
+                                            SrcEntry* srcU, int* pixU, SrcEntry* srcV, float* srcT,
+                                            int* cells) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  WarpMem w;
+  w.binv = reinterpret_cast<const float4*>(smem);
+  int* wsm = smem + (kCells ? 4 * a.npix : 0) + wib * a.warp_ints;
+  w.stk = wsm;
+  w.lstk = wsm + lane * 2 * (a.max_depth + 2);
+  w.off = wsm + a.region_ints;
+  w.order = w.off + a.npix;
+  w.far = reinterpret_cast<float*>(w.off + a.npix);
+  w.next_beam = w.off + 2 * a.npix + 32;  // after the beam order and its counts
+  w.chain = reinterpret_cast<NodeW*>(w.off + 2 * a.npix + 36);
+  w.U = srcU + gw * a.M;
+  w.Up = pixU + gw * a.M;
+  w.V = srcV + gw * a.M;
+  w.T = srcT + gw * a.M * 4;
+  w.cells = cells + gw * (a.cell_cap + 4 * a.M);
+  w.own = reinterpret_cast<float*>(w.cells + a.cell_cap);
+  return w;
+}
+
+// Fills a walk block's shared tables.
+template <bool kCells>
+__device__ __forceinline__ void init_block(const WalkArgs& a, int* smem) {
+  if constexpr (kCells) {
+    float4* binv = reinterpret_cast<float4*>(smem);
+    for (int k = threadIdx.x; k < a.npix; k += blockDim.x) binv[k] = a.beam_inv[k];
+  }
+  init_ext_tab();
 }
 
 }  // namespace trevr2

@@ -209,60 +209,6 @@ __device__ __forceinline__ void eval_sources(const WalkArgs& a, int lane, const 
   }
 }
 
-constexpr int kCellCap = 2048;  // cells of a cut listed at once
-
-// A warp's part of a walk block's shared memory and of the walk buffers.
-struct WarpMem {
-  int* stk;          // traversal stacks / increments, boxes and crossings
-  int* lstk;         // this lane's stack (beam by beam)
-  int* off;          // [npix] ends of the beams' buckets, then scratch
-  int* order;        // [npix] beams by distance (beam by beam)
-  int* next_beam;
-  NodeW* chain;      // the receiver's ancestors (beam by beam)
-  float* far;        // [npix] the beams' farthest sources (cell by cell)
-  const float4* binv;  // [npix] the block's copy of 1 / direction (cell by cell)
-  SrcEntry* U;
-  int* Up;
-  SrcEntry* V;
-  float* T;
-  float* own;        // [M][4] depth inside the cell that holds a source (cell by cell)
-  int* cells;
-};
-
-template <bool kCells>
-__device__ __forceinline__ WarpMem warp_mem(const WalkArgs& a, int* smem, int64_t gw,
-                                            SrcEntry* srcU, int* pixU, SrcEntry* srcV, float* srcT,
-                                            int* cells) {
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  WarpMem w;
-  w.binv = reinterpret_cast<const float4*>(smem);
-  int* wsm = smem + (kCells ? 4 * a.npix : 0) + wib * a.warp_ints;
-  w.stk = wsm;
-  w.lstk = wsm + lane * 2 * (a.max_depth + 2);
-  w.off = wsm + a.region_ints;
-  w.order = w.off + a.npix;
-  w.far = reinterpret_cast<float*>(w.off + a.npix);
-  w.next_beam = w.off + 2 * a.npix + 32;  // after the beam order and its counts
-  w.chain = reinterpret_cast<NodeW*>(w.off + 2 * a.npix + 36);
-  w.U = srcU + gw * a.M;
-  w.Up = pixU + gw * a.M;
-  w.V = srcV + gw * a.M;
-  w.T = srcT + gw * a.M * 4;
-  w.cells = cells + gw * (a.cell_cap + 4 * a.M);
-  w.own = reinterpret_cast<float*>(w.cells + a.cell_cap);
-  return w;
-}
-
-// Fills a walk block's shared tables.
-template <bool kCells>
-__device__ __forceinline__ void init_block(const WalkArgs& a, int* smem) {
-  if constexpr (kCells) {
-    float4* binv = reinterpret_cast<float4*>(smem);
-    for (int k = threadIdx.x; k < a.npix; k += blockDim.x) binv[k] = a.beam_inv[k];
-  }
-  init_ext_tab();
-}
-
 // tau of every source of one origin (n staged sources V binned by beam) into
 // w.T, from all its cells or (cell by cell) from the window of `listed` cells
 // that starts at clo: set for the first window, added for the later ones.
@@ -271,7 +217,7 @@ __device__ __forceinline__ void absorb(const WalkArgs& a, float3 x, int si, int 
                                        int n, int listed, int clo, int leaf, float rpp) {
   if constexpr (kCells) {
     absorb_cells<NBP, kPP, !kBucket>(a, x, lane, w.stk, w.binv, w.off, w.far, w.V, w.T, w.own, n, w.cells,
-                           min(listed - clo, a.cell_cap), clo == 0, rpp);
+                           min(listed - clo, a.cell_cap), clo == 0, rpp, [](int, const BandVec<NBP>&) {});
     if (clo + a.cell_cap >= listed) {
       sum_increments<NBP>(lane, a.npix, w.off, w.T, w.own);
       if constexpr (kCSM)
@@ -316,7 +262,7 @@ __device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si,
       make_sources<kBucket, kCSM>(a, x, si, lane, w.U, w.Up, staged);
       n = staged <= 0                        ? 0
           : kCells && staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
-                                          : bin_sources(a, lane, w.U, w.Up, staged, w.V, w.off);
+                                          : bin_sources(a.npix, lane, w.U, w.Up, staged, w.V, w.off);
     }
     if (n > 0) {
       absorb<NBP, kBucket, kPP, kCSM, kCells>(a, x, si, lane, w, n, listed, clo, leaf, rpp);
@@ -488,7 +434,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32, 2)
     if (wid == 0) {
       const int n0 = total <= 0           ? 0
                    : total <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, total, w.V, w.off, w.stk)
-                                        : bin_sources(a, lane, w.U, w.Up, total, w.V, w.off);
+                                        : bin_sources(a.npix, lane, w.U, w.Up, total, w.V, w.off);
       if (lane == 0) s_n = n0;
     }
     __syncthreads();
@@ -544,13 +490,14 @@ __global__ void __launch_bounds__(kTeamWarps * 32, 2)
           nq += __popc(m);
           __syncwarp();
           if ((nq ^ was) & 32)
-            add_crossings<NBP, true>(a, lane, true, queue[(was & 32) + lane], w.binv, ss, w.off, 0, n, 0.0f,
-                               w.T, w.own, true);
+            add_crossings<NBP, true>(a, lane, true, queue[(was & 32) + lane], w.binv, ss, w.off, 0, n,
+                                     0.0f, w.T, w.own, true, [](int, const BandVec<NBP>&) {});
         }
       }
       __syncwarp();
       if (nq & 31)
-        add_crossings<NBP, true>(a, lane, lane < (nq & 31), queue[(nq & 32) + lane], w.binv, ss, w.off, 0, n, 0.0f, w.T, w.own, true);
+        add_crossings<NBP, true>(a, lane, lane < (nq & 31), queue[(nq & 32) + lane], w.binv, ss,
+                                 w.off, 0, n, 0.0f, w.T, w.own, true, [](int, const BandVec<NBP>&) {});
       __syncthreads();
       sum_increments<NBP>(tid, a.npix, w.off, w.T, w.own, kTeamWarps * 32);
       __syncthreads();
@@ -1510,13 +1457,13 @@ size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
 //    sources 2.90 / 2.41, 60 3.24 / 3.26, 120 3.63 / 4.16; nside 2: 3 sources
 //    1.88 / 1.79, 12 2.00 / 2.08; nside 1: 1 source 1.63 / 1.43, 3 1.66 / 1.75;
 //  - refinement opens cells that no beam with sources comes near: beam by beam.
-static bool use_cells(const Tree* t, const Table* tb, float theta) {
+bool use_cells(const Tree* t, const Table* tb, float theta) {
   return tb->nside <= kCellNside && !t->refine_on && theta >= (tb->nside < 4 ? 0.45f : 0.4f) &&
          3 * t->n_luminous >= 12 * tb->nside * tb->nside;
 }
 
 // The beam look-up tables for a walk cell by cell.
-static int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st) {
+int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st) {
   T2_CHECK(ensure_beam_map(tb, st));
   a->beam_list = tb->beam_list;
   a->beam_count = tb->beam_count;

@@ -538,9 +538,8 @@ static __device__ void make_sources(const WalkArgs& a, float3 x, int si, int lan
 // Bucket the n records of U by beam into V, skipping beam -1; off[k] ends as
 // the end of bucket k (its start is off[k-1], or 0).  Each bucket is sorted
 // by (s, source).  Returns the number of records binned.
-static __device__ int bin_sources(const WalkArgs& a, int lane, SrcEntry* U, const int* Up, int n,
+static __device__ int bin_sources(int npix, int lane, SrcEntry* U, const int* Up, int n,
                                   SrcEntry* V, int* off) {
-  const int npix = a.npix;
   for (int k = lane; k < npix; k += 32) off[k] = 0;
   __syncwarp();
   for (int e = lane; e < n; e += 32)
@@ -668,6 +667,8 @@ int read_status(Tree* t, cudaStream_t st);
 // block's bytes.  Beam by beam: the traversal stacks, the beam bucket offsets,
 // the beam order and its 32 bucket counts, the next-beam counter (padded to 16
 // bytes), the receiver's ancestor records.  Cell by cell: see cells.cuh.
+bool use_cells(const Tree* t, const Table* tb, float theta);
+int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st);
 size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp);
 
 }  // namespace trevr2
