@@ -242,7 +242,8 @@ int trevr2_J_noalloc(trevr2_tree* tree, const int64_t* active, int64_t A, int ns
  *  g_lum    [N][nb] float32 output dLoss/dlum, overwritten
  * Positions, masses and sizes are not differentiated.  The call allocates
  * its gradient buffers (about the size of the alpha table for nside plus
- * 8 nb floats per element) stream ordered and frees them before returning.
+ * 8 nb floats per element), 12 bytes per receiver for their order and the walk
+ * buffers, stream ordered, and frees them before returning.
  * Errors: as trevr2_J (EINVAL, EUNSUPPORTED, ENOMEM, ECUDA).  Without
  * TREVR2_ASYNC the call synchronises `stream` and returns the device status.
  */

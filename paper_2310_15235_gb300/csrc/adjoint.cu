@@ -11,10 +11,11 @@
 // luminosity.  The discrete choices (the cut, beams, tree) are held fixed;
 // the traversals are recomputed, nothing from the forward is stored.
 //
-// The adjoint runs in four steps:
-//  1. walk (one warp per receiver, as the forward): the sources are found
-//     and binned exactly as in the forward.  Each lane then walks its beam
-//     twice.  Front to back it recomputes tau at every source and adds
+// The adjoint runs in three steps:
+//  1. walk (one warp per receiver, in the tree's order, as the forward): the
+//     sources are found and binned exactly as in the forward.  Where the
+//     forward goes cell by cell so does the adjoint (run_cells); else each
+//     lane walks its beam twice.  Front to back it recomputes tau at every source and adds
 //       dLoss/dL_src,b  += gJ_ib F_ib w e^{-tau},
 //       dLoss/dc_src    += sum_b c_b [ (w'/w) rhat - dtau_b/dc ]  (cells only),
 //       dtau/dc = (r/s) alpha(s) n + (tau_k(s)/s) (rhat - (r/s) n),
@@ -564,10 +565,15 @@ __global__ void __launch_bounds__(WARPS * 32, kAdjBlocksPerSM) k_walk_adjoint(co
 // [t0, t1) adds
 //   dLoss/dalpha -= S_(first s >= t1) (t1 - t0) + sum_{t0 <= s < t1} q (s - t0)
 // to its cell.  No order along the beam and no record of segments is needed.
-// 64^3 field, nside 2, 2 bands: 11.1 ms beam by beam.
+// Bound by issue slots and L2 latency, as k_walk.  Build, forward and adjoint
+// together against the adjoint beam by beam, which walks each beam and replays
+// its record: 64^3, nside 2, 2 bands, 17.8 -> 16.2 ms; nside 4, 3 bands, 43.1 ->
+// 40.3; 96^3, nside 4, 3 bands, 176 -> 148; 60^3 of clumps, nside 2, 21.0 -> 18.2.
+// With the two runs inlined apart (two copies of the look-up) 17.5, waiting for
+// instructions.
 constexpr int kAdjCellWarps = 4;
-// As k_walk: 28 warps per SM at nside 1 and 2 (64^3 gradient 17.9 -> 16.6 ms), 24
-// at nside 4.
+// As k_walk: 28 warps per SM at nside 1 and 2 (24: 17.9 ms, 28: 16.6 for the 64^3
+// gradient), 24 at nside 4.
 constexpr int kAdjCellBlocksPerSM = 7;
 constexpr int kAdjCellFineBlocksPerSM = 6;
 
@@ -1003,12 +1009,13 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
   g.w.cells = reinterpret_cast<int*>(p + b_walk);
   uint64_t* keys = reinterpret_cast<uint64_t*>(p + b_walk + up(b_cells));
   int* slots = reinterpret_cast<int*>(p + b_walk + up(b_cells) + b_keys);
-  if (A > 1) g.w.order = slots;
+  const bool sorted = A > 1 && A <= INT32_MAX;  // slots are 32-bit
+  if (sorted) g.w.order = slots;
   int rc = TREVR2_OK;
   auto run = [&]() -> int {
     T2_CUDA(cudaMemsetAsync(base, 0, zeroed, st));
     if (A > 0) {
-      if (A > 1) T2_CHECK(order_receivers(t, active, A, keys, slots, st));
+      if (sorted) T2_CHECK(order_receivers(t, active, A, keys, slots, st));
       T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
       void* args[] = {&g};
       T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(bw * 32)), args, smem, st));

@@ -11,14 +11,20 @@
 //    holds its direction (Sec. 2.5.1) with its projected distance s, r/s and
 //    the kernel g(r) = 1/(4 pi r^2) (or Eq. intint), then the sources are
 //    bucketed by beam and each bucket sorted by s.
-//  A (absorption, lane per beam): each lane walks its beam front to back
-//    through the same cut (near half first, so cells come in increasing
-//    distance), skipping cells without absorption and stopping at the
-//    farthest source of the beam.  Accepted internal cells use their
-//    transmission-averaged alpha for the beam's direction pair, leaves their
-//    bucket alpha.  Sources are resolved in order as the beam passes them:
-//    tau(s) = tau(t_in) + alpha (s - t_in), scaled by r/s (Sec. 2.5.1), and
-//    J_b += L_b e^{-tau_b} g(r) with a compensated FP32 sum per lane.
+//  A (absorption): the optical depth tau_k(s) of every source, along its beam
+//    through the same cut.  Two ways, chosen per tree and call by use_cells:
+//    - cell by cell (cells.cuh): the cut's absorbing cells are listed once, each
+//      is tested against the few beams that can cross it, and the depth of a
+//      crossing is added to the first source beyond it; running sums along each
+//      beam then give tau of all its sources.
+//    - beam by beam: each lane walks a beam front to back (near half first, so
+//      cells come in increasing distance), skipping cells without absorption,
+//      and stops at the farthest source of the beam; sources are resolved as
+//      the beam passes them, tau(s) = tau(t_in) + alpha (s - t_in).
+//    Accepted internal cells use their transmission-averaged alpha for the
+//    beam's direction pair, leaves their bucket alpha.  tau is scaled by r/s
+//    (Sec. 2.5.1), and J_b += L_b e^{-tau_b} g(r) with a compensated FP32 sum
+//    per lane.
 //  The lane partial sums are reduced in FP64, times Eq. taucorr with THICK.
 //
 // Discrete decisions (open or not, which beam) are taken in FP32 and taken
@@ -49,8 +55,9 @@ __device__ __forceinline__ void add_csm(const WalkArgs& a, int ref, int k, BandV
   for (int b = 0; b < NBP; ++b) tk.v[b] += c.v[b];
 }
 
-// Phase A beam by beam (beams finer than kCellNside, and directed beams, whose
-// directions no table holds): lanes take beams from the order above through a per-warp counter.
+// Phase A beam by beam (where use_cells says so, and for directed beams, whose
+// directions no table holds): lanes take beams from order_beams' list through a
+// per-warp counter.
 // Each beam first descends the receiver's ancestors (chain[0..], root to the
 // receiver's leaf, in shared memory): they hold the receiver, so they open,
 // and each one's chord is its parent's near-half interval; only their

@@ -106,3 +106,26 @@ def test_rows_do_not_depend_on_how_many_are_asked(t2, nside, theta, edge):
     with pytest.raises(t2.TrevrError, match="EINVAL"):
         tree.J(np.array([0, len(case["pos"]), 5]), nside, theta)
     tree.free()
+
+
+# the gradient on both sides of the same rule; 900 sources: two windows per
+# pass, 2500: two passes (1683 sources of a receiver at most)
+@pytest.mark.parametrize("nside,theta,n_src,nb", [
+    (1, 0.45, 4, 1), (2, 0.45, 16, 3), (2, 0.45, 15, 3), (2, 0.44, 16, 2), (4, 0.4, 64, 4),
+    (4, 0.4, 900, 2), (4, 0.4, 2500, 1)])
+def test_gradient_cells_and_beams(t2, oracle_mod, nside, theta, n_src, nb):
+    import test_gpu_adjoint as adj  # its bar holds here
+    case = workloads.random_case(300 if n_src > 64 else 800, n_src, nb=nb,
+                                 seed=nside * 100 + n_src, clumped=n_src > 60, n_active=24)
+    tree = _tree(t2, case)
+    act = case["active"]
+    rng = np.random.default_rng(3)
+    gJ = rng.uniform(0.0, 1.0, size=(len(act), nb)).astype(np.float32)
+    flags = t2.SOFT | t2.THICK
+    gk, gl = tree.J_backward(act, gJ, nside, theta, flags=flags)
+    ps = adj._all_params(case, n_kappa=100, n_dark=20)
+    ps = [ps[i] for i in rng.choice(len(ps), min(len(ps), 300), replace=False)]
+    want = adj._oracle_grad(oracle_mod.OracleTree.from_case(case), act, gJ.astype(np.float64),
+                            nside, theta, ps, flags)
+    adj._check(adj._gather(gk, gl, ps), want, f"nside={nside} sources={n_src}")
+    tree.free()
