@@ -21,11 +21,11 @@
 // receiver's J does not depend on the launch.
 //
 // What bounds it: L2 latency and instruction issue together (issue 53-60 % of
-// cycles, 28 of 32 lanes active, 42k instructions a receiver against 84k beam by
-// beam; the L1 is left about 50 KB and hits 7 %, so resident warps count: 28 a
-// SM at 72 registers beat 24, 20 and 16).  Measured against beam by beam, whole
-// calls: 2M clumpy field, nside 4, theta 0.5, 3 bands 259 -> 217 ms; its
-// per-bucket walk 45.2 -> 39.5 ms; 64^3, nside 2, 300 sources 6.6 -> 5.0 ms.
+// cycles, 28 of 32 lanes active, 51k instructions a receiver of the 96^3 field,
+// nside 4, against 84k beam by beam; the L1 is left about 50 KB and hits 17 %, so
+// resident warps count: see kCellWarpsPerSM).  Measured against beam by beam, whole
+// calls: 2M clumpy field, nside 4, theta 0.5, 3 bands 259 -> 200 ms; its
+// per-bucket walk 45.2 -> 35.7 ms; 64^3, nside 2, 300 sources 6.6 -> 5.0 ms.
 #pragma once
 
 #include "walk.cuh"

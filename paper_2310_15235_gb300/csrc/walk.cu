@@ -1463,8 +1463,12 @@ size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
 //  - sources: beams without any are not walked.  48^3, theta 0.5, nside 4: 30
 //    sources 2.90 / 2.41, 60 3.24 / 3.26, 120 3.63 / 4.16; nside 2: 3 sources
 //    1.88 / 1.79, 12 2.00 / 2.08; nside 1: 1 source 1.63 / 1.43, 3 1.66 / 1.75;
-//  - refinement opens cells that no beam with sources comes near: beam by beam.
-bool use_cells(const Tree* t, const Table* tb, float theta) {
+//  - refinement opens cells that no beam with sources comes near: beam by beam;
+//  - p-p absorption (pp) is mostly its particles, read through the L1, of which
+//    the cells' shared memory takes more.  64^3, nside 4: 3 bands 37.5 / 36.8 (80^3
+//    82.5 / 80.9), 1 band 31.9 / 33.8; nside 2: 3 bands 8.5 / 9.3.
+bool use_cells(const Tree* t, const Table* tb, float theta, bool pp) {
+  if (pp && tb->nside == 4 && t->nbp == 4) return false;
   return tb->nside <= kCellNside && !t->refine_on && theta >= (tb->nside < 4 ? 0.45f : 0.4f) &&
          3 * t->n_luminous >= 12 * tb->nside * tb->nside;
 }
@@ -1839,7 +1843,7 @@ static int launch_walk_bucket(Tree* t, Table* tb, const int64_t* active, int64_t
   bk.directed = target != nullptr;
   for (int c = 0; c < 3; ++c) bk.target[c] = target ? (target[c] - t->lo[c]) / t->size : 0.0;
   const bool csm = (flags & TREVR2_CSM) != 0;
-  const bool cells = use_cells(t, tb, theta) && !target;
+  const bool cells = use_cells(t, tb, theta, bk.pp != 0) && !target;
   if (cells) T2_CHECK(use_beam_map(tb, &a, st));
   const void* fn = bucket_kernel(t->nbp, bk.pp, csm, cells);
   const size_t smem = walk_layout(&a, kWalkWarps, cells, bk.pp != 0);
@@ -2259,7 +2263,7 @@ extern "C" int trevr2_batch_create(trevr2_tree* const* trees, int ntrees, const 
     Table* tb = nullptr;
     int rc = ensure_table(t, nside, st, &tb, (flags & TREVR2_LINEAR) != 0);
     if (rc) return fail(rc);
-    b->cells[i] = use_cells(t, tb, theta);
+    b->cells[i] = use_cells(t, tb, theta, b->pp);
     if (b->cells[i]) rc = ensure_beam_map(tb, st);
     if (rc) return fail(rc);
     if (!b->bucket) {

@@ -667,7 +667,7 @@ int read_status(Tree* t, cudaStream_t st);
 // block's bytes.  Beam by beam: the traversal stacks, the beam bucket offsets,
 // the beam order and its 32 bucket counts, the next-beam counter (padded to 16
 // bytes), the receiver's ancestor records.  Cell by cell: see cells.cuh.
-bool use_cells(const Tree* t, const Table* tb, float theta);
+bool use_cells(const Tree* t, const Table* tb, float theta, bool pp = false);
 int use_beam_map(Table* tb, WalkArgs* a, cudaStream_t st);
 size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp);
 
