@@ -42,7 +42,9 @@ extern "C" {
 #define TREVR2_ENOMEM (-2)      /* device or host allocation failed           */
 #define TREVR2_ECUDA (-3)       /* a CUDA runtime call failed                 */
 #define TREVR2_ETIMEOUT (-4)    /* a cooperative kernel's blocks gave up waiting
-                                   for one another (a bounded number of polls) */
+                                   for one another (a bounded number of polls);
+                                   the tree stays usable, a table that was not
+                                   finished is built again by the next call    */
 #define TREVR2_EUNSUPPORTED (-5)/* outside the supported sizes (see below)    */
 #define TREVR2_EINTERNAL (-6)   /* an internal capacity check failed          */
 
@@ -190,7 +192,9 @@ int trevr2_set_tau_refine(trevr2_tree* tree, double tau_refine, void* stream);
  * HEALPix beam table for `nside`, without running a walk.  trevr2_J does the
  * same on first use of an nside; calling this first keeps that work out of
  * a later trevr2_J.  The linear-average tables (TREVR2_LINEAR) are built by
- * the first call that asks for them.  Stream ordered, does not synchronise.
+ * the first call that asks for them.  Stream ordered, does not synchronise:
+ * a tables' kernel that gave up (ETIMEOUT) is reported by the next call that
+ * reads the tree's status.
  * Errors: EINVAL (NULL tree, bad nside), ENOMEM, ECUDA.
  */
 int trevr2_prepare(trevr2_tree* tree, int nside, void* stream);
@@ -366,6 +370,16 @@ const char* trevr2_last_error(void);
                                        the full capacity.  Read when a walk is
                                        set up (trevr2_J, trevr2_J_backward,
                                        trevr2_batch_create) */
+
+/* Further aids, beside the two above: */
+enum {
+  TREVR2_DEBUG_BARRIER_POLLS = 3  /* value n > 0: a cooperative kernel's blocks
+                                     wait for one another for at most n polls,
+                                     so that with n = 1 the wait runs out and
+                                     the call reports ETIMEOUT; 0 restores the
+                                     full number (about 16.8 million).  Read
+                                     when such a kernel is launched */
+};
 
 /* Sets one testing aid (EINVAL for an unknown `what` or a value out of range). */
 int trevr2_debug_set(int what, int64_t value);

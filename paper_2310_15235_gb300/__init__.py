@@ -94,12 +94,14 @@ def kernel_binary_version() -> int:
 
 DEBUG_FAIL_ALLOC = 1
 DEBUG_SOURCE_STACK = 2
+DEBUG_BARRIER_POLLS = 3
 
 
 def debug_set(what: int, value: int) -> None:
     """Testing aid: DEBUG_FAIL_ALLOC (the n-th device allocation from now on
-    fails with ENOMEM; -1 turns it off) or DEBUG_SOURCE_STACK (cap the source
-    cut's stack at c entries; 0 restores it)."""
+    fails with ENOMEM; -1 turns it off), DEBUG_SOURCE_STACK (cap the source
+    cut's stack at c entries; 0 restores it) or DEBUG_BARRIER_POLLS (a grid
+    barrier waits for at most n polls; 0 restores them)."""
     _check(load_library().trevr2_debug_set(int(what), int(value)))
 
 

@@ -50,6 +50,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 // Device allocations, and the failures a test can ask for (testing aids).
 static std::atomic<int64_t> g_fail_alloc_after{-1};   // -1: off
 static std::atomic<int> g_source_stack_cap{0};        // 0: off
+static std::atomic<uint32_t> g_barrier_polls{kBarrierSpins};
 
 // True for the one allocation a test asked to fail (then off again).
 static bool injected_alloc_failure() {
@@ -124,6 +125,7 @@ int device_alloc(void** p, size_t bytes, cudaStream_t st, const char* what) {
 }
 
 int debug_source_stack_cap() { return g_source_stack_cap.load(); }
+uint32_t barrier_polls() { return g_barrier_polls.load(); }
 
 // ---------------------------------------------------------------------------
 // Exclusive scan (block scan of 2048 values + recursive scan of block sums).
@@ -320,7 +322,7 @@ constexpr int kSortWarps = kSortThreads / 32;
 
 __global__ void __launch_bounds__(kSortThreads)
     k_radix_sort(uint64_t* ka, int* va, uint64_t* kb, int* vb, int64_t n, int passes, int* hist,
-                 uint32_t* bar, uint32_t* status) {
+                 uint32_t* bar, uint32_t* status, uint32_t polls) {
   __shared__ int base[256];
   __shared__ int wh[kSortWarps][256];
   __shared__ int tot2[2][256], bef2[2][256];
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(kSortThreads)
       atomicAdd(&base[(__ldcg(ka + i) >> shift) & 255u], 1);
     __syncthreads();
     if (t < 256) __stcg(hist + b * 256 + t, base[t]);
-    if (!grid_barrier(bar, nb, status)) return;
+    if (!grid_barrier(bar, nb, status, polls)) return;
     {
       const int d = t & 255, h = t >> 8;
       int tot = 0, bef = 0;
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kSortThreads)
     int* const tv = va;
     va = vb;
     vb = tv;
-    if (!grid_barrier(bar, nb, status)) return;
+    if (!grid_barrier(bar, nb, status, polls)) return;
   }
 }
 
@@ -486,7 +488,8 @@ int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, ui
   p += up(sizeof(int) * 256 * size_t(sort_blocks_bound(n)));
   uint32_t* bar = reinterpret_cast<uint32_t*>(p);
   T2_CUDA(cudaMemsetAsync(bar, 0, sizeof(uint32_t), st));
-  void* args[] = {&keys, &vals, &k2, &v2, &n, &passes, &hist, &bar, &status};
+  uint32_t polls = barrier_polls();
+  void* args[] = {&keys, &vals, &k2, &v2, &n, &passes, &hist, &bar, &status, &polls};
   T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_radix_sort), dim3(unsigned(nb)),
                                       dim3(kSortThreads), args, 0, st));
   note_launch();
@@ -726,6 +729,7 @@ struct TreeArgs {
   NodeW* nodes;
   BuildState* S;
   uint32_t* status;
+  uint32_t polls;     // of a grid barrier
 };
 constexpr int kTreeThreads = 512;
 constexpr int kSmallLevel = 1024;  // nodes of a level that block 0 does alone
@@ -983,7 +987,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_consta
       A.block_count[1] = le;
     }
   }
-  if (!grid_barrier(&S->bar, blocks, A.status)) return;
+  if (!grid_barrier(&S->bar, blocks, A.status, A.polls)) return;
   if (t == 0) {
     s_levels = __ldcg(&S->levels);
     s_int = __ldcg(&S->n_internal);
@@ -998,7 +1002,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_consta
   lb = s_lb;
   le = s_le;
   if (need) return;
-  if (!grid_barrier(&S->bar, blocks, A.status)) return;  // block_count is free again
+  if (!grid_barrier(&S->bar, blocks, A.status, A.polls)) return;  // block_count is free again
   // larger levels, all blocks
   while (le > lb) {
     const int per = (le - lb + blocks - 1) / blocks;
@@ -1014,7 +1018,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_consta
       mine += __syncthreads_count(m >= 0);
     }
     if (t == 0) __stcg(A.block_count + blockIdx.x, mine);
-    if (!grid_barrier(&S->bar, blocks, A.status)) return;
+    if (!grid_barrier(&S->bar, blocks, A.status, A.polls)) return;
     int before = 0, all = 0;
     {
       __shared__ int s_before, s_all;
@@ -1059,7 +1063,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_build_tree(const __grid_consta
     lb = le;
     le += 2 * all;
     ++level;
-    if (!grid_barrier(&S->bar, blocks, A.status)) return;
+    if (!grid_barrier(&S->bar, blocks, A.status, A.polls)) return;
     if (all == 0) break;
   }
   if (blockIdx.x == 0 && t == 0) {
@@ -1099,7 +1103,7 @@ __global__ void __launch_bounds__(kTreeThreads, 2) k_sum_levels(const __grid_con
     const int b0 = s_begin[d], b1 = s_begin[d + 1];
     const bool small = b1 - b0 <= kTreeThreads;
     if (together || (!small && d < level - 2)) {
-      if (!grid_barrier(&S->bar, blocks, A.status)) return;
+      if (!grid_barrier(&S->bar, blocks, A.status, A.polls)) return;
     } else {
       __syncthreads();
     }
@@ -1157,16 +1161,7 @@ static void free_tree(Tree* t, cudaStream_t st) {
   free_nodes(t, st);
   dfree(t->dtau, st);
   dfree(t->nodes_refined, st);
-  for (Table& tb : t->tables) {
-    dfree(tb.alpha, st);
-    dfree(tb.dirs, st);
-    dfree(tb.dirs64, st);
-    dfree(tb.geo, st);
-    dfree(tb.beam_inv, st);
-    dfree(tb.csm_tau, st);
-    dfree(tb.csm_d, st);
-    dfree(tb.csm_anti, st);
-  }
+  for (Table& tb : t->tables) free_table(&tb, st);
   t->tables.clear();
   if (t->scratch) cudaFreeAsync(t->scratch, st);
   t->scratch = nullptr;
@@ -1275,6 +1270,7 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
     A.nodes = t->nodes;
     A.S = state.p;
     A.status = t->status;
+    A.polls = barrier_polls();
     int blocks = 0, blocks_inner = 0;
     T2_CHECK(coop_blocks(cap, 2 * kTreeThreads, 1, &blocks));
     T2_CHECK(coop_blocks(cap, kTreeThreads, 2, &blocks_inner));
@@ -1345,6 +1341,10 @@ int trevr2_debug_set(int what, int64_t value) {
     case TREVR2_DEBUG_SOURCE_STACK:
       if (value < 0 || value > (int64_t(1) << 30)) break;
       g_source_stack_cap.store(int(value));
+      return TREVR2_OK;
+    case TREVR2_DEBUG_BARRIER_POLLS:
+      if (value < 0 || value > int64_t(kBarrierSpins)) break;
+      g_barrier_polls.store(value ? uint32_t(value) : kBarrierSpins);
       return TREVR2_OK;
     default:
       break;

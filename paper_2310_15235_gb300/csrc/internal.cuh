@@ -53,6 +53,7 @@ constexpr uint32_t kStatusBadInput = 1u << 2;
 constexpr uint32_t kStatusOutsideBox = 1u << 3;
 constexpr uint32_t kStatusBarrier = 1u << 4;     // a grid barrier gave up waiting
 constexpr uint32_t kStatusPPOverflow = 1u << 5;  // a p-p sphere held too many particles
+constexpr uint32_t kStatusTables = 1u << 6;      // the barrier was the tables' kernel's
 
 // Geometry of the transmission average for one cell shape and one beam pair:
 // weights V1/V (= V2/V), V12/V and the chord through the centre of a cell of
@@ -66,6 +67,10 @@ struct __align__(16) TransGeo {
 
 struct Table {
   int nside = 0;
+  // Whether a device status read after its kernel was free of kStatusTables.
+  // Until then the kernel may have given up at a barrier; settle_tables drops
+  // such a table, so that no later call takes it for a finished one.
+  bool checked = false;
   bool linear = false;         // linear absorption average instead of Eq. transmissionavg
   float* alpha = nullptr;      // [n_internal][P][nbp] normalised absorption
   float4* dirs = nullptr;      // [npix] beam directions (xyz), w = pair index (int bits)
@@ -147,12 +152,13 @@ struct Tree {
 // ---------------------------------------------------------------------------
 // Barrier of all blocks of one cooperative launch (so they are resident
 // together): *bar counts arrivals, from 0 at the launch.  The wait ends after
-// kBarrierSpins polls at the latest; then the barrier is marked as failed for
-// good and every block gets false and returns.
+// `polls` polls at the latest (barrier_polls()); then the barrier is marked as
+// failed for good, `bits` go to *status, and every block gets false and returns.
 constexpr uint32_t kBarrierSpins = 1u << 24;
 constexpr uint32_t kBarrierFailed = 0x80000000u;
 
-__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t blocks, uint32_t* status) {
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t blocks, uint32_t* status,
+                                             uint32_t polls, uint32_t bits = kStatusBarrier) {
   __shared__ uint32_t arrived_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -165,9 +171,9 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t blocks, uin
       do {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
         if ((seen | at) & kBarrierFailed) ok = 0;
-        if (ok && seen < target && ++spins == kBarrierSpins) {
+        if (ok && seen < target && ++spins == polls) {
           atomicOr(bar, kBarrierFailed);
-          if (status) atomicOr(status, kStatusBarrier);
+          if (status) atomicOr(status, bits);
           ok = 0;
         }
       } while (ok && seen < target);
@@ -231,6 +237,9 @@ struct DeviceTemp {
 // Capacity of the source cut's traversal stack set by
 // trevr2_debug_set(TREVR2_DEBUG_SOURCE_STACK, c); 0 when not set.
 int debug_source_stack_cap();
+// Polls of a grid barrier: kBarrierSpins, or what
+// trevr2_debug_set(TREVR2_DEBUG_BARRIER_POLLS, n) allows.
+uint32_t barrier_polls();
 
 // Blocks of a cooperative launch: at most per_sm per SM (the kernel's bound,
 // so that they are resident together), fewer where the work would leave them
@@ -259,6 +268,17 @@ int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, ui
 // cached): Eq. transmissionavg, or with `linear` the volume-weighted linear
 // average of the halves (Sec. 2.6's comparison scheme).
 int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear = false);
+
+// With the device status s of everything enqueued so far: drops the unchecked
+// tables where their kernel gave up, else marks them as checked.
+void settle_tables(Tree* t, uint32_t s, cudaStream_t st);
+
+// For callers that keep a table's pointers or hand its values out without a
+// read_status after them: reads the status if some table is unchecked
+// (synchronises `st` then; not while it is being captured), settles the tables
+// and returns ETIMEOUT when their kernel gave up.  Other status bits stay.
+int check_tables(Tree* t, cudaStream_t st);
+void free_table(Table* tb, cudaStream_t st);
 
 // The finest beams whose absorption is summed cell by cell (their indices fit
 // one byte: 192 beams at nside 4); finer ones are walked beam by beam.

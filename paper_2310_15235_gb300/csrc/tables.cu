@@ -210,6 +210,7 @@ struct TableArgs {
   float* tab;
   uint32_t* bar;
   uint32_t* status;
+  uint32_t polls;
   int level_begin[kMaxDepth + 3];
 };
 constexpr int kTableThreads = 512;
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) k_tables(const __grid_consta
   const int blocks = gridDim.x, t = threadIdx.x, P = A.P;
   const int64_t stride = int64_t(blocks) * kTableThreads, at = int64_t(blockIdx.x) * kTableThreads + t;
   for (int64_t k = at; k < A.npix; k += stride) table_dir(A.nside, A.npix, int(k), A.dirs64, A.dirs);
-  if (!grid_barrier(A.bar, blocks, A.status)) return;
+  if (!grid_barrier(A.bar, blocks, A.status, A.polls, kStatusBarrier | kStatusTables)) return;
   for (int64_t i = at; i < 3 * P; i += stride) {
     const int p = int(i % P);
     const double n[3] = {__ldcg(A.dirs64 + 3 * p), __ldcg(A.dirs64 + 3 * p + 1), __ldcg(A.dirs64 + 3 * p + 2)};
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) k_tables(const __grid_consta
     const int64_t items = int64_t(b1 - b0) * P;
     const bool small = items <= kTableSmall;
     if (together || !small) {
-      if (!grid_barrier(A.bar, blocks, A.status)) return;
+      if (!grid_barrier(A.bar, blocks, A.status, A.polls, kStatusBarrier | kStatusTables)) return;
     } else {
       __syncthreads();
     }
@@ -298,6 +299,50 @@ int ensure_beam_map(Table* tb, cudaStream_t st) {
   tb->beam_count = count;
   map.p = nullptr;
   return TREVR2_OK;
+}
+
+void free_table(Table* tb, cudaStream_t st) {
+  dfree(tb->alpha, st);
+  dfree(tb->dirs, st);
+  dfree(tb->dirs64, st);
+  dfree(tb->geo, st);
+  dfree(tb->beam_inv, st);
+  dfree(tb->csm_tau, st);
+  dfree(tb->csm_d, st);
+  dfree(tb->csm_anti, st);
+}
+
+void settle_tables(Tree* t, uint32_t s, cudaStream_t st) {
+  const bool gave_up = (s & kStatusTables) != 0;
+  for (size_t i = 0; i < t->tables.size();) {
+    Table& tb = t->tables[i];
+    if (gave_up && !tb.checked) {
+      free_table(&tb, st);
+      t->tables.erase(t->tables.begin() + i);
+    } else {
+      tb.checked = true;
+      ++i;
+    }
+  }
+}
+
+int check_tables(Tree* t, cudaStream_t st) {
+  bool all = true;
+  for (const Table& tb : t->tables) all = all && tb.checked;
+  if (all) return TREVR2_OK;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  T2_CUDA(cudaStreamIsCapturing(st, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return TREVR2_OK;
+  uint32_t s = 0;
+  T2_CUDA(cudaMemcpyAsync(&s, t->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  T2_CUDA(cudaStreamSynchronize(st));
+  settle_tables(t, s, st);
+  if (!(s & kStatusTables)) return TREVR2_OK;
+  const uint32_t rest = s & ~(kStatusBarrier | kStatusTables);
+  T2_CUDA(cudaMemcpyAsync(t->status, &rest, sizeof(uint32_t), cudaMemcpyHostToDevice, st));
+  T2_CUDA(cudaStreamSynchronize(st));
+  set_error("trevr2: a grid barrier of the absorption tables' kernel gave up waiting");
+  return TREVR2_ETIMEOUT;
 }
 
 int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear) {
@@ -339,6 +384,7 @@ int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear) 
   A.tab = tb.alpha;
   A.bar = t->status + 1;
   A.status = t->status;
+  A.polls = barrier_polls();
   int64_t widest = npix;
   for (int d = 0; d <= t->max_depth + 1; ++d) {
     A.level_begin[d] = int(t->level_begin[d]);
@@ -426,6 +472,7 @@ extern "C" int trevr2_alpha_table(trevr2_tree* tree, int nside, float* dst, size
   }
   Table* tb = nullptr;
   T2_CHECK(ensure_table(t, nside, st, &tb));
+  T2_CHECK(check_tables(t, st));
   int64_t total = t->n_nodes * int64_t(P) * t->nb;
   if (total > 0)
     k_export_alpha<<<unsigned((total + 255) / 256), 256, 0, st>>>(

@@ -1883,8 +1883,14 @@ int read_status(Tree* t, cudaStream_t st) {
   uint32_t s = 0;
   T2_CUDA(cudaMemcpyAsync(&s, t->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   T2_CUDA(cudaStreamSynchronize(st));
+  settle_tables(t, s, st);
   if (s == 0) return TREVR2_OK;
   T2_CUDA(cudaMemsetAsync(t->status, 0, sizeof(uint32_t), st));
+  if (s & kStatusBarrier) {  // first: every row of the call may be wrong
+    set_error("trevr2: a grid barrier of the %s gave up waiting",
+              (s & kStatusTables) ? "absorption tables' kernel" : "receivers' sort");
+    return TREVR2_ETIMEOUT;
+  }
   if (s & kStatusBadActive) {
     set_error("trevr2_J: an active index lies outside [0, N) (its row is NaN)");
     return TREVR2_EINVAL;
@@ -1897,10 +1903,6 @@ int read_status(Tree* t, cudaStream_t st) {
     set_error("trevr2_J: a bucket's p-p sphere holds more than %d particles (TREVR2_PP)",
               kPPCapacity);
     return TREVR2_EUNSUPPORTED;
-  }
-  if (s & kStatusBarrier) {
-    set_error("trevr2_J: a grid barrier of the receiver sort gave up waiting");
-    return TREVR2_ETIMEOUT;
   }
   set_error("trevr2: device status 0x%x", s);
   return TREVR2_EINTERNAL;
@@ -2292,6 +2294,10 @@ extern "C" int trevr2_batch_create(trevr2_tree* const* trees, int ntrees, const 
     b->bb.child[i] = t->child;
     b->bb.first[i] = t->first;
   }
+  // the plan keeps the tables' pointers: only of tables that were finished
+  if (nsub > 0)
+    for (Tree* t : b->trees)
+      if (const int rc = check_tables(t, st)) return fail(rc);
   // one shared-memory layout for all trees: the deepest one's
   for (int i = 0; i < ntrees; ++i) b->args.tree[i].max_depth = max_depth;
   b->args.max_depth = max_depth;

@@ -108,3 +108,15 @@ def test_new_entry_points_validate_on_host(lib):
     assert so.trevr2_J_directed(None, None, 0, 2, ctypes.c_float(0.75), None, 0, 16, None,
                                 None, None) == -1
     assert b"target is NULL" in so.trevr2_last_error()
+
+
+def test_further_testing_aids_match_header(lib):
+    """The header's enumerated testing aids and the binding's constants agree."""
+    with open(os.path.join(ROOT, "include", "trevr2.h")) as f:
+        hdr = f.read()
+    aids = {m.group(1): int(m.group(2)) for m in
+            re.finditer(r"^\s+TREVR2_(DEBUG_[A-Z_]+) = (\d+)", hdr, re.M)}
+    assert aids and all(getattr(lib, name) == value for name, value in aids.items())
+    so = lib.load_library()
+    for value in aids.values():
+        assert so.trevr2_debug_set(value, -1) == -1 and so.trevr2_debug_set(value, 0) == 0

@@ -1,0 +1,119 @@
+"""The cooperative kernels' bounded waits running out.
+
+A testing aid (trevr2_debug_set, DEBUG_BARRIER_POLLS) lets a grid barrier poll
+once, so that its blocks give up waiting for one another: the kernel returns,
+the call reports ETIMEOUT, and nothing the kernel left unfinished is used by
+a later call, whose results are those of an undisturbed one, bit for bit."""
+
+import numpy as np
+import pytest
+import torch
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+ETIMEOUT = -4
+
+
+@pytest.fixture(scope="module")
+def t2():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2310_15235_gb300 import build_lib
+    build_lib.build()
+    import paper_2310_15235_gb300 as mod
+    mod.load_library()
+    return mod
+
+
+@pytest.fixture(autouse=True)
+def _aid_off(t2):
+    yield
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+
+
+def _tree(t2, case):
+    return t2.build(case["pos"], case["mass"], case["kappa"], case["lum"], case["h"],
+                    case["box_lo"], case["box_size"], case["bucket"])
+
+
+def _batch(t2, trees, rows):
+    return t2.Batch(trees, np.array([0, rows], np.int64), np.array([0], np.int32), nside=2,
+                    theta=0.75)
+
+
+def test_aid_range(t2):
+    for v in (-1, (1 << 24) + 1):
+        with pytest.raises(t2.TrevrError, match="EINVAL"):
+            t2.debug_set(t2.DEBUG_BARRIER_POLLS, v)
+
+
+@pytest.mark.parametrize("how", ["J", "backward", "prepare", "alpha_table", "batch"])
+def test_unfinished_tables_are_not_kept(t2, how):
+    case = workloads.random_case(6000, 60, nb=2, seed=401, clumped=True)
+    act = case["active"][:900]
+    other = _tree(t2, case)
+    ref = other.J(act, 2, 0.75)
+    ref_alpha = other.alpha_table(2)
+    other.free()
+    tree = _tree(t2, case)
+    held = t2.debug_pool_used()
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1)
+    with pytest.raises(t2.TrevrError, match="absorption tables") as e:
+        if how == "J":
+            tree.J(act, 2, 0.75)
+        elif how == "backward":
+            tree.J_backward(act, np.ones((len(act), 2), np.float32), 2, 0.75)
+        elif how == "prepare":
+            tree.prepare(2)
+            tree.status()
+        elif how == "alpha_table":
+            tree.alpha_table(2)
+        else:
+            _batch(t2, [tree], len(act))
+    assert e.value.code == ETIMEOUT
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+    if how in ("prepare", "alpha_table", "batch"):
+        assert t2.debug_pool_used() == held  # J also keeps its walk buffers
+    tree.status()  # reported once
+    assert torch.equal(tree.J(act, 2, 0.75), ref)
+    assert torch.equal(tree.alpha_table(2), ref_alpha)
+    plan = _batch(t2, [tree], len(act))
+    assert torch.equal(plan.run(torch.as_tensor(act, device="cuda")), ref)
+    plan.status()
+    plan.free()
+    # a table found good before stays when a later one gives up
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1)
+    with pytest.raises(t2.TrevrError, match="absorption tables"):
+        tree.J(act, 4, 0.5)
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+    launches = t2.kernel_launches()
+    assert torch.equal(tree.J(act, 2, 0.75), ref)
+    assert t2.kernel_launches() - launches <= 2  # the walk, its receivers' order
+    tree.free()
+
+
+@pytest.mark.parametrize("flags", ["0", "BUCKET", "backward"])
+def test_receiver_order(t2, flags):
+    case = workloads.random_case(6000, 60, nb=2, seed=402)
+    act = np.random.default_rng(1).integers(0, 6000, size=60_000)
+    tree = _tree(t2, case)
+    g = np.ones((len(act), 2), np.float32)
+
+    def call():
+        if flags == "backward":
+            return tree.J_backward(act, g, 2, 0.75)[0]
+        return tree.J(act, 2, 0.75, flags=t2.BUCKET if flags == "BUCKET" else 0)
+
+    ref = call()
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1)
+    with pytest.raises(t2.TrevrError, match="receivers' sort") as e:
+        call()
+    assert e.value.code == ETIMEOUT
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+    if flags == "backward":  # summed with FP32 atomics in any order
+        torch.testing.assert_close(call(), ref, rtol=1e-4, atol=1e-6 * float(ref.abs().max()))
+    else:
+        assert torch.equal(call(), ref)
+    tree.free()
