@@ -1191,6 +1191,7 @@ struct BatchArgs {
   uint64_t* ukeys;                // [distinct] the distinct keys
   float* Ju;                      // [distinct][nbsel] J of each distinct key
   int* n_distinct;                // device count of distinct keys
+  const uint32_t* sort_status;    // the word that gets the sort's kStatusBarrier
   SrcEntry* srcU;
   int* pixU;
   SrcEntry* srcV;
@@ -1271,6 +1272,13 @@ __global__ void k_batch_distinct(const __grid_constant__ BatchArgs B) {
   if (p < B.total && first_of_key(B.keys, p)) B.ukeys[B.first_scan[p]] = B.keys[p];
 }
 
+// Whether the sort of the rows' keys gave up at a barrier: their order then
+// means nothing (a tree's range could hold other trees' element positions, past
+// its own elements), so no tree is walked and every row is NaN.
+__device__ __forceinline__ bool batch_unsorted(const BatchArgs& B) {
+  return (*B.sort_status & kStatusBarrier) != 0;
+}
+
 // Every row gets its key's J (NaN for an invalid receiver).
 __global__ void k_batch_scatter(const __grid_constant__ BatchArgs B) {
   const int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
@@ -1278,7 +1286,7 @@ __global__ void k_batch_scatter(const __grid_constant__ BatchArgs B) {
   const uint64_t key = B.keys[p];
   const int64_t r = B.rows[p];
   const int64_t u = B.first_scan[p] - (first_of_key(B.keys, p) ? 0 : 1);
-  const bool ok = int(key >> B.key_shift) < B.ntrees;
+  const bool ok = int(key >> B.key_shift) < B.ntrees && !batch_unsorted(B);
   for (int j = 0; j < B.nbsel; ++j)
     B.J[r * B.nbsel + j] = ok ? B.Ju[u * B.nbsel + j] : __int_as_float(0x7fc00000);
 }
@@ -1288,7 +1296,7 @@ __global__ void k_batch_scatter(const __grid_constant__ BatchArgs B) {
 __global__ void k_batch_tree_range(const __grid_constant__ BatchArgs B) {
   const int t = threadIdx.x;
   if (t > B.ntrees) return;
-  int lo = 0, hi = *B.n_distinct;
+  int lo = 0, hi = batch_unsorted(B) ? 0 : *B.n_distinct;
   const uint64_t key = uint64_t(t) << B.key_shift;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -2356,6 +2364,7 @@ extern "C" int trevr2_batch_create(trevr2_tree* const* trees, int ntrees, const 
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(cuda_fail(e, "cudaMemcpyAsync(batch metadata)"));
   }
+  b->args.sort_status = b->trees[0]->status;
   b->args.offsets = b->d_offsets;
   b->args.tree_of = b->d_tree_of;
   b->args.counter = b->counter;

@@ -117,3 +117,31 @@ def test_receiver_order(t2, flags):
     else:
         assert torch.equal(call(), ref)
     tree.free()
+
+
+@pytest.mark.parametrize("flags", ["0", "BUCKET"])
+def test_batch_rows(t2, flags):
+    """A batch whose rows were not sorted walks nothing (a tree's range could
+    hold another, larger tree's elements): NaN rows and ETIMEOUT."""
+    cases = [workloads.random_case(400, 30, nb=2, seed=404),
+             workloads.random_case(9000, 60, nb=2, seed=403, clumped=True)]
+    trees = [_tree(t2, c) for c in cases]
+    rng = np.random.default_rng(2)
+    active = torch.as_tensor(np.concatenate([rng.integers(0, 400, size=30_000),
+                                             rng.integers(0, 9000, size=50_001)]), device="cuda")
+    plan = t2.Batch(trees, np.array([0, 30_000, 80_001], np.int64), np.array([0, 1], np.int32),
+                    nside=2, theta=0.75, flags=t2.BUCKET if flags == "BUCKET" else 0)
+    ref = plan.run(active)
+    plan.status()
+    assert bool(torch.isfinite(ref).all())
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1)
+    J = plan.run(active)
+    with pytest.raises(t2.TrevrError, match="receivers' sort") as e:
+        plan.status()
+    assert e.value.code == ETIMEOUT and bool(torch.isnan(J).all())
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+    assert torch.equal(plan.run(active), ref)
+    plan.status()
+    plan.free()
+    for tr in trees:
+        tr.free()
