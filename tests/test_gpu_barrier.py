@@ -145,3 +145,40 @@ def test_batch_rows(t2, flags):
     plan.free()
     for tr in trees:
         tr.free()
+
+
+# sizes: one block's sort and the cooperative one
+@pytest.mark.parametrize("n", [6000, 30_000])
+def test_build(t2, n):
+    case = workloads.random_case(n, 60, nb=2, seed=405, clumped=True)
+    base = t2.debug_pool_used()
+    ref = _tree(t2, case)
+    perm, B = ref.export("perm"), ref.export("B")
+    ref.free()
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1)
+    with pytest.raises(t2.TrevrError, match="gave up waiting") as e:
+        _tree(t2, case)
+    assert e.value.code == ETIMEOUT and t2.debug_pool_used() == base
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 0)
+    tree = _tree(t2, case)
+    assert torch.equal(tree.export("perm"), perm) and torch.equal(tree.export("B"), B)
+    tree.free()
+
+
+def test_refusal_costs_no_build(t2):
+    """A set outside its cube is refused in about the time of its check and
+    sort: its positions are all clamped to one corner, and building that tree
+    took one thread 1M additions (634 ms; now 0.45 ms)."""
+    n = 1_000_000
+    x = torch.rand((n, 3), dtype=torch.float64, device="cuda") + 5.0
+    one = torch.ones(n, dtype=torch.float32, device="cuda")
+    cols = torch.ones((n, 1), dtype=torch.float32, device="cuda")
+    t2.build(x, one, cols, cols, one, box_lo=(5.0, 5.0, 5.0), box_size=1.0).free()
+    torch.cuda.synchronize()
+    e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    e0.record()
+    with pytest.raises(t2.TrevrError, match="outside the given root cube"):
+        t2.build(x, one, cols, cols, one, box_lo=(0.0, 0.0, 0.0), box_size=1.0)
+    e1.record()
+    torch.cuda.synchronize()
+    assert e0.elapsed_time(e1) < 100.0
