@@ -373,12 +373,22 @@ const char* trevr2_last_error(void);
 
 /* Further aids, beside the two above: */
 enum {
-  TREVR2_DEBUG_BARRIER_POLLS = 3  /* value n > 0: a cooperative kernel's blocks
+  TREVR2_DEBUG_BARRIER_POLLS = 3, /* value n > 0: a cooperative kernel's blocks
                                      wait for one another for at most n polls,
                                      so that with n = 1 the wait runs out and
                                      the call reports ETIMEOUT; 0 restores the
                                      full number (about 16.8 million).  Read
                                      when such a kernel is launched */
+  TREVR2_DEBUG_CELL_CAP = 4,      /* value c > 0, a multiple of 32: a walk lists
+                                     at most c absorbing cells of a cut at once
+                                     (2048 at most), so that a small field's cut
+                                     takes several windows; 0 restores 2048.
+                                     Read like TREVR2_DEBUG_SOURCE_STACK (and
+                                     by trevr2_batch_autotune) */
+  TREVR2_DEBUG_TEAM_HITS = 5      /* value c > 0: each warp of a block that walks
+                                     one receiver lists at most c crossings, so
+                                     that more of them take the one-warp way;
+                                     0 restores 2048 */
 };
 
 /* Sets one testing aid (EINVAL for an unknown `what` or a value out of range). */

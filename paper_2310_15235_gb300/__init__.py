@@ -95,13 +95,17 @@ def kernel_binary_version() -> int:
 DEBUG_FAIL_ALLOC = 1
 DEBUG_SOURCE_STACK = 2
 DEBUG_BARRIER_POLLS = 3
+DEBUG_CELL_CAP = 4
+DEBUG_TEAM_HITS = 5
 
 
 def debug_set(what: int, value: int) -> None:
     """Testing aid: DEBUG_FAIL_ALLOC (the n-th device allocation from now on
     fails with ENOMEM; -1 turns it off), DEBUG_SOURCE_STACK (cap the source
-    cut's stack at c entries; 0 restores it) or DEBUG_BARRIER_POLLS (a grid
-    barrier waits for at most n polls; 0 restores them)."""
+    cut's stack at c entries; 0 restores it), DEBUG_BARRIER_POLLS (a grid
+    barrier waits for at most n polls), DEBUG_CELL_CAP (a walk lists at most c
+    cells at once) or DEBUG_TEAM_HITS (a block's warp lists at most c
+    crossings); 0 restores each of these."""
     _check(load_library().trevr2_debug_set(int(what), int(value)))
 
 

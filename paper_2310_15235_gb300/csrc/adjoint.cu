@@ -958,7 +958,7 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
                             : adjoint_kernel<4>(cells, nside);
   const size_t smem = cells ? walk_layout(&wa, bw, true, false)
                             : adjoint_smem(bw, wa.stack_ints, wa.npix);
-  wa.cell_cap = cells ? kCellCap : 0;
+  wa.cell_cap = cells ? cell_list_cap() : 0;
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, bw, smem, &per_sm, &sms));
   int64_t blocks = int64_t(sms) * per_sm;
@@ -981,7 +981,7 @@ extern "C" int trevr2_J_backward(trevr2_tree* tree, const int64_t* active, int64
   const int seg_cap = !cells && int64_t(std::max<int64_t>(t->n_internal, 1)) * P < INT32_MAX ? kSegCap : 0;
   const size_t b_seg = up(sizeof(float4) * warps * size_t(seg_cap) * 32);
   const size_t b_walk = up(warps * size_t(wa.M) * (2 * sizeof(SrcEntry) + sizeof(int)));
-  const size_t b_cells = cells ? warps * (size_t(kCellCap) + 4 * size_t(wa.M)) * sizeof(int) : 0;
+  const size_t b_cells = cells ? warps * (size_t(wa.cell_cap) + 4 * size_t(wa.M)) * sizeof(int) : 0;
   // receivers in the tree's order, so that neighbouring walks share its nodes
   const size_t b_keys = up(sizeof(uint64_t) * size_t(A)), b_slots = up(sizeof(int) * size_t(A));
   char* base = nullptr;

@@ -13,6 +13,7 @@
 // walk of few receivers by blocks: 33k elements 2.21 -> 0.87 ms, 4k 1.45 -> 0.41,
 // 2.1M and a 1000-receiver rung 5.96 -> 2.78.
 #include <atomic>
+#include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -51,6 +52,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 static std::atomic<int64_t> g_fail_alloc_after{-1};   // -1: off
 static std::atomic<int> g_source_stack_cap{0};        // 0: off
 static std::atomic<uint32_t> g_barrier_polls{kBarrierSpins};
+static std::atomic<int> g_cell_cap{INT_MAX}, g_team_hits{INT_MAX};
 
 // True for the one allocation a test asked to fail (then off again).
 static bool injected_alloc_failure() {
@@ -126,6 +128,8 @@ int device_alloc(void** p, size_t bytes, cudaStream_t st, const char* what) {
 
 int debug_source_stack_cap() { return g_source_stack_cap.load(); }
 uint32_t barrier_polls() { return g_barrier_polls.load(); }
+int debug_cell_cap() { return g_cell_cap.load(); }
+int debug_team_hits() { return g_team_hits.load(); }
 
 // ---------------------------------------------------------------------------
 // Exclusive scan (block scan of 2048 values + recursive scan of block sums).
@@ -1354,6 +1358,14 @@ int trevr2_debug_set(int what, int64_t value) {
     case TREVR2_DEBUG_BARRIER_POLLS:
       if (value < 0 || value > int64_t(kBarrierSpins)) break;
       g_barrier_polls.store(value ? uint32_t(value) : kBarrierSpins);
+      return TREVR2_OK;
+    case TREVR2_DEBUG_CELL_CAP:  // (the buffers behind the list are 16-byte aligned)
+      if (value < 0 || value > (1 << 20) || value % 32 != 0) break;
+      g_cell_cap.store(value ? int(value) : INT_MAX);
+      return TREVR2_OK;
+    case TREVR2_DEBUG_TEAM_HITS:
+      if (value < 0 || value > (1 << 20)) break;
+      g_team_hits.store(value ? int(value) : INT_MAX);
       return TREVR2_OK;
     default:
       break;

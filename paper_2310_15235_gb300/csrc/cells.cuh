@@ -28,6 +28,8 @@
 // per-bucket walk 45.2 -> 35.7 ms; 64^3, nside 2, 300 sources 6.6 -> 5.0 ms.
 #pragma once
 
+#include <algorithm>
+
 #include "walk.cuh"
 
 namespace trevr2 {
@@ -480,6 +482,8 @@ __device__ __forceinline__ void sum_increments(int lane, int npix, const int* of
 }
 
 constexpr int kCellCap = 2048;  // cells of a cut listed at once
+// The same, or fewer with trevr2_debug_set(TREVR2_DEBUG_CELL_CAP, c).
+inline int cell_list_cap() { return std::min(kCellCap, debug_cell_cap()); }
 
 // A warp's part of a walk block's shared memory and of the walk buffers.
 struct WarpMem {

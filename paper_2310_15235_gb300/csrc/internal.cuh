@@ -240,6 +240,10 @@ int debug_source_stack_cap();
 // Polls of a grid barrier: kBarrierSpins, or what
 // trevr2_debug_set(TREVR2_DEBUG_BARRIER_POLLS, n) allows.
 uint32_t barrier_polls();
+// Capacities lowered by TREVR2_DEBUG_CELL_CAP and TREVR2_DEBUG_TEAM_HITS
+// (INT_MAX when not set).
+int debug_cell_cap();
+int debug_team_hits();
 
 // Blocks of a cooperative launch: at most per_sm per SM (the kernel's bound,
 // so that they are resident together), fewer where the work would leave them

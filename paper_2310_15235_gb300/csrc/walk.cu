@@ -381,6 +381,7 @@ constexpr int kTeamBatches = kCellCap / 32;
 
 struct TeamArgs {
   float4* hits;  // [blocks][kTeamWarps][kTeamHits]
+  int max_hits;  // crossings a warp lists (kTeamHits, or fewer in a test)
 };
 
 template <int NBP>
@@ -470,13 +471,13 @@ __global__ void __launch_bounds__(kTeamWarps * 32, 2)
         cross_batch<false>(a, x, lane, q, stage, w.binv, w.far, 0.0f, [&](bool hit, float t0, float t1, int row, int k) {
           const unsigned hm = __ballot_sync(0xffffffffu, hit);
           const int at = nh + __popc(hm & lt);
-          if (hit && at < kTeamHits)
+          if (hit && at < tm.max_hits)
             mine[at] = make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
           nh += __popc(hm);
         });
         if (lane == 0) seg[b] = make_int2(from, nh - from);
       }
-      if (nh > kTeamHits && lane == 0) s_full = 1;
+      if (nh > tm.max_hits && lane == 0) s_full = 1;
       __syncthreads();
       if (s_full) {
         if (wid == 0) walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
@@ -1574,7 +1575,7 @@ static int launch_walk_team(Tree* t, WalkArgs a, cudaStream_t st) {
   int per_sm = 0, sms = 0;
   T2_CHECK(config_walk_kernel(fn, kTeamWarps, smem, &per_sm, &sms));
   const size_t blocks = size_t(std::max<int64_t>(1, std::min<int64_t>(int64_t(sms) * per_sm, a.A)));
-  a.cell_cap = kCellCap;
+  a.cell_cap = cell_list_cap();
   const size_t wb = (walk_buffer_bytes(blocks, a.M, a.cell_cap) + 255) & ~size_t(255);
   const size_t need = wb + blocks * kTeamWarps * kTeamHits * sizeof(float4);
   T2_CHECK(grow_buffer(&t->scratch, &t->scratch_bytes, need, st, "walk buffers"));
@@ -1582,6 +1583,7 @@ static int launch_walk_team(Tree* t, WalkArgs a, cudaStream_t st) {
   place_walk_buffers(base, blocks, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU, &a.cells);
   TeamArgs tm;
   tm.hits = reinterpret_cast<float4*>(base + wb);
+  tm.max_hits = std::min(kTeamHits, debug_team_hits());
   T2_CUDA(cudaMemsetAsync(t->counter, 0, sizeof(unsigned long long), st));
   void* args[] = {&a, &tm};
   T2_CUDA(cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(kTeamWarps * 32), args, smem, st));
@@ -1618,7 +1620,7 @@ static int launch_walk(Tree* t, Table* tb, const int64_t* active, int64_t A, int
   blocks = std::min<int64_t>(blocks, (A + kWalkWarps - 1) / kWalkWarps);
   blocks = std::max<int64_t>(blocks, 1);
   const size_t warps = size_t(blocks) * kWalkWarps;
-  a.cell_cap = cells ? kCellCap : 0;
+  a.cell_cap = cells ? cell_list_cap() : 0;
   const size_t need = walk_buffer_bytes(warps, a.M, a.cell_cap);
   T2_CHECK(grow_buffer(&t->scratch, &t->scratch_bytes, need, st, "walk buffers"));
   place_walk_buffers(static_cast<char*>(t->scratch), warps, a.M, &a.srcU, &a.srcV, &a.srcT, &a.pixU,
@@ -1861,7 +1863,7 @@ static int launch_walk_bucket(Tree* t, Table* tb, const int64_t* active, int64_t
   blocks = std::min<int64_t>(blocks, (A + kWalkWarps - 1) / kWalkWarps);
   blocks = std::max<int64_t>(blocks, 1);
   const size_t warps = size_t(blocks) * kWalkWarps;
-  a.cell_cap = cells ? kCellCap : 0;
+  a.cell_cap = cells ? cell_list_cap() : 0;
   const size_t wb = (walk_buffer_bytes(warps, a.M, a.cell_cap) + 255) & ~size_t(255);
   const size_t ob = (warps * kOriginWords * sizeof(double) + 255) & ~size_t(255);
   const size_t pb = warps * size_t(bk.pp_cap) *
@@ -2055,10 +2057,11 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
   const void* fn[2] = {nullptr, nullptr};
   size_t smem[2] = {0, 0};
   int64_t blocks[2] = {0, 0};
+  const int cells = cell_list_cap();
   for (size_t i = 0; i < b->trees.size(); ++i) {
     const int c = b->cells[i] ? 1 : 0;
     smem[c] = walk_layout(&b->args.tree[i], warps, c != 0, b->pp);
-    b->args.tree[i].cell_cap = c ? kCellCap : 0;
+    b->args.tree[i].cell_cap = c ? cells : 0;
     if (fn[c]) continue;
     fn[c] = b->bucket ? bucket_batched_kernel(b->nbp, b->pp, b->csm, c != 0)
                       : walk_kernel(b->nbp, warps, true, c != 0, b->nside);
@@ -2067,7 +2070,7 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
     const int64_t g = std::min<int64_t>(int64_t(sms) * per_sm, (limit + warps - 1) / warps);
     blocks[c] = std::max<int64_t>(g, 1);
   }
-  const int cell_cap = blocks[1] ? kCellCap : 0;
+  const int cell_cap = blocks[1] ? cells : 0;
   const size_t nw = size_t(std::max(blocks[0], blocks[1])) * warps;
   // per-bucket plans: the warps' FP64 origin slots and p-p particle arrays
   const size_t wb = (walk_buffer_bytes(nw, M, cell_cap) + 255) & ~size_t(255);
