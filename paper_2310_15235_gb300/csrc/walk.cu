@@ -373,7 +373,12 @@ __global__ void __launch_bounds__(WARPS * 32, kWarpsPerSM / WARPS)
 // round the warps, which list their crossings batch by batch; then every warp
 // takes the crossings of its own beams from all batches, in their order, so
 // each source's sums run exactly as in k_walk and the row is bit for bit the
-// same.  A receiver whose cut or crossings do not fit is walked by warp 0 alone.
+// same.  More sources or cells than the buffers hold go through passes and
+// windows, as in k_walk.  (Walked by warp 0 alone, seven warps waiting, such
+// receivers made rungs slower than a warp each or the walk beam by beam: 96^3,
+// 200k sources, nside 4, 1000 receivers, theta 0.5 1.75 ms, 0.4 3.87; now 0.94,
+// 1.90; beam by beam 1.53, 2.31.)  A receiver whose crossings overflow a warp's
+// list (a window holds about three a cell, for eight lists) is walked by warp 0.
 // 100 receivers of the 96^3 field: 0.49 -> 0.20 ms a call (see team_receivers).
 constexpr int kTeamWarps = 8;
 constexpr int kTeamHits = 2048;  // crossings a warp lists
@@ -424,98 +429,119 @@ __global__ void __launch_bounds__(kTeamWarps * 32, 2)
     const int si = a.inv[io];
     const float4 xr = a.pos32[si];
     const float3 x = grazing_coords(a, si, make_float3(xr.x, xr.y, xr.z));
-    if (wid == 0) {
-      const int2 c = phase_cut<false, false>(a, x, si, lane, w.stk, a.src_stack_cap, w.U, 0, w.cells, 0, 0.0f);
-      if (lane == 0) {
-        s_total = c.x;
-        s_listed = c.y;
-      }
-    }
-    __syncthreads();
-    const int total = s_total, listed = s_listed;
-    if (total > a.M || listed > a.cell_cap) {
-      if (wid == 0) walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
-      continue;
-    }
-    make_sources(a, x, si, tid, w.U, w.Up, total, kTeamWarps * 32);
-    __syncthreads();
-    if (wid == 0) {
-      const int n0 = total <= 0           ? 0
-                   : total <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, total, w.V, w.off, w.stk)
-                                        : bin_sources(a.npix, lane, w.U, w.Up, total, w.V, w.off);
-      if (lane == 0) s_n = n0;
-    }
-    __syncthreads();
-    const int n = s_n;
-    if (n > 0) {
-      BandVec<NBP> zero;
+    float Js[NBP], Jc[NBP];  // warp 0's lane sums
 #pragma unroll
-      for (int b = 0; b < NBP; ++b) zero.v[b] = 0.0f;
-      for (int e = tid; e < n; e += kTeamWarps * 32) {
-        ss[e] = w.V[e].s;
-        store_bands<NBP>(w.T + e * NBP, zero);
-        store_bands<NBP>(w.own + e * NBP, zero);
-      }
-      for (int k = tid; k < a.npix; k += kTeamWarps * 32) {
-        const int s1 = w.off[k];
-        w.far[beam_slot(k)] = s1 > (k ? w.off[k - 1] : 0) ? w.V[s1 - 1].s : -1.0f;
-      }
-      __syncthreads();
-      // this warp's batches: their crossings, listed
-      const int batches = (listed + 31) / 32;
-      int nh = 0;
-      float4* mine = lists + wid * kTeamHits;
-      for (int b = wid; b < batches; b += kTeamWarps) {
-        const int from = nh;
-        const int q = 32 * b + lane < listed ? w.cells[32 * b + lane] : -1;
-        cross_batch<false>(a, x, lane, q, stage, w.binv, w.far, 0.0f, [&](bool hit, float t0, float t1, int row, int k) {
-          const unsigned hm = __ballot_sync(0xffffffffu, hit);
-          const int at = nh + __popc(hm & lt);
-          if (hit && at < tm.max_hits)
-            mine[at] = make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
-          nh += __popc(hm);
-        });
-        if (lane == 0) seg[b] = make_int2(from, nh - from);
-      }
-      if (nh > tm.max_hits && lane == 0) s_full = 1;
-      __syncthreads();
-      if (s_full) {
-        if (wid == 0) walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
-        continue;
-      }
-      // this warp's beams: their crossings of all batches, in order
-      int nq = 0;
-      for (int b = 0; b < batches; ++b) {
-        const int2 sg = seg[b];
-        const float4* from = lists + (b % kTeamWarps) * kTeamHits + sg.x;
-        for (int i = 0; i < sg.y; i += 32) {
-          float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          if (i + lane < sg.y) h = __ldcg(from + i + lane);
-          const bool take = i + lane < sg.y && (__float_as_int(h.w) % kTeamWarps) == wid;
-          const unsigned m = __ballot_sync(0xffffffffu, take);
-          if (take) queue[(nq + __popc(m & lt)) & 63] = h;
-          const int was = nq;
-          nq += __popc(m);
-          __syncwarp();
-          if ((nq ^ was) & 32)
-            add_crossings<NBP, true>(a, lane, true, queue[(was & 32) + lane], w.binv, ss, w.off, 0, n,
-                                     0.0f, w.T, w.own, true, [](int, const BandVec<NBP>&) {});
+    for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
+    bool fits = true;
+    int n = 0;
+    for (int lo = 0, clo = 0;;) {  // passes and windows, as walk_origin
+      if (wid == 0) {
+        // a later window only lists cells: no source has an index that high
+        const int2 c = phase_cut<false, false>(a, x, si, lane, w.stk, a.src_stack_cap, w.U,
+                                               clo ? INT32_MAX : lo, w.cells, clo, 0.0f);
+        if (lane == 0) {
+          s_total = c.x;
+          s_listed = c.y;
         }
       }
-      __syncwarp();
-      if (nq & 31)
-        add_crossings<NBP, true>(a, lane, lane < (nq & 31), queue[(nq & 32) + lane], w.binv, ss,
-                                 w.off, 0, n, 0.0f, w.T, w.own, true, [](int, const BandVec<NBP>&) {});
       __syncthreads();
-      sum_increments<NBP>(tid, a.npix, w.off, w.T, w.own, kTeamWarps * 32);
-      __syncthreads();
+      const int total = s_total, listed = s_listed;
+      const bool first = clo == 0;
+      if (first) {
+        const int staged = min(total - lo, a.M);
+        make_sources(a, x, si, tid, w.U, w.Up, staged, kTeamWarps * 32);
+        __syncthreads();
+        if (wid == 0) {
+          const int n0 = staged <= 0           ? 0
+                       : staged <= a.bin_cap ? bin_sources_small(a, lane, w.U, w.Up, staged, w.V, w.off, w.stk)
+                                             : bin_sources(a.npix, lane, w.U, w.Up, staged, w.V, w.off);
+          if (lane == 0) s_n = n0;
+        }
+        __syncthreads();
+        n = s_n;
+      }
+      if (n > 0) {
+        if (first) {
+          BandVec<NBP> zero;
+#pragma unroll
+          for (int b = 0; b < NBP; ++b) zero.v[b] = 0.0f;
+          for (int e = tid; e < n; e += kTeamWarps * 32) {
+            ss[e] = w.V[e].s;
+            store_bands<NBP>(w.T + e * NBP, zero);
+            store_bands<NBP>(w.own + e * NBP, zero);
+          }
+          for (int k = tid; k < a.npix; k += kTeamWarps * 32) {
+            const int s1 = w.off[k];
+            w.far[beam_slot(k)] = s1 > (k ? w.off[k - 1] : 0) ? w.V[s1 - 1].s : -1.0f;
+          }
+          __syncthreads();
+        }
+        // this warp's batches: their crossings, listed
+        const int nc = min(listed - clo, a.cell_cap), batches = (nc + 31) / 32;
+        int nh = 0;
+        float4* mine = lists + wid * kTeamHits;
+        for (int b = wid; b < batches; b += kTeamWarps) {
+          const int from = nh;
+          const int q = 32 * b + lane < nc ? w.cells[32 * b + lane] : -1;
+          cross_batch<false>(a, x, lane, q, stage, w.binv, w.far, 0.0f, [&](bool hit, float t0, float t1, int row, int k) {
+            const unsigned hm = __ballot_sync(0xffffffffu, hit);
+            const int at = nh + __popc(hm & lt);
+            if (hit && at < tm.max_hits)
+              mine[at] = make_float4(t0, t1, __int_as_float(row), __int_as_float(k));
+            nh += __popc(hm);
+          });
+          if (lane == 0) seg[b] = make_int2(from, nh - from);
+        }
+        if (nh > tm.max_hits && lane == 0) s_full = 1;
+        __syncthreads();
+        if (s_full) {
+          fits = false;
+          break;
+        }
+        // this warp's beams: their crossings of all batches, in order
+        int nq = 0;
+        for (int b = 0; b < batches; ++b) {
+          const int2 sg = seg[b];
+          const float4* from = lists + (b % kTeamWarps) * kTeamHits + sg.x;
+          for (int i = 0; i < sg.y; i += 32) {
+            float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (i + lane < sg.y) h = __ldcg(from + i + lane);
+            const bool take = i + lane < sg.y && (__float_as_int(h.w) % kTeamWarps) == wid;
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            if (take) queue[(nq + __popc(m & lt)) & 63] = h;
+            const int was = nq;
+            nq += __popc(m);
+            __syncwarp();
+            if ((nq ^ was) & 32)
+              add_crossings<NBP, true>(a, lane, true, queue[(was & 32) + lane], w.binv, ss, w.off, 0, n,
+                                       0.0f, w.T, w.own, first, [](int, const BandVec<NBP>&) {});
+          }
+        }
+        __syncwarp();
+        if (nq & 31)
+          add_crossings<NBP, true>(a, lane, lane < (nq & 31), queue[(nq & 32) + lane], w.binv, ss,
+                                   w.off, 0, n, 0.0f, w.T, w.own, first, [](int, const BandVec<NBP>&) {});
+        __syncthreads();
+        if (clo + a.cell_cap < listed) {
+          clo += a.cell_cap;
+          continue;
+        }
+        sum_increments<NBP>(tid, a.npix, w.off, w.T, w.own, kTeamWarps * 32);
+        __syncthreads();
+        if (wid == 0) {
+          eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
+          __syncwarp();  // the next pass's records take T's place
+        }
+      }
+      clo = 0;
+      lo += a.M;
+      if (lo >= total) break;
     }
     if (wid == 0) {
-      float Js[NBP], Jc[NBP];
-#pragma unroll
-      for (int b = 0; b < NBP; ++b) Js[b] = Jc[b] = 0.0f;
-      if (n > 0) eval_sources<NBP>(a, lane, w.V, w.T, n, Js, Jc);
-      store_J<NBP>(a, si, lane, Js, Jc, Jrow);
+      if (fits)
+        store_J<NBP>(a, si, lane, Js, Jc, Jrow);
+      else
+        walk_receiver_si<NBP, true>(a, si, Jrow, lane, w);
     }
   }
 }

@@ -129,3 +129,32 @@ def test_gradient_cells_and_beams(t2, oracle_mod, nside, theta, n_src, nb):
                             nside, theta, ps, flags)
     adj._check(adj._gather(gk, gl, ps), want, f"nside={nside} sources={n_src}")
     tree.free()
+
+
+def test_short_rungs_of_many_sources(t2):
+    """Receivers with more sources than a pass holds: a block for each gives the
+    rows of a warp for each (as a plan walks them), in clearly less time.  When
+    such receivers were left to one of the block's warps it took the same time."""
+    case = workloads.random_case(100_000, 200_000, nb=2, seed=12, clumped=True)
+    tree = _tree(t2, case)
+    act = torch.as_tensor(np.random.default_rng(3).choice(100_000, 300, replace=False), device="cuda")
+    plan = t2.Batch([tree], np.array([0, 300], np.int64), np.array([0], np.int32), nside=4, theta=0.5)
+
+    def ms(run):
+        best = np.inf
+        for _ in range(8):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            J = run()
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best, J
+
+    block, J = ms(lambda: tree.J(act, 4, 0.5))
+    warp, ref = ms(lambda: plan.run(act))
+    plan.status()
+    assert torch.equal(J, ref)
+    assert block <= 0.75 * warp, (block, warp)
+    plan.free()
+    tree.free()
