@@ -12,6 +12,8 @@
 // now eight launches and one read-back.  Whole steps, with the pool below and the
 // walk of few receivers by blocks: 33k elements 2.21 -> 0.87 ms, 4k 1.45 -> 0.41,
 // 2.1M and a 1000-receiver rung 5.96 -> 2.78.
+#include <cuda.h>
+
 #include <atomic>
 #include <climits>
 #include <cstdarg>
@@ -413,10 +415,46 @@ __global__ void __launch_bounds__(kSortThreads)
   }
 }
 
-int coop_blocks(int64_t work, int64_t per_block, int per_sm, int* out) {
+// SMs of the stream's green context, 0 where it has none (or the driver does
+// not know them): a stream of one runs on some of the device's SMs, and a
+// cooperative launch sized by the device could not be resident there at once.
+static int green_context_sms(cudaStream_t st) {
+  using GetCtx = CUresult (*)(CUstream, CUcontext*, CUgreenCtx*);
+  using GetResource = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+  struct Entry {
+    GetCtx ctx = nullptr;
+    GetResource resource = nullptr;
+    Entry() {
+      cudaDriverEntryPointQueryResult found;
+      void *c = nullptr, *r = nullptr;
+      if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &c, 12050, cudaEnableDefault, &found) ==
+              cudaSuccess && found == cudaDriverEntryPointSuccess &&
+          cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &r, 12040, cudaEnableDefault,
+                                           &found) == cudaSuccess &&
+          found == cudaDriverEntryPointSuccess) {
+        ctx = reinterpret_cast<GetCtx>(c);
+        resource = reinterpret_cast<GetResource>(r);
+      } else {
+        cudaGetLastError();
+      }
+    }
+  };
+  static const Entry entry;
+  if (!entry.ctx) return 0;
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  if (entry.ctx(st, &ctx, &green) != CUDA_SUCCESS || !green) return 0;
+  CUdevResource r;
+  std::memset(&r, 0, sizeof(r));
+  if (entry.resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return 0;
+  return int(r.sm.smCount);
+}
+
+int coop_blocks(int64_t work, int64_t per_block, int per_sm, cudaStream_t st, int* out) {
   int dev = 0, sms = 0;
   T2_CUDA(cudaGetDevice(&dev));
   T2_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (const int green = green_context_sms(st)) sms = std::min(sms, green);
   const int64_t most = std::min<int64_t>(int64_t(sms) * per_sm, kMaxCoopBlocks);
   *out = int(std::max<int64_t>(1, std::min<int64_t>(most, (work + per_block - 1) / per_block)));
   return TREVR2_OK;
@@ -481,7 +519,7 @@ int radix_sort_u64_i32(uint64_t* keys, int* vals, int64_t n, cudaStream_t st, ui
     ws = own.p;
   }
   int nb = 0;
-  T2_CHECK(coop_blocks(n, kSortPerBlock, 1, &nb));
+  T2_CHECK(coop_blocks(n, kSortPerBlock, 1, st, &nb));
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   char* p = static_cast<char*>(ws);
   uint64_t* k2 = reinterpret_cast<uint64_t*>(p);
@@ -1285,8 +1323,8 @@ static int build_impl(Tree* t, const double* pos, const float* mass, const float
     A.status = t->status;
     A.polls = barrier_polls();
     int blocks = 0, blocks_inner = 0;
-    T2_CHECK(coop_blocks(cap, 2 * kTreeThreads, 1, &blocks));
-    T2_CHECK(coop_blocks(cap, kTreeThreads, 2, &blocks_inner));
+    T2_CHECK(coop_blocks(cap, 2 * kTreeThreads, 1, st, &blocks));
+    T2_CHECK(coop_blocks(cap, kTreeThreads, 2, st, &blocks_inner));
     void* args[] = {&A};
     T2_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_build_tree),
                                         dim3(unsigned(blocks)), dim3(kTreeThreads), args, 0, st));

@@ -245,11 +245,11 @@ uint32_t barrier_polls();
 int debug_cell_cap();
 int debug_team_hits();
 
-// Blocks of a cooperative launch: at most per_sm per SM (the kernel's bound,
-// so that they are resident together), fewer where the work would leave them
-// idle at the barriers.
+// Blocks of a cooperative launch on `st`: at most per_sm (the kernel's bound,
+// so that they are resident together) per SM that the stream's work may use,
+// fewer where the work would leave them idle at the barriers.
 constexpr int kMaxCoopBlocks = 512;
-int coop_blocks(int64_t work, int64_t per_block, int per_sm, int* out);
+int coop_blocks(int64_t work, int64_t per_block, int per_sm, cudaStream_t st, int* out);
 
 // The receivers' slots in their elements' sorted order (keys: their sorted
 // positions, N for an index outside [0, N)).

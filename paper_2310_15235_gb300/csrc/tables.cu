@@ -391,7 +391,7 @@ int ensure_table(Tree* t, int nside, cudaStream_t st, Table** out, bool linear) 
     if (d) widest = std::max(widest, (t->level_begin[d] - t->level_begin[d - 1]) * P);
   }
   int blocks = 0;
-  T2_CHECK(coop_blocks(widest, 2 * kTableThreads, 2, &blocks));
+  T2_CHECK(coop_blocks(widest, 2 * kTableThreads, 2, st, &blocks));
   T2_CUDA(cudaMemsetAsync(A.bar, 0, sizeof(uint32_t), st));
   const void* fn = t->nbp == 1 ? reinterpret_cast<const void*>(&k_tables<1>)
                  : t->nbp == 2 ? reinterpret_cast<const void*>(&k_tables<2>)
