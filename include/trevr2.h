@@ -396,8 +396,10 @@ int trevr2_debug_set(int what, int64_t value);
 
 /* Bytes the library currently holds in its own stream-ordered memory pool of
  * the current device (synchronises the device first; ECUDA if the query
- * fails).  The pool keeps up to 2 GiB of freed memory for later calls and
- * gives it back when an allocation fails. */
+ * fails).  The pool keeps up to 2 GiB of freed memory for later calls; an
+ * allocation that fails gives back what is free by then, and the driver takes it
+ * back itself for any other allocation of the process.  A pool is not used after
+ * a reset of the device's context: the next call makes another. */
 int trevr2_debug_pool_used(uint64_t* bytes);
 
 /* The architecture the library's kernels run as on the current device

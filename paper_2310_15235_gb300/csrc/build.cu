@@ -38,7 +38,14 @@ void set_error(const char* fmt, ...) {
   vsnprintf(g_err, sizeof(g_err), fmt, ap);
   va_end(ap);
 }
-void clear_error() { g_err[0] = 0; }
+
+// The pool of the entry point that runs on this thread, once it has looked it up.
+static thread_local cudaMemPool_t g_call_pool;
+
+void clear_error() {
+  g_err[0] = 0;
+  g_call_pool = nullptr;
+}
 
 static std::atomic<unsigned long long> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -73,9 +80,65 @@ static bool injected_alloc_failure() {
 constexpr uint64_t kPoolKeep = uint64_t(2) << 30;
 constexpr int kMaxDevices = 64;
 
+// The driver's ids of contexts, which no later context gets again.
+struct ContextIds {
+  CUresult (*current)(CUcontext*) = nullptr;
+  CUresult (*id)(CUcontext, unsigned long long*) = nullptr;
+  CUresult (*retain)(CUcontext*, CUdevice) = nullptr;
+  CUresult (*release)(CUdevice) = nullptr;
+  template <class F>
+  static bool find(const char* name, int version, F* fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    *fn = reinterpret_cast<F>(p);
+    return true;
+  }
+  bool known;
+  ContextIds()
+      : known(find("cuCtxGetCurrent", 4000, &current) && find("cuCtxGetId", 12000, &id) &&
+              find("cuDevicePrimaryCtxRetain", 7000, &retain) &&
+              find("cuDevicePrimaryCtxRelease", 11000, &release)) {}
+  // 0 where there is none
+  unsigned long long of_thread() const {
+    CUcontext ctx = nullptr;
+    unsigned long long v = 0;
+    if (!known || current(&ctx) != CUDA_SUCCESS || !ctx || id(ctx, &v) != CUDA_SUCCESS) return 0;
+    return v;
+  }
+  unsigned long long of_primary(int dev) const {
+    CUcontext ctx = nullptr;
+    unsigned long long v = 0;
+    if (!known || retain(&ctx, dev) != CUDA_SUCCESS) return 0;
+    if (id(ctx, &v) != CUDA_SUCCESS) v = 0;
+    release(dev);
+    return v;
+  }
+};
+
+// The pool outlives a reset of the device's (primary) context, with the blocks it
+// keeps (CUDA 13.0: the handle stays good, 1 GiB kept stays reserved), but nothing
+// says that blocks mapped before may be used after: a pool is used in the
+// context it was made in, and replaced after a reset.  Checked by the first
+// allocation of every entry point (each of a build's thirty cost 0.3 us): by the
+// thread's current context where that was seen before, else by the primary
+// context itself.
 static int library_pool(cudaMemPool_t* pool) {
+  if (g_call_pool) {
+    *pool = g_call_pool;
+    return TREVR2_OK;
+  }
+  struct Kept {
+    cudaMemPool_t pool = nullptr;
+    unsigned long long primary = 0, seen = 0;
+  };
   static std::mutex lock;
-  static cudaMemPool_t pools[kMaxDevices] = {};
+  static Kept kept[kMaxDevices];
+  static const ContextIds ids;
   int dev = 0;
   T2_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) {
@@ -83,7 +146,20 @@ static int library_pool(cudaMemPool_t* pool) {
     return TREVR2_OK;
   }
   std::lock_guard<std::mutex> hold(lock);
-  if (!pools[dev]) {
+  Kept& k = kept[dev];
+  unsigned long long now = ids.of_thread();
+  if (!k.pool || !now || now != k.seen) {
+    T2_CUDA(cudaFree(nullptr));  // the runtime's context, current to this thread
+    now = ids.of_thread();
+    const unsigned long long primary = ids.of_primary(dev);
+    if (k.pool && primary != k.primary) {
+      if (cudaMemPoolDestroy(k.pool) != cudaSuccess) cudaGetLastError();
+      k.pool = nullptr;
+    }
+    k.primary = primary;
+    k.seen = now;
+  }
+  if (!k.pool) {
     cudaMemPoolProps props;
     std::memset(&props, 0, sizeof(props));
     props.allocType = cudaMemAllocationTypePinned;
@@ -98,9 +174,9 @@ static int library_pool(cudaMemPool_t* pool) {
       cudaMemPoolDestroy(fresh);
       return cuda_fail(e, "cudaMemPoolSetAttribute");
     }
-    pools[dev] = fresh;
+    k.pool = fresh;
   }
-  *pool = pools[dev];
+  *pool = g_call_pool = k.pool;
   return TREVR2_OK;
 }
 

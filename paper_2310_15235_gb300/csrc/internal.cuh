@@ -188,7 +188,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t blocks, uin
 // ---------------------------------------------------------------------------
 // Host helpers (errors, allocation).
 void set_error(const char* fmt, ...);
-void clear_error();
+void clear_error();  // first in every entry point (it also forgets the last one's pool)
 
 int cuda_fail(cudaError_t e, const char* what);
 
