@@ -1502,10 +1502,12 @@ size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
 //  - p-p absorption (pp) is mostly its particles, read through the L1, of which
 //    the cells' shared memory takes more.  64^3, nside 4: 3 bands 37.5 / 36.8 (80^3
 //    82.5 / 80.9), 1 band 31.9 / 33.8; nside 2: 3 bands 8.5 / 9.3.
+static bool may_use_cells(const Tree* t, const Table* tb) {
+  return tb->nside <= kCellNside && 3 * t->n_luminous >= 12 * tb->nside * tb->nside;
+}
 bool use_cells(const Tree* t, const Table* tb, float theta, bool pp) {
   if (pp && tb->nside == 4 && t->nbp == 4) return false;
-  return tb->nside <= kCellNside && !t->refine_on && theta >= (tb->nside < 4 ? 0.45f : 0.4f) &&
-         3 * t->n_luminous >= 12 * tb->nside * tb->nside;
+  return may_use_cells(t, tb) && !t->refine_on && theta >= (tb->nside < 4 ? 0.45f : 0.4f);
 }
 
 // The beam look-up tables for a walk cell by cell.
@@ -2563,7 +2565,9 @@ extern "C" int trevr2_prepare(trevr2_tree* tree, int nside, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   t->last_stream = st;
   Table* tb = nullptr;
-  return ensure_table(t, nside, st, &tb);
+  T2_CHECK(ensure_table(t, nside, st, &tb));
+  // the look-up of the walks cell by cell, where some theta may ask for it
+  return may_use_cells(t, tb) ? ensure_beam_map(tb, st) : TREVR2_OK;
 }
 
 // ---------------------------------------------------------------------------

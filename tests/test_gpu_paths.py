@@ -158,3 +158,17 @@ def test_short_rungs_of_many_sources(t2):
     assert block <= 0.75 * warp, (block, warp)
     plan.free()
     tree.free()
+
+
+@pytest.mark.parametrize("nside,theta", [(1, 0.5), (2, 0.75), (4, 0.5), (4, 0.3), (8, 0.6)])
+def test_prepare_leaves_nothing_to_the_first_call(t2, nside, theta):
+    """After trevr2_prepare the first J launches what a later one does."""
+    case = workloads.random_case(3000, 300, nb=1, seed=13)
+    tree = _tree(t2, case)
+    tree.prepare(nside)
+    launches = [t2.kernel_launches()]
+    for _ in range(2):
+        tree.J(case["active"], nside, theta)
+        launches.append(t2.kernel_launches())
+    assert launches[1] - launches[0] == launches[2] - launches[1]
+    tree.free()
