@@ -172,3 +172,24 @@ def test_prepare_leaves_nothing_to_the_first_call(t2, nside, theta):
         launches.append(t2.kernel_launches())
     assert launches[1] - launches[0] == launches[2] - launches[1]
     tree.free()
+
+
+@pytest.mark.parametrize("n,bucket", [(20_000, 1), (9000, 2), (1500, 1)])
+def test_topology_outgrows_its_arrays(t2, oracle_mod, n, bucket):
+    """Elements on a line split along one axis of three, so the tree has more nodes
+    than the arrays it is first built into (4 n / bucket + 64): built again into
+    larger ones, from a level all blocks share (20,000; 9,000) or block 0's."""
+    case = workloads.random_case(n - 1, 1, nb=1, seed=n, bucket=bucket)
+    case["pos"][:, 1:] = 0.375
+    e = oracle_mod.OracleTree.from_case(case).export()
+    first = max(1024, 4 * (n // bucket) + 64)
+    assert len(e["depth"]) > first
+    full = np.searchsorted(np.cumsum(np.bincount(e["depth"])), first, side="right")  # its level
+    assert (np.bincount(e["depth"])[full - 1] > 1024) == (n > 1500)
+    tree = _tree(t2, case)
+    np.testing.assert_array_equal(tree.export("perm").cpu().numpy(), e["perm"])
+    for f in ("prefix", "depth", "first", "count", "child", "parent"):
+        got = tree.export(f).cpu().numpy()
+        got = got.view(np.uint64) if f == "prefix" else got
+        np.testing.assert_array_equal(got.astype(e[f].dtype), e[f], err_msg=f)
+    tree.free()
