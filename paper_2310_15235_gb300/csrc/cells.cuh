@@ -371,7 +371,7 @@ __device__ __forceinline__ void cross_batch(const WalkArgs& a, float3 x, int lan
       box1[slot] = make_float4(hy, hz, __int_as_float((sq << 13) | start), __int_as_float(row));
       beams[slot] = near16;
     } else {
-      start = INT32_MIN;  // owns no pair
+      start = -1;  // owns no pair: stays negative below, which is no bit
     }
     __syncwarp();
   }
