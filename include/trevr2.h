@@ -449,7 +449,8 @@ int trevr2_tree_export(const trevr2_tree* tree, int field, void* dst, size_t byt
 
 /* Per-direction absorption of every node for one nside, as float32
  * [n_nodes][6 nside^2][nb] in caller units (leaves repeat their isotropic
- * value); builds and caches the tables if needed. */
+ * value); builds and caches the tables if needed, and waits for tables that no
+ * status read has found good yet (ETIMEOUT when their kernel gave up). */
 int trevr2_alpha_table(trevr2_tree* tree, int nside, float* dst, size_t bytes, void* stream);
 
 /* HEALPix RING pixel centres, float64 [12 nside^2][3] (Gorski et al. 2005). */

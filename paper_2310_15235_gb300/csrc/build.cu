@@ -274,7 +274,7 @@ size_t scan_ws_ints(int64_t n) {
 }
 
 // ws: the last input value, then the block sums of each recursion level.
-static int scan_with_ws(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws) {
+int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws) {
   int* last = ws;
   k_copy_last<<<1, 1, 0, st>>>(d, n, last); note_launch();
   if (n > 0) {
@@ -284,21 +284,13 @@ static int scan_with_ws(int* d, int64_t n, int* d_total, cudaStream_t st, int* w
     } else {
       int* sums = ws + 1;
       k_scan_block<<<unsigned(nblocks), kScanThreads, 0, st>>>(d, n, sums); note_launch();
-      T2_CHECK(scan_with_ws(sums, nblocks, nullptr, st, sums + nblocks));
+      T2_CHECK(scan_exclusive_i32(sums, nblocks, nullptr, st, sums + nblocks));
       k_scan_add<<<unsigned(nblocks), 256, 0, st>>>(d, n, sums); note_launch();
     }
   }
   if (d_total) k_scan_total<<<1, 1, 0, st>>>(d, last, n, d_total); note_launch();
   T2_CUDA(cudaGetLastError());
   return TREVR2_OK;
-}
-
-int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws) {
-  if (ws) return scan_with_ws(d, n, d_total, st, ws);
-  T2_CHECK(dalloc(&ws, scan_ws_ints(n), st));
-  const int rc = scan_with_ws(d, n, d_total, st, ws);
-  dfree(ws, st);
-  return rc;
 }
 
 // ---------------------------------------------------------------------------

@@ -19,7 +19,8 @@ constexpr int kMaxDepth = 63;
 constexpr int kKeyBits = 21;
 
 // ---------------------------------------------------------------------------
-// Node record read by the walk: 32 bytes = two 16-byte loads.
+// Node record read by the walk: one 32-byte load from the tree's arrays, which
+// start on 256 bytes (load_node); copies in shared memory are 16-byte aligned.
 struct __align__(16) NodeW {
   float lo[3];    // normalised lower corner (exact)
   float B;        // largest distance from the centre of luminosity to a corner
@@ -28,6 +29,7 @@ struct __align__(16) NodeW {
   int count;      // elements under the node
   uint32_t meta;  // depth | flags
 };
+static_assert(sizeof(NodeW) == 32, "load_node reads a record at once, 32-byte aligned");
 constexpr uint32_t kMetaDepthMask = 63u;
 constexpr uint32_t kMetaLeaf = 1u << 8;
 constexpr uint32_t kMetaHasL = 1u << 9;      // some luminosity below
@@ -257,9 +259,9 @@ int order_receivers(const Tree* t, const int64_t* active, int64_t A, uint64_t* k
                     cudaStream_t st);
 
 // Exclusive scan of n int32 values in place; *d_total (device) gets the sum.
-// ws (device, scan_ws_ints(n) ints) or NULL to allocate one stream ordered.
+// ws: device, scan_ws_ints(n) ints.
 size_t scan_ws_ints(int64_t n);
-int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws = nullptr);
+int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws);
 
 // Stable LSD radix sort of keys below 2^key_bits with int32 payload (in place).
 // ws (device, radix_ws_bytes(n) bytes) or NULL to allocate one stream ordered.

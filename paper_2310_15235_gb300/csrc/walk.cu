@@ -246,9 +246,9 @@ __device__ __forceinline__ void absorb(const WalkArgs& a, float3 x, int si, int 
 }
 
 // The sources of one origin in passes of M, each pass's absorbing cells in
-// windows of cell_cap (one pass and one window unless a cut holds more):
-// stages a pass's sources, sums their tau over the windows, and hands the
-// pass to eval(n).
+// windows of cell_cap (one pass and one window unless a cut holds more; within
+// a window absorb_cells goes over the cells once per bin_cap sources): stages a
+// pass's sources, sums their tau over the windows, and hands the pass to eval(n).
 template <int NBP, bool kBucket, bool kPP, bool kCSM, bool kCells, class Eval>
 __device__ __forceinline__ void walk_origin(const WalkArgs& a, float3 x, int si, int lane,
                                             const WarpMem& w, int leaf, float rpp, Eval eval) {
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32, 2)
     }
     __syncthreads();
     if (s_slot >= (unsigned long long)a.A) break;
-    const int64_t r = a.order ? int64_t(a.order[s_slot]) : int64_t(s_slot);
+    const int64_t r = int64_t(s_slot);  // as given: too few for their order to matter
     const int64_t io = a.active[r];
     float* Jrow = a.J + r * a.nbsel;
     if (io < 0 || io >= a.N) {
@@ -1497,11 +1497,15 @@ size_t walk_layout(WalkArgs* a, int warps, bool cells, bool pp) {
 //    96.7 / 95.6, 68.5 / 77.7; nside 4: 0.35 220 / 198, 0.42 145 / 160, 0.5 104 / 134;
 //  - sources: beams without any are not walked.  48^3, theta 0.5, nside 4: 30
 //    sources 2.90 / 2.41, 60 3.24 / 3.26, 120 3.63 / 4.16; nside 2: 3 sources
-//    1.88 / 1.79, 12 2.00 / 2.08; nside 1: 1 source 1.63 / 1.43, 3 1.66 / 1.75;
-//  - refinement opens cells that no beam with sources comes near: beam by beam;
+//    1.88 / 1.79, 12 2.00 / 2.08; nside 1: 1 source 1.63 / 1.43, 3 1.66 / 1.75.
+//    No upper end: 96^3, 200,000 sources: nside 4, theta 0.5 137 / 169, 0.4 244 /
+//    270; nside 2, theta 0.75 39.8 / 51.0, 0.45 136 / 140; nside 1 94 / 114;
+//  - refinement opens cells that no beam with sources comes near: 200k clumped
+//    elements, nside 2 324 / 29.7; 64^3, nside 4 1812 / 100, nside 2 585 / 74;
 //  - p-p absorption (pp) is mostly its particles, read through the L1, of which
 //    the cells' shared memory takes more.  64^3, nside 4: 3 bands 37.5 / 36.8 (80^3
-//    82.5 / 80.9), 1 band 31.9 / 33.8; nside 2: 3 bands 8.5 / 9.3.
+//    82.5 / 80.9), 2 bands 32.2 / 33.2 (80^3 73.3 / 75.4), 1 band 31.9 / 33.8; nside
+//    2: 3 bands 8.5 / 9.3.
 static bool may_use_cells(const Tree* t, const Table* tb) {
   return tb->nside <= kCellNside && 3 * t->n_luminous >= 12 * tb->nside * tb->nside;
 }
@@ -1590,7 +1594,10 @@ static int grow_buffer(void** buf, size_t* bytes, size_t need, cudaStream_t st, 
 // Receivers up to which a block walks each one: measured on the 96^3 clumpy
 // field against a warp each (ms a call): nside 4, theta 0.5: 100 receivers
 // 0.20 / 0.49, 600 0.32 / 0.53, 1000 0.48 / 0.57, 1500 0.67 / 0.58; nside 2,
-// theta 0.75: 100 0.12 / 0.18, 600 0.17 / 0.19, 1000 0.24 / 0.21.
+// theta 0.75: 100 0.12 / 0.18, 600 0.17 / 0.19, 1000 0.24 / 0.21.  With 200,000
+// sources (passes): nside 4, theta 0.5: 100 0.36 / 0.85, 640 0.69 / 1.01, 1000 0.94 /
+// 1.06; nside 2, theta 0.45: 640 0.74 / 1.11.  Few or clumped sources meet earlier:
+// 100k clumped elements, 200k sources, nside 4: 640 0.68 / 0.63, 1000 0.92 / 0.64.
 static int64_t team_receivers(int nside) { return nside < 4 ? 640 : 1024; }
 
 // The walk of few receivers, cell by cell; a holds everything but the buffers.
@@ -2149,8 +2156,9 @@ static int batch_select(Batch* b, int warps, int M, int64_t limit, cudaStream_t 
 }
 
 // Enqueues the run in the selected shape (keys, sort, distinct keys, walk,
-// scatter) with no allocation, synchronisation or attribute call, so that it
-// can be recorded into a CUDA graph.
+// scatter) with no allocation or synchronisation, so that it can be recorded
+// into a CUDA graph (the sort of up to 8192 rows sets its kernel's
+// shared-memory attribute, which a capture allows).
 static int batch_enqueue(Batch* b, const int64_t* active, float* J, cudaStream_t st) {
   b->args.active = active;
   b->args.J = J;

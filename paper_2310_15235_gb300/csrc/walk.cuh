@@ -18,8 +18,9 @@ constexpr int kWalkWarps = 4;                 // warps per block
 // than 8 at 64 registers, which spills.
 constexpr int kWalkWarpsPerSM = 28;
 // Resident warps per SM of the kernels that sum the absorption cell by cell: 28
-// (72 registers a thread) where the walks are short, 24 (80, no spills) where a
-// receiver has several hundred sources and per bucket.  ms at 28 / 24: nside 2,
+// (72 registers a thread) where the walks are short, 24 (80: 3 bands no spills, per
+// bucket 44 bytes) where a receiver has several hundred sources and per bucket.
+// ms at 28 / 24: nside 2,
 // 64^3 5.62 / 5.94, 96^3 32.3 / 34.3; nside 4, 96^3 69.9 / 66.3, 64^3 10.2 /
 // 10.5; per bucket 96^3 nside 4 14.5 / 13.3, nside 2 6.4 / 6.2; 20: all slower.
 constexpr int kCellWarpsPerSM = 28;
