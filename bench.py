@@ -39,6 +39,8 @@ NODE_BYTES = 32  # walk record of one node
 # while the sources still hash the same.
 WALK_PROFILE = os.path.join(ROOT, "profiles", "k_walk_clumpy96.md")
 WALK_SOURCES = ["walk.cu", "walk.cuh", "healpix.cuh", "internal.cuh"]
+# the walk cell by cell, which they include; its hash stands beside theirs
+WALK_CELLS = os.path.join(ROOT, "paper_2310_15235_gb300", "csrc", "cells.cuh")
 
 
 def kernel_sources_sha256():
@@ -97,6 +99,22 @@ def _walk_counters(hbm_peak):
             "issue_active_pct": rec["issue_active_pct"],
             "note": "ncu counters of one cold, serialised launch; the walk is bound by "
                     "instruction issue, not by DRAM"}
+
+
+def cells_source_sha256():
+    import hashlib
+    with open(WALK_CELLS, "rb") as f:
+        return hashlib.sha256(f.read()).hexdigest()
+
+
+def _walk_profile(receivers, hbm_peak):
+    """What the walk profile says of a launch over `receivers`: (DRAM bytes, note,
+    counters), without bytes and counters when it was captured on other sources."""
+    rec, why = _walk_profile_record()
+    if rec is not None and rec.get("cells_sha256") != cells_source_sha256():
+        why = "the walk profile was captured on another cells.cuh; capture it again"
+        return None, why, None
+    return (*_walk_traffic(receivers), _walk_counters(hbm_peak))
 
 
 def _workload_name(case):
@@ -355,10 +373,10 @@ def run_ours(args, world, rank, local):
         ot, sample, st, t_j, t_build, cores = _oracle_sample(case, args.cpu_seconds)
         per_rec, means = _algorithmic_bytes_per_receiver(st, nb)
         achieved = per_rec * A / (walk_avg * 1e-3) / 1e9
-        traffic, traffic_note = _walk_traffic(A)
+        traffic, traffic_note, ncu = _walk_profile(A, hbm_peak)
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "traffic": traffic,
-                    "traffic_note": traffic_note, "ncu": _walk_counters(hbm_peak),
+                    "traffic_note": traffic_note, "ncu": ncu,
                     "kernel": "k_walk", "peak_kind": peak_kind,
                     "algorithmic_bytes_per_unit": per_rec / (npix * nb),
                     "per_receiver_counts": means}

@@ -297,8 +297,9 @@ int scan_exclusive_i32(int* d, int64_t n, int* d_total, cudaStream_t st, int* ws
 // Stable sort of 64-bit keys with a 32-bit payload.
 //
 // Up to kSmallSort keys: one block, a merge sort in shared memory, every key
-// finding its place in the neighbouring run by a binary search (4097 keys: 14
-// us; a bitonic network's 91 steps took 75).  More: one cooperative
+// finding its place in the neighbouring run by a binary search (4097 keys: 56
+// us by itself and cold; a bitonic network's 91 steps took 1.7 times as long),
+// bound by shared-memory loads.  More: one cooperative
 // launch does every pass of an LSD radix sort (8 bits a pass), with a grid
 // barrier where a pass needs all blocks' counts or keys: a launch for each
 // step of each pass left the GPU idle between them for longer than the steps

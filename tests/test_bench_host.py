@@ -57,3 +57,20 @@ def test_traffic_only_for_the_captured_sources(monkeypatch):
     traffic, note = bench._walk_traffic(rec["receivers"])
     assert traffic is None and "capture it again" in note
     assert bench._walk_counters(6672.2) is None
+
+
+def test_traffic_only_for_the_captured_cells(monkeypatch, tmp_path):
+    """The walk's kernel also includes cells.cuh: a profile captured on another
+    one says nothing."""
+    rec = _profile_record()
+    monkeypatch.setattr(bench, "kernel_sources_sha256", lambda: rec["sources_sha256"])
+    monkeypatch.setattr(bench, "cells_source_sha256", lambda: rec["cells_sha256"])
+    traffic, note, ncu = bench._walk_profile(rec["receivers"], 6798.2)
+    assert traffic == rec["dram_read_bytes"] + rec["dram_write_bytes"] and ncu is not None
+    monkeypatch.undo()
+    monkeypatch.setattr(bench, "kernel_sources_sha256", lambda: rec["sources_sha256"])
+    other = tmp_path / "cells.cuh"
+    other.write_bytes(open(bench.WALK_CELLS, "rb").read() + b"\n")
+    monkeypatch.setattr(bench, "WALK_CELLS", str(other))
+    traffic, note, ncu = bench._walk_profile(rec["receivers"], 6798.2)
+    assert traffic is None and ncu is None and "capture it again" in note
