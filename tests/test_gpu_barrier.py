@@ -182,3 +182,60 @@ def test_refusal_costs_no_build(t2):
     e1.record()
     torch.cuda.synchronize()
     assert e0.elapsed_time(e1) < 100.0
+
+
+def test_waits_hold_beside_other_work(t2):
+    """Cooperative launches beside a walk that fills the GPU, from several threads
+    and streams, and in a captured call: none of them waits for blocks that are
+    not resident (2^20 polls are a fraction of a second)."""
+    import threading
+    big = workloads.random_case(30_000, 3000, nb=2, seed=406, clumped=True)
+    small = workloads.random_case(20_000, 300, nb=2, seed=407, clumped=True)
+    f = [torch.as_tensor(small[k], device="cuda").to(d) for k, d in
+         (("pos", torch.float64), ("mass", torch.float32), ("kappa", torch.float32),
+          ("lum", torch.float32), ("h", torch.float32))]
+    rows = torch.as_tensor(np.random.default_rng(5).integers(0, 20_000, size=30_000), device="cuda")
+    walked = _tree(t2, big)
+    every = torch.arange(30_000, device="cuda")
+    walked.J(every, 8, 0.3)
+    ref = t2.build(*f, small["box_lo"], small["box_size"], small["bucket"]).J(rows, 2, 0.75)
+    t2.debug_set(t2.DEBUG_BARRIER_POLLS, 1 << 20)
+    torch.cuda.synchronize()
+    errors = []
+
+    def steps():
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(4):
+                    tree = t2.build(*f, small["box_lo"], small["box_size"], small["bucket"], stream=stream)
+                    J = tree.J(rows, 2, 0.75, stream=stream)
+                    assert torch.equal(J, ref)
+                    tree.free()
+        except Exception as e:
+            errors.append(e)
+
+    long = torch.cuda.Stream()
+    for _ in range(4):
+        walked.J(every, 8, 0.3, flags=t2.ASYNC, stream=long)
+    threads = [threading.Thread(target=steps) for _ in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    walked.status()
+    tree = t2.build(*f, small["box_lo"], small["box_size"], small["bucket"])
+    out = torch.empty_like(ref)
+    tree.J(rows, 2, 0.75, out=out)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        tree.J(rows, 2, 0.75, flags=t2.ASYNC, out=out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    tree.status()
+    assert torch.equal(out, ref)
+    tree.free()
+    walked.free()
